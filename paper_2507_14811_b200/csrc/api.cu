@@ -150,7 +150,7 @@ sq_status segquant_calib_scales(const void *X, sq_dtype dt, int64_t rows, int64_
     if ((st = check_ws(workspace, ws_bytes)) != SQ_OK) return st;
     uint32_t *partials = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(workspace) + kWsStatusBytes);
     return launch_calib(X, dt, rows, K, ld, hs.b, is_weight, dual, code_qmax(code), code_qmin_abs(code, flags),
-                        s_pos, s_neg, partials, static_cast<cudaStream_t>(stream));
+                        s_pos, s_neg, partials, static_cast<uint32_t *>(workspace) + 1, static_cast<cudaStream_t>(stream));
 }
 
 sq_status segquant_calib_scales_static(const void *X, sq_dtype dt, int64_t rows, int64_t K, int64_t ld,
@@ -217,7 +217,8 @@ sq_status segquant_calib_zero_point(const void *X, sq_dtype dt, int64_t rows, in
     if (hs.status != SQ_OK) return hs.status;
     if ((st = check_ws(workspace, ws_bytes)) != SQ_OK) return st;
     uint32_t *partials = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(workspace) + kWsStatusBytes);
-    return launch_calib_zero_point(X, dt, rows, K, ld, hs.b, s_x, z_x, partials, static_cast<cudaStream_t>(stream));
+    return launch_calib_zero_point(X, dt, rows, K, ld, hs.b, s_x, z_x, partials, static_cast<uint32_t *>(workspace) + 1,
+                                   static_cast<cudaStream_t>(stream));
 }
 
 sq_status segquant_quantize_act_zero_point(const void *X, sq_dtype dt, int64_t M, int64_t K, int64_t ld,

@@ -8,7 +8,7 @@
 namespace sq {
 
 // Workspace layout (device, 256-byte aligned):
-//   [0,256)        status words: word 0 = first expired wait (0 = none)
+//   [0,256)        status words: word 0 = first expired wait (0 = none); word 1 = arrival count of a calibration launch
 //   [256, 256+32Ki) calibration partials: 2 ordered-uint words per (p,q) block
 constexpr size_t kWsStatusBytes = 256;
 constexpr int kMaxBlocks = SQ_MAX_P * SQ_MAX_Q;               // 4096 (p,q) blocks
@@ -46,7 +46,7 @@ inline float code_qmin_abs(sq_code c, uint32_t flags)
 // kernels' host launchers (defined in the .cu files)
 sq_status launch_calib(const void *X, sq_dtype dt, int64_t rows, int64_t K, int64_t ld, const SegBounds &sb,
                        int is_weight, int dual, float q_max, float q_min_abs, float *s_pos, float *s_neg,
-                       uint32_t *partials, cudaStream_t st);
+                       uint32_t *partials, uint32_t *done_count, cudaStream_t st);
 
 sq_status launch_calib_static(const void *X, sq_dtype dt, int64_t rows, int64_t K, int64_t ld, const SegBounds &sb,
                               int is_weight, int dual, float q_max, float q_min_abs, float *s_pos, float *s_neg,
@@ -102,7 +102,7 @@ sq_status launch_pack_w4(const void *Wq8, int64_t ld8, int64_t N, int64_t K, voi
                          cudaStream_t st);
 
 sq_status launch_calib_zero_point(const void *X, sq_dtype dt, int64_t rows, int64_t K, int64_t ld, const SegBounds &sb,
-                                  float *s_x, int32_t *z_x, uint32_t *partials, cudaStream_t st);
+                                  float *s_x, int32_t *z_x, uint32_t *partials, uint32_t *done_count, cudaStream_t st);
 
 sq_status launch_fold_zero_point(const void *Wq, int64_t ldw, int64_t N, int64_t K, const SegBounds &sb,
                                  const float *s_x, const int32_t *z_x, const float *s_w, const float *bias,

@@ -17,6 +17,40 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
+# ------------------------------------------------------------------ calibration: grid and piece edges
+
+@pytest.mark.parametrize("x_dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("case", [
+    # rows, K, kb, nb: single rows, fewer rows than a block's warps, a last piece that is not whole, K-bounds inside a
+    # 16-byte piece, rows that leave their N-segment inside a warp's batch of loads, one-row segments, several blocks
+    (1, 16, [0, 16], [0, 1]),
+    (7, 40, [0, 13, 40], [0, 3, 7]),
+    (65, 333, [0, 5, 100, 333], [0, 1, 2, 3, 65]),
+    (1000, 1544, [0, 512, 1544], [0, 100, 1000]),
+    (2500, 96, [0, 1, 2, 96], [0, 2499, 2500]),
+    (130, 4100, list(range(0, 4101, 100)), [0, 64, 130]),
+])
+def test_calibration_scales_are_exact(case, x_dtype):
+    """Extrema and one IEEE division per scale: bit-exact against the oracle, twice on one workspace whose contents are
+    not zero, with the values beyond K (row pitch) larger than any inside."""
+    rows, K, kb, nb = case
+    rs = np.random.default_rng(11)
+    X = torch.from_numpy((rs.standard_normal((rows, K)) * np.exp(rs.standard_normal((rows, 1)))).astype(np.float32)).to(x_dtype)
+    Xd = torch.full((rows, (K + 15) // 16 * 16 + 16), 1e6, dtype=x_dtype, device=DEV)
+    Xd[:, :K] = X.to(DEV)
+    Xn, seg, ws = X.float().numpy(), B.SegTable(kb, nb), B.new_workspace(DEV)
+    ws[4:] = 0x5A
+    for dual in (True, False):
+        r_pos, r_neg = O.calib_act(Xn, kb, dual)
+        g_pos, g_neg = B.segquant_calib_scales(Xd[:, :K], seg, "int8", False, dual, ws)
+        assert np.array_equal(g_pos.cpu().numpy(), r_pos) and (not dual or np.array_equal(g_neg.cpu().numpy(), r_neg))
+    g_w, _ = B.segquant_calib_scales(Xd[:, :K], seg, "int8", True, False, ws)
+    assert np.array_equal(g_w.cpu().numpy().reshape(len(kb) - 1, -1), O.calib_weight(Xn, kb, nb))
+    g_s, g_z = B.segquant_calib_zero_point(Xd[:, :K], seg, ws)
+    r_s, r_z = O.calib_act_asym(Xn, kb)
+    assert np.array_equal(g_s.cpu().numpy(), r_s) and np.array_equal(g_z.cpu().numpy(), r_z)
+
+
 # ------------------------------------------------------------------ zero-point scheme (App. A)
 
 def run_zero_point_parity(spec):
