@@ -149,7 +149,7 @@ sq_status segquant_quantize_act(const void *X, sq_dtype dt, int64_t M, int64_t K
  *   have stored it in), then x = a * mult[k] as one fp32 multiply (mult dev [K] fp32, or NULL), then the codes
  *   of segquant_quantize_act for x.  The activation never goes through device memory.
  *   Accuracy of the activation: evaluated in fp32 with relative error <= (|h| + 8) 2^-23 (SiLU) and
- *   (3 h^2 + 48) 2^-24 (GELU); where the exact value lies that close to a rounding boundary of dt the stored
+ *   (3 h^2 + 48) 2^-24 (GELU; a result below 2^-100 in magnitude may be zero); where the exact value lies that close to a rounding boundary of dt the stored
  *   value, and with it the code, may be that of the neighbouring dt value.  With SQ_ACT_NONE the codes are exact.
  *   SQ_ACT_GEGLU (gated GELU; App. B names it without a form): H is [M, 2K] with ld >= 2K, value half in columns
  *   [0, K), gate half in [K, 2K), a[k] = H[k] * GELU(H[K + k]) with relative error <= (3 g^2 + 49) 2^-24, g the
@@ -332,7 +332,7 @@ sq_status segquant_set_tuning(int tile_n, int stages, int cta_group, int segment
 /* The fused activation of segquant_quantize_act_fused has two implementations with identical results: one that
  * evaluates SiLU / GELU per element, and, for bf16 inputs, one that looks the stored activation up in a table of
  * all 65536 bf16 values which every thread block builds in shared memory first (about 9 us per launch, then one
- * load per element).  fused_table_mode: 0 automatic (the table from 8 Mi elements up for GELU, 16 Mi for SiLU), 1 the table wherever it
+ * load per element).  fused_table_mode: 0 automatic (the table from 10 Mi elements up for GELU, 18 Mi for SiLU), 1 the table wherever it
  * applies, 2 never.  Process-wide and for tests and sweeps, like segquant_set_tuning. */
 sq_status segquant_set_quantize_tuning(int fused_table_mode);
 

@@ -7,6 +7,7 @@
 // even, clip"; the common case computes them with a handful of full-rate fp32 instructions per element (see
 // SegConst) so that the pass stays memory bound.
 #include <cuda_bf16.h>
+#include <algorithm>
 #include <atomic>
 #include "sq_common.cuh"
 
@@ -98,6 +99,39 @@ __device__ __forceinline__ void quant1(float x, float sp, float sn, int zp, int 
     }
 }
 
+// packed fp32 pairs: sm_100 executes mul / fma / add on two fp32 values per instruction
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void unpack2u(uint64_t v, uint32_t &lo, uint32_t &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 // The act-to-linear segment in front of the quantizer (Sec. 4.3.2; App. B: SiLU and GELU feed DualScale layers),
 // evaluated in fp32 and rounded once to the dtype the unfused graph would have stored the activation in.
 // SiLU(h) = h sigma(h) with z = exp(-|h|): sigma = 1 / (1 + z) for h >= 0, z / (1 + z) below (no overflow).  The
@@ -115,53 +149,98 @@ __device__ __forceinline__ void quant1(float x, float sp, float sn, int zp, int 
 // What remains is the hardware exponential's own error (|s| 2^-24 from the product with log2 e, one unit in the
 // last place from the approximation), the fast division's 2 units and a dozen roundings: relative error
 // <= (3 h^2 + 48) 2^-24; in |h| <= 4 it stays below 2^-20.
-__device__ __forceinline__ float silu_f32(float h)
+// Both are written for TWO elements: the multiplies, FMAs and adds go two per instruction (packed fp32 pairs), each of
+// them rounding exactly as the scalar instruction does, which is what bounds the fused pass (the ALUs, not memory).
+// (8192 x 2560 gated GELU, dual int8, 126 MB: 49.4 us one element at a time with the gate half one row ahead in registers,
+// 35.0 us with pairs and the gate half in the ring; without the table, 54 M elements of GELU 93 -> 72 us.)
+// GELU without branches: with a = min(|h|, 20), v = max(h, 0) - (a / 2) E in one FMA is h - (h / 2) E for h >= 0 and
+// (h / 2) E below; at a = 20 the exponential has long underflowed to zero, so v is h or 0 beyond it and t^2 stays
+// finite for every h.
+__device__ __forceinline__ float rcp_approx(float x)
 {
-    const float z = __expf(-fabsf(h));
-    const float num = h >= 0.0f ? h : __fmul_rn(h, z);
-    return __fdividef(num, __fadd_rn(1.0f, z));
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
-__device__ __forceinline__ float gelu_f32(float h)
+__device__ __forceinline__ float ex2_approx_ftz(float x)
 {
-    const float t = __fmul_rn(fabsf(h), 0.70710678118654752440f);
-    const float z = __fdividef(t - 2.5f, t + 2.5f);
-    float g = -5.388610225e-05f;
-    g = fmaf(g, z, 2.161547454e-04f);
-    g = fmaf(g, z, 8.157527773e-04f);
-    g = fmaf(g, z, -2.643950749e-03f);
-    g = fmaf(g, z, -3.974915482e-03f);
-    g = fmaf(g, z, 3.992317244e-02f);
-    g = fmaf(g, z, -1.250353903e-01f);
-    g = fmaf(g, z, 2.517131865e-01f);
-    g = fmaf(g, z, -3.717366457e-01f);
-    g = fmaf(g, z, 2.108063698e-01f);
-    const float s = __fmul_rn(t, t);
-    const float e = fmaf(t, t, -s);                       // t^2 = s + e exactly
-    float E = __fmul_rn(__expf(-s), g);
-    E = fmaf(-E, e, E);                                   // exp(-(s + e)) = exp(-s) (1 - e) to first order
-    const float half = __fmul_rn(0.5f, h);
-    const float v = h >= 0.0f ? fmaf(-half, E, h) : __fmul_rn(half, E);
-    // beyond t = 13.5 the exponential has long underflowed: h or -0, also where t^2 overflows or h is infinite
-    return t >= 13.5f ? (h >= 0.0f ? h : -0.0f) : v;
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ uint64_t dup2(float v) { return pack2(v, v); }
+__device__ __forceinline__ uint64_t silu2(float h0, float h1)
+{
+    const float z0 = __expf(-fabsf(h0)), z1 = __expf(-fabsf(h1));
+    float d0, d1, n0, n1;
+    unpack2(add2(pack2(z0, z1), dup2(1.0f)), d0, d1);
+    unpack2(mul2(pack2(h0, h1), pack2(z0, z1)), n0, n1);
+    return mul2(pack2(h0 >= 0.0f ? h0 : n0, h1 >= 0.0f ? h1 : n1), pack2(rcp_approx(d0), rcp_approx(d1)));
+}
+__device__ __forceinline__ uint64_t gelu2(float h0, float h1)
+{
+    const uint64_t a = pack2(fminf(fabsf(h0), 20.0f), fminf(fabsf(h1), 20.0f));
+    const uint64_t t = mul2(a, dup2(0.70710678118654752440f));
+    float d0, d1;
+    unpack2(add2(t, dup2(2.5f)), d0, d1);
+    const uint64_t z = mul2(add2(t, dup2(-2.5f)), pack2(rcp_approx(d0), rcp_approx(d1)));
+    uint64_t g = fma2(dup2(-5.388610225e-05f), z, dup2(2.161547454e-04f));
+    g = fma2(g, z, dup2(8.157527773e-04f));
+    g = fma2(g, z, dup2(-2.643950749e-03f));
+    g = fma2(g, z, dup2(-3.974915482e-03f));
+    g = fma2(g, z, dup2(3.992317244e-02f));
+    g = fma2(g, z, dup2(-1.250353903e-01f));
+    g = fma2(g, z, dup2(2.517131865e-01f));
+    g = fma2(g, z, dup2(-3.717366457e-01f));
+    g = fma2(g, z, dup2(2.108063698e-01f));
+    const uint64_t s = mul2(t, t);
+    const uint64_t neg_e = fma2(mul2(t, dup2(-1.0f)), t, s);      // t^2 = s - neg_e exactly
+    float x0, x1;
+    unpack2(mul2(s, dup2(-1.4426950408889634f)), x0, x1);
+    uint64_t E = mul2(pack2(ex2_approx_ftz(x0), ex2_approx_ftz(x1)), g);
+    E = fma2(E, neg_e, E);                                        // exp(-(s + e)) = exp(-s) (1 - e) to first order
+    return fma2(mul2(a, dup2(-0.5f)), E, pack2(fmaxf(h0, 0.0f), fmaxf(h1, 0.0f)));
+}
+// two activations as the unfused graph would have stored them, times the per-channel multipliers (one fp32 multiply)
+template <typename Tin>
+__device__ __forceinline__ uint64_t stored2(uint64_t a, uint64_t mult)
+{
+    if (sizeof(Tin) == 2) {
+        float a0, a1;
+        unpack2(a, a0, a1);
+        const __nv_bfloat162 r = __floats2bfloat162_rn(a0, a1);
+        const uint32_t w = *reinterpret_cast<const uint32_t *>(&r);
+        a = pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+    }
+    return mul2(a, mult);
 }
 template <typename Tin>
-__device__ __forceinline__ float pre1(float h, int act, float mult)
+__device__ __forceinline__ uint64_t pre2(float h0, float h1, int act, uint64_t mult)
 {
-    float a = h;
-    if (act) {
-        a = act == 1 ? silu_f32(h) : gelu_f32(h);
-        if (sizeof(Tin) == 2) a = __bfloat162float(__float2bfloat16_rn(a));      // stored as bf16 in the unfused graph
-    }
-    return __fmul_rn(a, mult);                                // the per-channel multiplier: one fp32 multiply
+    if (!act) return mul2(pack2(h0, h1), mult);
+    return stored2<Tin>(act == 1 ? silu2(h0, h1) : gelu2(h0, h1), mult);
 }
 // Gated GELU (App. B lists GEGLU with SiLU and GELU): value * GELU(gate), the product in fp32 (one more rounding
 // on top of the GELU's error: relative error <= (3 g^2 + 49) 2^-24), rounded once to the stored dtype.
 template <typename Tin>
+__device__ __forceinline__ uint64_t pre_gated2(float v0, float v1, float g0, float g1, uint64_t mult)
+{
+    return stored2<Tin>(mul2(pack2(v0, v1), gelu2(g0, g1)), mult);
+}
+// single elements (row tails, segment bounds inside a chunk, extreme scales)
+template <typename Tin>
+__device__ __forceinline__ float pre1(float h, int act, float mult)
+{
+    float lo, hi;
+    unpack2(pre2<Tin>(h, h, act, dup2(mult)), lo, hi);
+    return lo;
+}
+template <typename Tin>
 __device__ __forceinline__ float pre_gated(float value, float gate, float mult)
 {
-    float a = __fmul_rn(value, gelu_f32(gate));
-    if (sizeof(Tin) == 2) a = __bfloat162float(__float2bfloat16_rn(a));
-    return __fmul_rn(a, mult);
+    float lo, hi;
+    unpack2(pre_gated2<Tin>(value, value, gate, gate, dup2(mult)), lo, hi);
+    return lo;
 }
 
 // Per-segment constants of the fast form.  The quotient x / s is obtained from the correctly rounded
@@ -198,39 +277,6 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c)
     return d;
 }
 
-// packed fp32 pairs: sm_100 executes mul / fma / add on two fp32 values per instruction
-__device__ __forceinline__ uint64_t pack2(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ void unpack2u(uint64_t v, uint32_t &lo, uint32_t &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
 // two quotients x / s from r = RN(1/s): q0 = RN(x r), e = x - q0 s, q = RN(q0 + e r)
 __device__ __forceinline__ uint64_t div2_rn_fast(uint64_t x2, uint64_t neg_s2, uint64_t r2)
 {
@@ -350,8 +396,8 @@ __device__ __forceinline__ void quant4(const float (&x)[4], const SegConst &cp, 
 // flight while the current row is converted.
 // PRE != 0 compiles in the act-to-linear prologue: activation function and per-channel multiplier in front of the
 // quantizer, so that the activation's output never goes through HBM.  PRE == 2 is the gated form: the row holds
-// 2 K pre-activations, the value half travels through the ring like any input and the gate half (K elements
-// further on) is fetched into registers one row ahead.
+// 2 K pre-activations, value half and gate half (K elements further on); both travel through the ring (fp32: the gate
+// half is fetched into registers one row ahead, its ring would not fit).
 // RING: depth of the shared-memory ring the rows travel through (see below); 4 when a thread has many rows to
 // walk (large inputs: more bytes in flight), 2 otherwise (less shared memory, more L1 for the copies).
 template <typename Tin, int CODE, int MODE, int PRE, int RING>
@@ -384,36 +430,48 @@ quantize_kernel(const __grid_constant__ QuantParams prm)
     uint8_t *dn = DUAL ? prm.c_neg + int64_t(r0) * prm.ldc + k0 : nullptr;
     const int64_t src_step = int64_t(R) * prm.ld, dst_step = int64_t(R) * prm.ldc;
 
-    float mreg[PRE ? kVec : 1];                              // this chunk's multipliers, loaded once
+    uint64_t mreg[PRE ? kVec / 2 : 1];                       // this chunk's multipliers, loaded once
     if (PRE) {
 #pragma unroll
-        for (int i = 0; i < kVec; i++) mreg[i] = (prm.mult && k0 + i < K) ? __ldg(prm.mult + k0 + i) : 1.0f;
+        for (int i = 0; i < kVec; i += 2)
+            mreg[i / 2] = pack2((prm.mult && k0 + i < K) ? __ldg(prm.mult + k0 + i) : 1.0f,
+                                (prm.mult && k0 + i + 1 < K) ? __ldg(prm.mult + k0 + i + 1) : 1.0f);
     }
 
     // The rows of this chunk travel through a thread-private ring in shared memory: asynchronous 16-byte copies
     // (global -> shared without passing through registers) of the next kDepth - 1 rows are in flight while the
     // current row is converted, so the bytes in flight per SM do not cost registers.  Every thread reads only what
     // it copied itself, so a wait on its own copy groups is all the synchronisation there is.
+    // (gated, bf16) the chunk of the gate half travels in the same slots, behind the value half's pieces.
     constexpr int NV = int(sizeof(Tin)) * kVec / 16;                        // 16-byte pieces per row chunk
-    constexpr int kDepth = (sizeof(Tin) == 2 || RING == 2) ? RING : RING / 2;  // ring slots (32 KiB per block at most)
-    __shared__ uint4 ring[kDepth * NV * kThreads];
+    constexpr bool kGateRing = GATED && sizeof(Tin) == 2;
+    constexpr int NS = kGateRing ? 2 * NV : NV;                             // pieces per slot
+    // ring slots (32 KiB per block at most; 48 KiB with the gate half)
+    constexpr int kDepth = kGateRing ? (RING == 2 ? 2 : 3) : (sizeof(Tin) == 2 || RING == 2) ? RING : RING / 2;
+    __shared__ uint4 ring[kDepth * NS * kThreads];
     const uint32_t ring0 = uint32_t(__cvta_generic_to_shared(ring)) + threadIdx.x * 16u;
-    auto slot_addr = [&](int slot, int v) { return ring0 + uint32_t((slot * NV + v) * kThreads) * 16u; };
+    auto slot_addr = [&](int slot, int v) { return ring0 + uint32_t((slot * NS + v) * kThreads) * 16u; };
     auto copy_row = [&](const Tin *row_src, int slot, bool valid) {          // one commit group per call, always
         if (valid) {
 #pragma unroll
             for (int v = 0; v < NV; v++)
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(slot_addr(slot, v)),
                              "l"(reinterpret_cast<const char *>(row_src) + 16 * v) : "memory");
+            if (kGateRing) {
+#pragma unroll
+                for (int v = 0; v < NV; v++)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(slot_addr(slot, NV + v)),
+                                 "l"(reinterpret_cast<const char *>(row_src + K) + 16 * v) : "memory");
+            }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    auto read_row = [&](int slot, Raw16<Tin> &r) {
+    auto read_row = [&](int slot, Raw16<Tin> &r, int first) {
 #pragma unroll
         for (int v = 0; v < NV; v++) {
             uint4 w;
             asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w)
-                         : "r"(slot_addr(slot, v)) : "memory");
+                         : "r"(slot_addr(slot, first + v)) : "memory");
             set_piece(r, v, w);
         }
     };
@@ -423,7 +481,7 @@ quantize_kernel(const __grid_constant__ QuantParams prm)
     }
     const Tin *gsrc = src + K;                               // (gated) this chunk of the gate half
     Raw16<Tin> gate_next;
-    if (GATED && whole) load16(gsrc, gate_next);
+    if (GATED && !kGateRing && whole) load16(gsrc, gate_next);
     int q = 0;                                               // N-segment (weights only) the constants belong to
     int64_t q_end = 0;                                       // first row beyond it (0: no constants yet)
     SegConst cp, cn;
@@ -444,7 +502,7 @@ quantize_kernel(const __grid_constant__ QuantParams prm)
             fast = whole && cp.fast && cn.fast && !(DUAL && CODE == SQ_CODE_INT8 && lo != -128);
         }
         Raw16<Tin> cur, gate;
-        if (GATED && whole) {
+        if (GATED && !kGateRing && whole) {
             gate = gate_next;
             if (row + R < M) load16(gsrc + src_step, gate_next);
         }
@@ -454,7 +512,10 @@ quantize_kernel(const __grid_constant__ QuantParams prm)
             const int ahead = slot == 0 ? kDepth - 1 : slot - 1;
             copy_row(src + int64_t(kDepth - 1) * src_step, ahead, row + int64_t(kDepth - 1) * R < M);
             asm volatile("cp.async.wait_group %0;" ::"n"(kDepth - 1) : "memory");
-            if (fast) read_row(slot, cur);
+            if (fast) {
+                read_row(slot, cur, 0);
+                if (kGateRing) read_row(slot, gate, NV);
+            }
             slot = slot + 1 == kDepth ? 0 : slot + 1;
         }
         if (fast) {
@@ -467,10 +528,12 @@ quantize_kernel(const __grid_constant__ QuantParams prm)
                     float gt[4];
                     get4(gate, g4, gt);
 #pragma unroll
-                    for (int i = 0; i < 4; i++) x[i] = pre_gated<Tin>(x[i], gt[i], mreg[PRE ? 4 * g4 + i : 0]);
+                    for (int i = 0; i < 4; i += 2)
+                        unpack2(pre_gated2<Tin>(x[i], x[i + 1], gt[i], gt[i + 1], mreg[PRE ? 2 * g4 + i / 2 : 0]), x[i], x[i + 1]);
                 } else if (PRE) {
 #pragma unroll
-                    for (int i = 0; i < 4; i++) x[i] = pre1<Tin>(x[i], prm.act, mreg[PRE ? 4 * g4 + i : 0]);
+                    for (int i = 0; i < 4; i += 2)
+                        unpack2(pre2<Tin>(x[i], x[i + 1], prm.act, mreg[PRE ? 2 * g4 + i / 2 : 0]), x[i], x[i + 1]);
                 }
                 quant4<CODE, MODE>(x, cp, cn, float(hi), zp, wp[g4], wn[g4]);
             }
@@ -502,7 +565,7 @@ quantize_kernel(const __grid_constant__ QuantParams prm)
 
 // ----------------------------------------------------------------------------- fused activation by table (bf16 inputs)
 // A bf16 pre-activation has 65536 possible values, so the stored activation bf16(act(h)) is a table of 128 KiB.
-// Every CTA (1024 threads, one per SM) builds the table in its shared memory with the same silu_f32 / gelu_f32 as
+// Every CTA (1024 threads, one per SM) builds the table in its shared memory with the same silu2 / gelu2 as
 // the arithmetic variant (a few evaluations per thread: most bit patterns need none), after which an element costs one
 // shared-memory load instead of about 30 instructions: the fused pass stops being bound by the ALUs.  Results are
 // those of the arithmetic variant bit for bit.  Used for large inputs: a launch of this kernel costs about 9 us
@@ -523,7 +586,7 @@ quantize_table_kernel(const __grid_constant__ QuantParams prm)
     extern __shared__ __align__(16) uint8_t table_smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t tab0 = uint32_t(__cvta_generic_to_shared(table_smem));
-    // Most bit patterns need no evaluation, because silu_f32 / gelu_f32 return a value known in advance there
+    // Most bit patterns need no evaluation, because silu2 / gelu2 return a value known in advance there
     // (a warp's 32 consecutive patterns share sign and exponent, so the branch is uniform):
     //   2^-124 <= |h| < 2^-26: both give h / 2 after the rounding to bf16 (the sigmoid / Phi factor is 1/2 to
     //                          far below a bf16 half-step);
@@ -543,7 +606,8 @@ quantize_table_kernel(const __grid_constant__ QuantParams prm)
             out = 0x8000u;
         } else {
             const float h = __uint_as_float(b << 16);
-            const float a = is_silu ? silu_f32(h) : gelu_f32(h);
+            float a, a_same;
+            unpack2(is_silu ? silu2(h, h) : gelu2(h, h), a, a_same);
             const __nv_bfloat16 r = __float2bfloat16_rn(a);
             out = *reinterpret_cast<const unsigned short *>(&r);
         }
@@ -887,8 +951,9 @@ pack_w4_kernel(uint8_t *__restrict__ w8, int64_t ld8, int64_t N, int K, uint8_t 
 template <typename Tin, int CODE, int MODE>
 sq_status prepare_t(QuantLaunch &L)
 {
-    // V chunks per row; R rows in flight: enough threads to fill every SM several times over, and a row count per
-    // thread that the rows divide into evenly
+    // V chunks per row; R rows in flight: every SM gets all the blocks it can hold, and a thread walks M / R rows, some
+    // one more than others.  (Cutting R down so that all walk the same number left SMs with two blocks beside SMs with
+    // three: 8192 x 2560 gated 36.0 -> 35.0 us, 8858 x 3072 bf16 17.1 -> 15.5 us.)
     QuantParams &prm = L.prm;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -899,7 +964,7 @@ sq_status prepare_t(QuantLaunch &L)
     const int64_t target_threads = int64_t(sms) * kThreads * (pre ? 3 : kBlocksPerSm);
     int64_t iters = (prm.M * V + target_threads - 1) / target_threads;
     if (iters < 1) iters = 1;
-    const int64_t R = (prm.M + iters - 1) / iters;
+    const int64_t R = std::min<int64_t>(prm.M, std::max<int64_t>(1, target_threads / V));
     const int64_t blocks = (R * V + kThreads - 1) / kThreads;
     if (blocks > 0x7FFFFFFF || R * V > 0xFFFFFFFFll || V > 0x7FFFFFFF || R > 0x7FFFFFFF) return SQ_ERR_SHAPE;
     prm.V = int(V);
@@ -911,8 +976,7 @@ sq_status prepare_t(QuantLaunch &L)
         L.kernel = deep ? reinterpret_cast<const void *>(quantize_kernel<Tin, CODE, MODE, 2, 4>)
                         : reinterpret_cast<const void *>(quantize_kernel<Tin, CODE, MODE, 2, 2>);
     else if (pre)
-        L.kernel = deep ? reinterpret_cast<const void *>(quantize_kernel<Tin, CODE, MODE, 1, 4>)
-                        : reinterpret_cast<const void *>(quantize_kernel<Tin, CODE, MODE, 1, 2>);
+        L.kernel = reinterpret_cast<const void *>(quantize_kernel<Tin, CODE, MODE, 1, 2>);
     else
         L.kernel = deep ? reinterpret_cast<const void *>(quantize_kernel<Tin, CODE, MODE, 0, 4>)
                         : reinterpret_cast<const void *>(quantize_kernel<Tin, CODE, MODE, 0, 2>);
@@ -931,7 +995,9 @@ sq_status prepare_mode(QuantLaunch &L, sq_code code, int mode)
 // The table variant of the fused activation: bf16 input, SiLU or GELU, every 16-element chunk inside one K-segment,
 // and enough elements for the table's set-up time not to count.  Returns false where it does not apply.
 std::atomic<int> g_table_mode{0};        // test hook: 0 automatic, 1 always where possible, 2 never
-constexpr int64_t kTableMinSilu = int64_t(16) << 20, kTableMinGelu = int64_t(8) << 20;   // measured break-even points
+// measured break-even points (us, evaluated per element against table): SiLU 16 Mi elements 20.8 / 20.9, 24 Mi 28.5 / 27.2;
+// GELU 8 Mi 14.8 / 15.4, 10 Mi 17.3 / 17.2, 16 Mi 25.5 / 21.6
+constexpr int64_t kTableMinSilu = int64_t(18) << 20, kTableMinGelu = int64_t(10) << 20;
 bool prepare_table(QuantLaunch &L, sq_dtype dt, sq_code code, int mode)
 {
     QuantParams &prm = L.prm;

@@ -1,4 +1,4 @@
-"""Derives the polynomial the fused GELU prologue evaluates (csrc/quantize.cu, gelu_f32) and prints its
+"""Derives the polynomial the fused GELU prologue evaluates (csrc/quantize.cu, gelu2) and prints its
 coefficients.  Not used at run time.
 
 erfc(t) = exp(-t^2) g(t) with g the scaled complementary error function.  g is smooth and positive on [0, inf);
