@@ -11,7 +11,10 @@ CSRC = os.path.join(_HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 LIB_PATH = os.path.join(_HERE, "libsegquant.so")
 OBJ_DIR = os.path.join(_HERE, "_build")
-SOURCES = ["api.cu", "calib.cu", "quantize.cu", "zero_point.cu", "gemm_tcgen05.cu"]
+# (source, object, defines): the GEMM's kernel instantiations are spread over four units that compile side by side
+UNITS = [(f, f.replace(".cu", ".o"), []) for f in ("api.cu", "calib.cu", "quantize.cu", "zero_point.cu", "gemm_tcgen05.cu")]
+UNITS += [("gemm_tcgen05.cu", f"gemm_kind{k}_npol{n}.o", [f"-DSQ_GEMM_KIND={k}", f"-DSQ_GEMM_NPOL={n}"])
+          for k in (0, 1) for n in (1, 2)]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC"]
 
@@ -32,13 +35,13 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ_DIR, exist_ok=True)
     extra = ["-Xptxas", "-v"] if verbose else []
 
-    def compile_one(src):
-        obj = os.path.join(OBJ_DIR, src.replace(".cu", ".o"))
-        subprocess.check_call([nvcc, *NVCC_FLAGS, *extra, "-I", INCLUDE, "-I", CSRC, "-c", os.path.join(CSRC, src), "-o", obj])
+    def compile_one(unit):
+        src, obj, defines = unit[0], os.path.join(OBJ_DIR, unit[1]), unit[2]
+        subprocess.check_call([nvcc, *NVCC_FLAGS, *extra, *defines, "-I", INCLUDE, "-I", CSRC, "-c", os.path.join(CSRC, src), "-o", obj])
         return obj
 
-    with ThreadPoolExecutor(max_workers=len(SOURCES)) as pool:
-        objs = list(pool.map(compile_one, SOURCES))
+    with ThreadPoolExecutor(max_workers=len(UNITS)) as pool:
+        objs = list(pool.map(compile_one, UNITS))
     subprocess.check_call([nvcc, "-shared", "-cudart", "static", "-gencode", "arch=compute_100a,code=sm_100a",
                            "-o", LIB_PATH, *objs])
     return LIB_PATH

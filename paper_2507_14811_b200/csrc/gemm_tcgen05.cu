@@ -6,9 +6,9 @@
 // activation rows and HALF of the weight tile, the pair's leader issues every MMA, and each CTA
 // holds the accumulators of its own 128 rows in its tensor memory (TMEM).  CG = 1 is the same
 // kernel with one CTA per 128-row tile (used when M <= 128).
-//   warp 0      TMA producer (one lane): per 128-byte K-block, one tile of each activation code
+//   warp 0      TMA producer (one elected lane): per 128-byte K-block, one tile of each activation code
 //               matrix and this CTA's part of ONE weight tile into a shared-memory ring
-//   warp 1      tcgen05.mma issuer (one lane, leader CTA only): for every 32-byte K-step one MMA of the
+//   warp 1      tcgen05.mma issuer (one elected lane, leader CTA only): for every 32-byte K-step one MMA of the
 //               positive (or only) code matrix against the weight tile; every (K-segment, polarity) has
 //               its own accumulator in TMEM
 //   warp 2      dual layers: the same for the negative code matrix, against the SAME weight tile
@@ -30,6 +30,8 @@
 // normally.  No load uses cluster multicast.
 // Host side: prepare_gemm works out everything a launch needs (tile plan, kernel instantiation, tensor maps,
 // shared-memory size, grid) without launching; run_gemm is one cudaLaunchKernelExC from that.
+// The file is compiled several times (build.py): with SQ_GEMM_KIND / SQ_GEMM_NPOL set, the kernel instantiations of that
+// code type and polarity count; without, the dispatch in front of them.  The units compile side by side.
 #include <atomic>
 #include <mutex>
 #include <vector>
@@ -37,11 +39,22 @@
 #include "sq_common.cuh"
 
 namespace sq {
+
+// Tile-plan overrides for benchmarking sweeps and tests (segquant_set_tuning); 0 = automatic.
+extern std::atomic<int> g_tune_tile_n, g_tune_stages, g_tune_cta_group, g_tune_seq;
+
+// Fills L for one code type (KIND 0 int8, 1 e4m3) and polarity count, given the tile plan.
+template <int KIND, int NPOL>
+sq_status prepare_kind(const GemmArgs &g, GemmLaunch &L, int cg, int tile_n, bool seq, int device, int sm_count);
+
+// Raises the kernel's dynamic shared-memory limit if need be; *clusters: how many CTA pairs can be resident (cg == 2).
+sq_status kernel_facts(int device, const void *kern, size_t smem, int cg, const cudaLaunchConfig_t &cfg, int *clusters);
+
 namespace {
 
 constexpr int TILE_M = 128;           // rows per CTA (TMEM lanes)
-constexpr int BLOCK_K = 128;          // bytes (= codes) per K-block: one 128B swizzle row
-constexpr int MMA_K = 32;             // codes per tcgen05.mma of an 8-bit kind
+[[maybe_unused]] constexpr int BLOCK_K = 128;          // bytes (= codes) per K-block: one 128B swizzle row
+[[maybe_unused]] constexpr int MMA_K = 32;             // codes per tcgen05.mma of an 8-bit kind
 constexpr int kEpiWarps = 8;
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kFrontThreads = 128;     // warpgroup 0: producer, MMA issuer, two idle warps
@@ -53,17 +66,26 @@ constexpr int kFrontRegs = 56, kEpiRegs = 224;     // per-thread register counts
 static_assert(kFrontThreads * kFrontRegs + kEpiThreads * kEpiRegs <= kThreads * kLaunchRegs,
               "register counts after the role split exceed the CTA's allocation");
 static_assert(kFrontRegs % 8 == 0 && kEpiRegs % 8 == 0 && kFrontRegs >= 24 && kEpiRegs <= 256, "setmaxnreg operand");
-constexpr int kEpiBufRegs = 192;      // of kEpiRegs: accumulator load buffers plus running sums (SEQ)
-constexpr int kResidentBufs = 4;      // accumulator load buffers of the resident epilogue
-constexpr int kMaxStages = 8;
+[[maybe_unused]] constexpr int kEpiBufRegs = 192;      // of kEpiRegs: accumulator load buffers plus running sums (SEQ)
+[[maybe_unused]] constexpr int kResidentBufs = 4;      // accumulator load buffers of the resident epilogue
+[[maybe_unused]] constexpr int kMaxStages = 8;
 constexpr int kTmemCols = 512;
-constexpr uint32_t kSmemBudget = 227 * 1024;
-constexpr long long kWaitLimitCycles = 4000000000ll;   // about 2 s
+[[maybe_unused]] constexpr int kMaxAccSets = 4;        // accumulator sets in TMEM (narrow SEQ tiles; otherwise 1 or 2)
+[[maybe_unused]] constexpr uint32_t kSmemBudget = 227 * 1024;
+[[maybe_unused]] constexpr long long kWaitLimitCycles = 4000000000ll;   // about 2 s
 constexpr uint32_t kStageBytesPerWarp = 32 * 64;       // one 32 x 32 bf16 output block per epilogue warp
-constexpr uint32_t kStageBytes = kEpiWarps * kStageBytesPerWarp;
+[[maybe_unused]] constexpr uint32_t kStageBytes = kEpiWarps * kStageBytesPerWarp;
 constexpr int kMaxTokenSegments = 32;                  // per-token layers: channel scales of up to 32 K-segments (32 KiB at 256 columns) are staged per tile
-constexpr int kMaxFactorTable = 2048;                  // (K-segments x polarities) x N-segments factors in shared memory
+[[maybe_unused]] constexpr int kMaxFactorTable = 2048;                  // (K-segments x polarities) x N-segments factors in shared memory
 
+// Split tiles hold 256 accumulator columns per CTA (two sets fit in TMEM, and a CTA's partial sums are 128 KiB):
+// 256-column tiles for single-scale layers, 128-column tiles for dual ones.  (256-column dual tiles were measured
+// too: twice the partial sums to exchange, one accumulator set, slower on every shape tried.)
+constexpr int sk_tile_n(int npol) { return npol == 2 ? 128 : 256; }
+constexpr size_t kSkSlotBytes = size_t(TILE_M) * 256 * 4;                  // one CTA's accumulators of such a tile
+inline size_t sk_counter_bytes(int64_t tiles) { return size_t((tiles * 2 * 4 + 255) / 256 * 256); }
+
+#ifdef SQ_GEMM_KIND
 // ----------------------------------------------------------------------------- PTX wrappers
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return uint32_t(__cvta_generic_to_shared(p)); }
@@ -153,6 +175,39 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
         }
     }
     return true;
+}
+
+// The same wait by a whole converged warp; every lane returns the same answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint32_t abort_flag,
+                                               uint32_t *status, uint32_t where)
+{
+    if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
+    long long t0 = 0;
+    uint32_t polls = 0;
+    while (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) {
+        if ((++polls & 63u) == 0) {
+            if (__any_sync(0xFFFFFFFFu, ld_shared_volatile_u32(abort_flag) != 0u)) return false;
+            const long long now = clock64();
+            if (t0 == 0) t0 = now;
+            if (__any_sync(0xFFFFFFFFu, now - t0 > kWaitLimitCycles)) {
+                st_shared_volatile_u32(abort_flag, 1u);
+                if ((threadIdx.x & 31) == 0) atomicCAS(status, 0u, where);
+                return false;
+            }
+        }
+    }
+    return true;
+}
+// One lane of a converged warp, the same one every time.  The loops that feed the TMA and the tensor pipe are run by
+// all 32 lanes and only the asynchronous instructions by the elected one: their operands then are warp-uniform
+// for the compiler.  (With the loops inside `if (lane == 0)` an issuing thread needed some 70 cycles per MMA, which
+// bounded every layer whose K-blocks give the pipe less than that.  8858 x 3072 -> 4608, two K-segments: 89.5 -> 80.8 us;
+// 1 x 7104 -> 768: 19.9 -> 15.8; 24 K-segments of 64 codes 58.3 -> 55.5; 149 x 1200 -> 576: 6.1 -> 5.1.)
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+    return ok != 0u;
 }
 
 // 2-D tiled TMA load into this CTA's shared memory; completion bytes go to `bar`, which for CG = 2
@@ -311,8 +366,8 @@ __host__ __device__ constexpr uint32_t epi_table_bytes(int nacc, int Q, int tile
 struct SharedHeader {
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
-    uint64_t tmem_full[2];
-    uint64_t tmem_empty[2];
+    uint64_t tmem_full[kMaxAccSets];
+    uint64_t tmem_empty[kMaxAccSets];
     uint32_t tmem_base;
     uint32_t abort_flag;
     uint32_t sk_flag;            // (split tiles) the arrival count the CTA's thread 0 read, for the other epilogue threads
@@ -669,7 +724,7 @@ __device__ __forceinline__ void store_slab(const uint64_t (&y2)[16], const Param
 // cache.  GENERIC = true adds the fp32 output, the accumulator dump for the parity tests and a
 // per-column factor lookup for slabs that straddle an N-bound.
 // SEQ = true (layers with more than one K-segment): TMEM holds the accumulators of ONE K-segment at a time,
-// in two alternating sets.  The MMA issuer fills a set with segment p while the epilogue warps drain the set
+// in two alternating sets (four on tiles of half the width, see prepare_gemm).  The MMA issuer fills a set with segment p while the epilogue warps drain the set
 // of segment p - 1, scale it and add it to fp32 running sums kept in registers for the whole tile; the sums
 // are converted and stored after the last segment.  Any number of K-segments fits, tiles stay wide, and the
 // drain of every segment but the last overlaps tensor work.  SEQ = false keeps every (segment, polarity)
@@ -732,7 +787,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
             mbar_init(smem_u32(&hdr->full[s]), 1);
             mbar_init(smem_u32(&hdr->empty[s]), kIssuers);      // one arrival per MMA-issuing thread
         }
-        for (int s = 0; s < 2; s++) {
+        for (int s = 0; s < kMaxAccSets; s++) {
             mbar_init(smem_u32(&hdr->tmem_full[s]), kIssuers);
             mbar_init(smem_u32(&hdr->tmem_empty[s]), CG * kEpiWarps);
         }
@@ -769,14 +824,14 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
     constexpr bool kSplitRel = (NPOL == 2 && TILE_N == 256 && !SEQ && !GENERIC && !SK) || WIDE;
     const int sk_pairs = min(num_units, num_tiles * prm.sk_kblocks);    // (SK) pairs that have a range
 
-    // The producer and the MMA issuer are single threads: their loops are kept to a few dozen
+    // The producer and the MMA issuer are one warp each: their loops are kept to a few dozen
     // instructions per K-block (ring slot and phase advance incrementally, descriptors by addition).
     if (warp < kFrontThreads / 32) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFrontRegs));
       if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            const uint32_t stages = prm.stages, P = prm.sb.P;
+        {
+            const uint32_t stages = prm.stages;
             const uint32_t full0 = smem_u32(&hdr->full[0]), empty0 = smem_u32(&hdr->empty[0]);
             grid_dependency_wait();                 // the code matrices come from the previous kernel
             // completion bytes of both CTAs' loads are counted on the leader's barrier
@@ -791,16 +846,19 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                     const int m0 = (tile / prm.num_n_tiles) * (TILE_M * CG) + int(rank) * TILE_M;
                     const int n0 = (tile % prm.num_n_tiles) * kTileCols + int(rank) * B_ROWS;
                     for (int kbi = k0; kbi < k1; kbi++) {
-                        if (!mbar_wait(empty0 + 8 * s, ph ^ 1, abort_flag, prm.status, kWhereProducer)) {
+                        if (!mbar_wait_warp(empty0 + 8 * s, ph ^ 1, abort_flag, prm.status, kWhereProducer)) {
                             ok = false;
                             break;
                         }
                         const uint32_t dst = ring0 + s * stage_bytes;
-                        if (rank == 0) mbar_expect_tx(full0 + 8 * s, CG * stage_bytes);
                         const uint32_t bar = full0_sig + 8 * s;
-                        tma_load_2d<CG>(dst, &tm_a_pos, bar, kbi * BLOCK_K, m0);
-                        if (NPOL == 2) tma_load_2d<CG>(dst + a_bytes, &tm_a_neg, bar, kbi * BLOCK_K, m0);
-                        tma_load_2d<CG>(dst + NPOL * a_bytes, &tm_b, bar, kbi * BLOCK_K, n0);
+                        if (elect_one()) {
+                            if (rank == 0) mbar_expect_tx(full0 + 8 * s, CG * stage_bytes);
+                            tma_load_2d<CG>(dst, &tm_a_pos, bar, kbi * BLOCK_K, m0);
+                            if (NPOL == 2) tma_load_2d<CG>(dst + a_bytes, &tm_a_neg, bar, kbi * BLOCK_K, m0);
+                            tma_load_2d<CG>(dst + NPOL * a_bytes, &tm_b, bar, kbi * BLOCK_K, n0);
+                        }
+                        __syncwarp();
                         issued++;
                         if (++s == stages) { s = 0; ph ^= 1; }
                     }
@@ -809,23 +867,23 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
             for (int tile = unit; !SK && tile < num_tiles && ok; tile += num_units) {
                 const int m0 = (tile / prm.num_n_tiles) * (TILE_M * CG) + int(rank) * TILE_M;
                 const int n0 = (tile % prm.num_n_tiles) * kTileCols + int(rank) * B_ROWS;
-                for (uint32_t p = 0; p < P && ok; p++) {
-                    const int k_end = prm.sb.kb[p + 1];
-                    for (int k = prm.sb.kb[p]; k < k_end; k += BLOCK_K) {
-                        if (!mbar_wait(empty0 + 8 * s, ph ^ 1, abort_flag, prm.status, kWhereProducer)) {
-                            ok = false;
-                            break;
-                        }
-                        const uint32_t dst = ring0 + s * stage_bytes;
+                for (int k = 0; k < prm.K; k += BLOCK_K) {         // K-blocks do not care about segment bounds
+                    if (!mbar_wait_warp(empty0 + 8 * s, ph ^ 1, abort_flag, prm.status, kWhereProducer)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t dst = ring0 + s * stage_bytes;
+                    const uint32_t bar = full0_sig + 8 * s;
+                    if (elect_one()) {
                         if (rank == 0) mbar_expect_tx(full0 + 8 * s, CG * stage_bytes);
-                        const uint32_t bar = full0_sig + 8 * s;
                         tma_load_2d<CG>(dst, &tm_a_pos, bar, k, m0);
                         if (NPOL == 2) tma_load_2d<CG>(dst + a_bytes, &tm_a_neg, bar, k, m0);
                         tma_load_2d<CG>(dst + NPOL * a_bytes, &tm_b, bar, k, n0);
                         if (WIDE) tma_load_2d<CG>(dst + NPOL * a_bytes + b_bytes, &tm_b, bar, k, n0 + TILE_N);
-                        issued++;
-                        if (++s == stages) { s = 0; ph ^= 1; }
                     }
+                    __syncwarp();
+                    issued++;
+                    if (++s == stages) { s = 0; ph ^= 1; }
                 }
             }
             grid_launch_dependents();               // all of this CTA's loads are issued: the tail begins
@@ -842,14 +900,13 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
         }
       } else if (warp == 1 || (kIssuers == 2 && warp == 2)) {
         // ------------------------------------------------------------------ MMA issuers (leader CTA)
-        // One thread per polarity: warp 1 issues the MMAs of the positive code matrix, warp 2 (dual layers)
-        // those of the negative one, each into its own accumulators.  A tcgen05.mma keeps its issuing thread
-        // busy for about 70 cycles, more than a 128-column MMA occupies the tensor pipe, so one thread cannot
-        // feed the pipe for narrow dual tiles.  Ring slots and accumulator sets are handed on when BOTH
-        // threads' MMAs have retired (barrier counts NPOL).  With the per-polarity release of a dual 256-wide
+        // One warp per polarity: warp 1 issues the MMAs of the positive code matrix, warp 2 (dual layers)
+        // those of the negative one, each into its own accumulators (the accumulators of a dual 256-wide tile come
+        // free one after the other, see kSplitRel).  Ring slots and accumulator sets are handed on when BOTH
+        // issuing threads' MMAs have retired (barrier counts NPOL).  With the per-polarity release of a dual 256-wide
         // tile each thread waits for its own accumulator only, so the positive thread starts the next tile
         // while the negative accumulator is still being read (it can run ahead by the depth of the ring).
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             const uint32_t pol = uint32_t(warp - 1);
             constexpr uint32_t idesc = make_idesc(KIND, TILE_N, TILE_M * CG);
             const uint32_t stages = prm.stages, P = prm.sb.P, acc_stages = prm.acc_stages;
@@ -865,7 +922,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                 SkWalk w = sk_range(unit, sk_pairs, num_tiles, prm.sk_kblocks);
                 int tile = 0, k0 = 0, k1 = 0;
                 while (ok && unit < sk_pairs && sk_next(w, tile, k0, k1)) {
-                    if (!mbar_wait(smem_u32(&hdr->tmem_empty[as]), aph ^ 1, abort_flag, prm.status, kWhereMmaTmem)) {
+                    if (!mbar_wait_warp(smem_u32(&hdr->tmem_empty[as]), aph ^ 1, abort_flag, prm.status, kWhereMmaTmem)) {
                         ok = false;
                         break;
                     }
@@ -873,7 +930,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                     const uint32_t d0 = tmem_base + as * acc_cols + pol * TILE_N;
                     uint32_t accumulate = 0;                       // a segment starts from zero wherever it begins in K
                     for (int kbi = k0; kbi < k1; kbi++) {
-                        if (!mbar_wait(full0 + 8 * s, ph, abort_flag, prm.status, kWhereMmaFull)) {
+                        if (!mbar_wait_warp(full0 + 8 * s, ph, abort_flag, prm.status, kWhereMmaFull)) {
                             ok = false;
                             break;
                         }
@@ -881,19 +938,21 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                         const uint64_t da = desc0 + s * kStageDesc;
                         const int rem = prm.K - kbi * BLOCK_K;
                         const int nk = rem >= BLOCK_K ? BLOCK_K / MMA_K : (rem + MMA_K - 1) / MMA_K;
-                        issue_kblock<KIND, 1, TILE_N, CG>(d0, da, da + b_off, idesc, nk, accumulate);
+                        if (elect_one()) {
+                            issue_kblock<KIND, 1, TILE_N, CG>(d0, da, da + b_off, idesc, nk, accumulate);
+                            tc_commit<CG>(empty0 + 8 * s);
+                        }
                         accumulate = 1;
-                        tc_commit<CG>(empty0 + 8 * s);
                         if (++s == stages) { s = 0; ph ^= 1; }
                     }
-                    if (ok) tc_commit<CG>(smem_u32(&hdr->tmem_full[as]));
+                    if (ok && elect_one()) tc_commit<CG>(smem_u32(&hdr->tmem_full[as]));
                     if (++as == acc_stages) { as = 0; aph ^= 1; }
                 }
             }
             for (int tile = unit; !SK && tile < num_tiles && ok; tile += num_units) {
                 if (!SEQ) {
                     const uint32_t bar = smem_u32(&hdr->tmem_empty[kSplitRel ? pol : as]);
-                    if (!mbar_wait(bar, aph ^ 1, abort_flag, prm.status, kWhereMmaTmem)) {
+                    if (!mbar_wait_warp(bar, aph ^ 1, abort_flag, prm.status, kWhereMmaTmem)) {
                         ok = false;
                         break;
                     }
@@ -901,7 +960,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                 }
                 for (uint32_t p = 0; p < P && ok; p++) {
                     if (SEQ) {                                     // one accumulator set per K-segment
-                        if (!mbar_wait(smem_u32(&hdr->tmem_empty[as]), aph ^ 1, abort_flag, prm.status, kWhereMmaTmem)) {
+                        if (!mbar_wait_warp(smem_u32(&hdr->tmem_empty[as]), aph ^ 1, abort_flag, prm.status, kWhereMmaTmem)) {
                             ok = false;
                             break;
                         }
@@ -910,8 +969,27 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                     const uint32_t d0 = tmem_base + as * acc_cols + (SEQ ? 0u : p * (NPOL * TILE_N)) + pol * TILE_N;
                     const int k_end = prm.sb.kb[p + 1];
                     uint32_t accumulate = 0;
-                    for (int k = prm.sb.kb[p]; k < k_end; k += BLOCK_K) {
-                        if (!mbar_wait(full0 + 8 * s, ph, abort_flag, prm.status, kWhereMmaFull)) {
+                    int k = prm.sb.kb[p];
+                    if (P > 1) {
+                        // K-segment bounds are multiples of 32, so every K-step of a K-block belongs to one segment: a
+                        // block that a bound cuts is loaded once, and each segment issues its own K-steps of it.  The
+                        // segment's first and last partial blocks are issued here and below, apart from the loop of
+                        // whole blocks, which has to stay as short as it is.
+                        if (k % BLOCK_K != 0) {                    // the block is in the ring: the segment before had its first part
+                            const int k_stop = min(k_end, (k + BLOCK_K) / BLOCK_K * BLOCK_K);
+                            const uint64_t da = desc0 + s * kStageDesc + uint64_t((k % BLOCK_K) >> 4);
+                            if (elect_one()) issue_kblock<KIND, 1, TILE_N, CG>(d0, da, da + b_off, idesc, (k_stop - k + MMA_K - 1) / MMA_K, 0u);
+                            accumulate = 1;
+                            k = k_stop;
+                            if (k % BLOCK_K == 0 || k == prm.K) {
+                                if (elect_one()) tc_commit<CG>(empty0 + 8 * s);
+                                if (++s == stages) { s = 0; ph ^= 1; }
+                            }
+                        }
+                    }
+                    const int k_loop = P == 1 || k_end == prm.K ? k_end : k_end / BLOCK_K * BLOCK_K;
+                    for (; k < k_loop; k += BLOCK_K) {
+                        if (!mbar_wait_warp(full0 + 8 * s, ph, abort_flag, prm.status, kWhereMmaFull)) {
                             ok = false;
                             break;
                         }
@@ -919,18 +997,29 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                         const uint64_t da = desc0 + s * kStageDesc;
                         const int rem = k_end - k;
                         const int nk = rem >= BLOCK_K ? BLOCK_K / MMA_K : (rem + MMA_K - 1) / MMA_K;
-                        issue_kblock<KIND, 1, TILE_N, CG>(d0, da, da + b_off, idesc, nk, accumulate);
+                        if (elect_one()) {
+                            issue_kblock<KIND, 1, TILE_N, CG>(d0, da, da + b_off, idesc, nk, accumulate);
+                            tc_commit<CG>(empty0 + 8 * s);         // the slot is free when both threads' MMAs have retired
+                        }
                         accumulate = 1;
-                        tc_commit<CG>(empty0 + 8 * s);             // the slot is free when both threads' MMAs have retired
                         if (++s == stages) { s = 0; ph ^= 1; }
                     }
+                    if (P > 1 && ok && k < k_end) {                // the segment ends inside this block
+                        if (!mbar_wait_warp(full0 + 8 * s, ph, abort_flag, prm.status, kWhereMmaFull)) {
+                            ok = false;
+                        } else {
+                            tc_fence_after();
+                            const uint64_t da = desc0 + s * kStageDesc;
+                            if (elect_one()) issue_kblock<KIND, 1, TILE_N, CG>(d0, da, da + b_off, idesc, (k_end - k) / MMA_K, accumulate);
+                        }
+                    }
                     if (SEQ) {
-                        if (ok) tc_commit<CG>(smem_u32(&hdr->tmem_full[as]));  // accumulators of this segment complete
+                        if (ok && elect_one()) tc_commit<CG>(smem_u32(&hdr->tmem_full[as]));  // accumulators of this segment complete
                         if (++as == acc_stages) { as = 0; aph ^= 1; }
                     }
                 }
                 if (!SEQ) {
-                    if (ok) tc_commit<CG>(smem_u32(&hdr->tmem_full[as]));  // accumulators of this tile complete
+                    if (ok && elect_one()) tc_commit<CG>(smem_u32(&hdr->tmem_full[as]));  // accumulators of this tile complete
                     if (++as == acc_stages) { as = 0; aph ^= 1; }
                 }
             }
@@ -1061,7 +1150,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                 }
                 for (int p = 0; p < P; p++) {
                     const uint32_t cur_as = as, cur_aph = aph;
-                    if (++as == 2u) { as = 0; aph ^= 1; }
+                    if (++as == uint32_t(prm.acc_stages)) { as = 0; aph ^= 1; }
                     if (ok) ok = mbar_wait(smem_u32(&hdr->tmem_full[cur_as]), cur_aph, abort_flag, prm.status, kWhereEpilogue);
                     if (!ok) continue;
                     tc_fence_after();
@@ -1441,52 +1530,6 @@ bool make_map_y(CUtensorMap *map, void *base, int64_t M, int64_t N, int64_t ldy)
     return r == CUDA_SUCCESS;
 }
 
-// Tile-plan overrides for benchmarking sweeps and tests (segquant_set_tuning); 0 = automatic.
-std::atomic<int> g_tune_tile_n{0}, g_tune_stages{0}, g_tune_cta_group{0}, g_tune_seq{0};
-
-// What has been found out per (device, kernel instantiation, dynamic shared-memory size): how many CTA pairs can
-// be resident; and per (device, kernel instantiation) the largest dynamic shared-memory size the kernel's
-// attribute has been raised to (it is only ever raised, so that earlier plans stay launchable).  Guarded by a
-// mutex; a handful of entries.
-struct KernelFacts { int device; const void *kernel; size_t smem; int clusters; };
-struct KernelSmem { int device; const void *kernel; size_t max_smem; };
-std::mutex g_facts_mu;
-std::vector<KernelFacts> g_facts;
-std::vector<KernelSmem> g_smem;
-
-template <typename Kern>
-sq_status kernel_facts(int device, Kern kern, size_t smem, int cg, const cudaLaunchConfig_t &cfg, int *clusters)
-{
-    const void *key = reinterpret_cast<const void *>(kern);
-    std::lock_guard<std::mutex> lock(g_facts_mu);
-    KernelSmem *ks = nullptr;
-    for (KernelSmem &e : g_smem)
-        if (e.device == device && e.kernel == key) ks = &e;
-    if (!ks || ks->max_smem < smem) {
-        const cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (ea != cudaSuccess) { note_cuda_error(ea); return SQ_ERR_CUDA; }
-        if (ks) ks->max_smem = smem;
-        else g_smem.push_back({device, key, smem});
-    }
-    for (const KernelFacts &f : g_facts)
-        if (f.device == device && f.kernel == key && f.smem == smem) { *clusters = f.clusters; return SQ_OK; }
-    int n = 0;
-    if (cg == 2) {
-        const cudaError_t eo = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-        if (eo != cudaSuccess || n <= 0) { note_cuda_error(eo != cudaSuccess ? eo : cudaErrorLaunchOutOfResources); return SQ_ERR_CUDA; }
-    }
-    g_facts.push_back({device, key, smem, n});
-    *clusters = n;
-    return SQ_OK;
-}
-
-// Split tiles hold 256 accumulator columns per CTA (two sets fit in TMEM, and a CTA's partial sums are 128 KiB):
-// 256-column tiles for single-scale layers, 128-column tiles for dual ones.  (256-column dual tiles were measured
-// too: twice the partial sums to exchange, one accumulator set, slower on every shape tried.)
-constexpr int sk_tile_n(int npol) { return npol == 2 ? 128 : 256; }
-constexpr size_t kSkSlotBytes = size_t(TILE_M) * 256 * 4;                  // one CTA's accumulators of such a tile
-inline size_t sk_counter_bytes(int64_t tiles) { return size_t((tiles * 2 * 4 + 255) / 256 * 256); }
-
 template <int KIND, int NPOL, int TILE_N, int CG, bool GENERIC, bool SEQ, bool WIDE = false, bool PT = false, bool SK = false>
 sq_status prepare_variant(const GemmArgs &g, GemmLaunch &L, int device, int sm_count)
 {
@@ -1529,7 +1572,7 @@ sq_status prepare_variant(const GemmArgs &g, GemmLaunch &L, int device, int sm_c
 
     // persistent grid: one CTA (pair) per SM (pair) that can be resident at the same time
     int units = sm_count / CG, clusters = 0;
-    const sq_status fs = kernel_facts(device, kern, smem, CG, cfg, &clusters);
+    const sq_status fs = kernel_facts(device, reinterpret_cast<const void *>(kern), smem, CG, cfg, &clusters);
     if (fs != SQ_OK) return fs;
     if (CG == 2 && clusters < units) units = clusters;
     const int tiles = prm.num_m_tiles * prm.num_n_tiles;
@@ -1567,12 +1610,16 @@ sq_status prepare_tile(const GemmArgs &g, GemmLaunch &L, int tile_n, bool seq, i
     // it does for up to 32 K-segments, int8 codes and CTA pairs; anything else runs the checking variant
     const bool pt = prm.col_scale != nullptr;
     if (pt && !(KIND == 0 && CG == 2 && prm.sb.P <= kMaxTokenSegments)) dbg = true;
-    if (seq) {      // sequential K-segments: one tile width per polarity count
-        constexpr int TN = NPOL == 1 ? 256 : 128;
+    if (seq) {      // sequential K-segments
+        constexpr int TN = NPOL == 1 ? 256 : 128;         // two accumulator sets fill TMEM
+        const bool narrow = tile_n < TN && !dbg;          // half that width and four sets: see prepare_gemm
+        prm.acc_stages = narrow ? 4 : 2;
         if (dbg) return prepare_variant<KIND, NPOL, TN, CG, true, true>(g, L, device, sm_count);
         if constexpr (KIND == 0 && CG == 2)
-            if (pt) return prepare_variant<KIND, NPOL, TN, CG, false, true, false, true>(g, L, device, sm_count);
-        return prepare_variant<KIND, NPOL, TN, CG, false, true>(g, L, device, sm_count);
+            if (pt) return narrow ? prepare_variant<KIND, NPOL, TN / 2, CG, false, true, false, true>(g, L, device, sm_count)
+                                  : prepare_variant<KIND, NPOL, TN, CG, false, true, false, true>(g, L, device, sm_count);
+        return narrow ? prepare_variant<KIND, NPOL, TN / 2, CG, false, true>(g, L, device, sm_count)
+                      : prepare_variant<KIND, NPOL, TN, CG, false, true>(g, L, device, sm_count);
     }
     if constexpr (KIND == 0 && CG == 2) {
         if (pt && !dbg) {     // 256- and 128-column tiles only (the automatic choice never goes below for these layers)
@@ -1641,17 +1688,69 @@ sq_status prepare_tile(const GemmArgs &g, GemmLaunch &L, int tile_n, bool seq, i
     return SQ_ERR_UNSUPPORTED;
 }
 
-template <int KIND>
-sq_status prepare_kind(const GemmArgs &g, GemmLaunch &L, int npol, int cg, int tile_n, bool seq, int device, int sm_count)
+}  // namespace
+
+template <>
+sq_status prepare_kind<SQ_GEMM_KIND, SQ_GEMM_NPOL>(const GemmArgs &g, GemmLaunch &L, int cg, int tile_n, bool seq, int device,
+                                                  int sm_count)
 {
-    if (npol == 2)
-        return cg == 2 ? prepare_tile<KIND, 2, 2>(g, L, tile_n, seq, device, sm_count)
-                       : prepare_tile<KIND, 2, 1>(g, L, tile_n, seq, device, sm_count);
-    return cg == 2 ? prepare_tile<KIND, 1, 2>(g, L, tile_n, seq, device, sm_count)
-                   : prepare_tile<KIND, 1, 1>(g, L, tile_n, seq, device, sm_count);
+    return cg == 2 ? prepare_tile<SQ_GEMM_KIND, SQ_GEMM_NPOL, 2>(g, L, tile_n, seq, device, sm_count)
+                   : prepare_tile<SQ_GEMM_KIND, SQ_GEMM_NPOL, 1>(g, L, tile_n, seq, device, sm_count);
 }
 
+#else   // the dispatch
+
+// What has been found out per (device, kernel instantiation, dynamic shared-memory size): how many CTA pairs can
+// be resident; and per (device, kernel instantiation) the largest dynamic shared-memory size the kernel's
+// attribute has been raised to (it is only ever raised, so that earlier plans stay launchable).  Guarded by a
+// mutex; a handful of entries.
+struct KernelFacts { int device; const void *kernel; size_t smem; int clusters; };
+struct KernelSmem { int device; const void *kernel; size_t max_smem; };
+std::mutex g_facts_mu;
+std::vector<KernelFacts> g_facts;
+std::vector<KernelSmem> g_smem;
+
 }  // namespace
+
+std::atomic<int> g_tune_tile_n{0}, g_tune_stages{0}, g_tune_cta_group{0}, g_tune_seq{0};
+
+sq_status kernel_facts(int device, const void *key, size_t smem, int cg, const cudaLaunchConfig_t &cfg, int *clusters)
+{
+    std::lock_guard<std::mutex> lock(g_facts_mu);
+    KernelSmem *ks = nullptr;
+    for (KernelSmem &e : g_smem)
+        if (e.device == device && e.kernel == key) ks = &e;
+    if (!ks || ks->max_smem < smem) {
+        const cudaError_t ea = cudaFuncSetAttribute(key, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        if (ea != cudaSuccess) { note_cuda_error(ea); return SQ_ERR_CUDA; }
+        if (ks) ks->max_smem = smem;
+        else g_smem.push_back({device, key, smem});
+    }
+    for (const KernelFacts &f : g_facts)
+        if (f.device == device && f.kernel == key && f.smem == smem) { *clusters = f.clusters; return SQ_OK; }
+    int n = 0;
+    if (cg == 2) {
+        const cudaError_t eo = cudaOccupancyMaxActiveClusters(&n, key, &cfg);
+        if (eo != cudaSuccess || n <= 0) { note_cuda_error(eo != cudaSuccess ? eo : cudaErrorLaunchOutOfResources); return SQ_ERR_CUDA; }
+    }
+    g_facts.push_back({device, key, smem, n});
+    *clusters = n;
+    return SQ_OK;
+}
+
+extern template sq_status prepare_kind<0, 1>(const GemmArgs &, GemmLaunch &, int, int, bool, int, int);
+extern template sq_status prepare_kind<0, 2>(const GemmArgs &, GemmLaunch &, int, int, bool, int, int);
+extern template sq_status prepare_kind<1, 1>(const GemmArgs &, GemmLaunch &, int, int, bool, int, int);
+extern template sq_status prepare_kind<1, 2>(const GemmArgs &, GemmLaunch &, int, int, bool, int, int);
+
+static sq_status prepare_for(const GemmArgs &g, GemmLaunch &L, int npol, int cg, int tile_n, bool seq, int device, int sm_count)
+{
+    if (g.code == SQ_CODE_INT8)
+        return npol == 2 ? prepare_kind<0, 2>(g, L, cg, tile_n, seq, device, sm_count)
+                         : prepare_kind<0, 1>(g, L, cg, tile_n, seq, device, sm_count);
+    return npol == 2 ? prepare_kind<1, 2>(g, L, cg, tile_n, seq, device, sm_count)
+                     : prepare_kind<1, 1>(g, L, cg, tile_n, seq, device, sm_count);
+}
 
 size_t gemm_split_scratch_bytes(int64_t M, int64_t N, int dual)
 {
@@ -1710,9 +1809,16 @@ sq_status prepare_gemm(const GemmArgs &g, GemmLaunch *out)
     if (tune_seq == 2) seq = true;
     if (prm.nacc * g.sb.Q > kMaxFactorTable) return SQ_ERR_UNSUPPORTED;
     if (seq) {
-        prm.acc_stages = 2;
-        return g.code == SQ_CODE_INT8 ? prepare_kind<0>(g, L, npol, cg, 0, true, dev, sm_count)
-                                      : prepare_kind<1>(g, L, npol, cg, 0, true, dev, sm_count);
+        const int wide_n = npol == 1 ? 256 : 128;
+        int tile_n = wide_n;
+        // The tile of half the width, with four accumulator sets in flight, is the better one as long as it costs no
+        // further wave: its epilogue handles half the columns per segment.  (us, wide / narrow, K-segments of 64 codes:
+        // 1024 x 1536 -> 1536 on 24 / 48 of 74 CTA pairs 20.2 / 17.0; 8858 rows, 210 / 420 tiles, 55.4 / 83.9.)
+        const int64_t m_tiles = (g.M + TILE_M * cg - 1) / (TILE_M * cg), units = sm_count / cg;
+        auto waves = [&](int tn) { return (m_tiles * ((g.N + tn - 1) / tn) + units - 1) / units; };
+        if (waves(wide_n / 2) <= waves(wide_n)) tile_n = wide_n / 2;
+        if (tune_tile_n == wide_n || tune_tile_n == wide_n / 2) tile_n = tune_tile_n;
+        return prepare_for(g, L, npol, cg, tile_n, true, dev, sm_count);
     }
 
     // Tile width: the widest tile whose accumulators fit the 512 TMEM columns, unless half that width
@@ -1740,8 +1846,7 @@ sq_status prepare_gemm(const GemmArgs &g, GemmLaunch *out)
         tile_n = tune_tile_n;
     prm.acc_stages = (2 * tile_n * prm.nacc <= kTmemCols) ? 2 : 1;
 
-    return g.code == SQ_CODE_INT8 ? prepare_kind<0>(g, L, npol, cg, tile_n, false, dev, sm_count)
-                                  : prepare_kind<1>(g, L, npol, cg, tile_n, false, dev, sm_count);
+    return prepare_for(g, L, npol, cg, tile_n, false, dev, sm_count);
 }
 
 // One launch from a prepared plan: no queries, no encoding.
@@ -1775,5 +1880,7 @@ sq_status launch_gemm(const GemmArgs &g, cudaStream_t st)
     const sq_status s = prepare_gemm(g, &L);
     return s == SQ_OK ? run_gemm(L, st) : s;
 }
+
+#endif
 
 }  // namespace sq

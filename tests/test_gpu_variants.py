@@ -520,3 +520,31 @@ def test_w4a8_calls_reject_bad_arguments_before_launch():
                              B.new_workspace(DEV))
     assert e.value.status == 3                                                      # output segments: not with per-channel scales
     assert B.segquant_launch_count() == n0
+
+
+# ------------------------------------------------------------------ K-segments that cut K-blocks, both tile widths
+
+@pytest.mark.parametrize("M", [5, 300])
+@pytest.mark.parametrize("code,dual", [("int8", True), ("int8", False), ("e4m3", True), ("e4m3", False)])
+@pytest.mark.parametrize("kb", [
+    [0, 32, 64, 96, 128], [0, 96, 416], [0, 160, 192, 224, 400], [0, 128, 256, 288], list(range(0, 2049, 64)),
+])
+def test_segments_inside_a_k_block_on_both_tile_widths(kb, code, dual, M):
+    """Several K-segments in one 128-code block, blocks cut by a bound, a last block that is not whole, more segments
+    than accumulator sets: both tile widths give the checking variant's output (whose accumulators the parity tests
+    hold to the oracle) bit for bit, since all add the same terms in the same order."""
+    K, N = kb[-1], 328
+    spec = custom_spec("cut_blocks", M, K, N, kb, [0, N], dual, code, x_kind="normal+gelu" if dual else "normal", seed=71,
+                       x_seg_std=[0.5 + 0.25 * i for i in range(len(kb) - 1)])
+    data = WL.make_layer(spec)
+    layer = SegQuantLinear(data.W, data.bias, kb, [0, N], dual, code, DEV)
+    layer.calibrate(data.X_cal)
+    ref, _, _, _ = layer.forward_steps(data.X.to(DEV), dump_acc=True)
+    try:
+        for tile_n in (256, 128, 64):                # the width a polarity count does not have falls back to the automatic one
+            B.segquant_set_tuning(tile_n=tile_n)
+            Y = layer.forward(data.X.to(DEV))
+            layer.check_status()
+            assert torch.equal(Y, ref), tile_n
+    finally:
+        B.segquant_set_tuning()
