@@ -499,6 +499,9 @@ __device__ __forceinline__ void issue_kblock(uint32_t d0, uint64_t da, uint64_t 
 
 // ----------------------------------------------------------------------------- epilogue pieces
 
+// Variants of the kernel's epilogue (see the kernel).
+enum : int { kProduction = 0, kFlexible = 1, kChecking = 2 };
+
 // N-segment of column n: the number of interior bounds nb[1..Q-1] that are <= n, counted warp-wide
 // (all 32 lanes call it together).
 __device__ __forceinline__ int seg_of_column(int n, int Q, uint32_t nb_addr, int lane)
@@ -510,6 +513,20 @@ __device__ __forceinline__ int seg_of_column(int n, int Q, uint32_t nb_addr, int
         cnt += __popc(__ballot_sync(0xFFFFFFFFu, le));
     }
     return cnt;
+}
+
+// N-segments of the 32 columns nf .. nf + 31 of a slab: of the first (lo), the last (hi) and this lane's own column.
+struct SlabSegs { int lo, hi, lane; };
+template <int VAR>
+__device__ __forceinline__ SlabSegs slab_segs(int nf, int N, int Q, uint32_t nb_addr, int lane)
+{
+    SlabSegs g;
+    g.lo = seg_of_column(min(nf, N - 1), Q, nb_addr, lane);
+    g.hi = VAR == kProduction ? g.lo : seg_of_column(min(nf + 31, N - 1), Q, nb_addr, lane);
+    g.lane = g.lo;
+    if (VAR == kFlexible)
+        while (g.lane < g.hi && nf + lane >= int(ld_shared_u32(nb_addr + 4u * uint32_t(g.lane + 1)))) g.lane++;
+    return g;
 }
 
 // y += c[a][q(column)] * acc for the 32 columns nf .. nf + 31 of one row; y holds 16 packed fp32 pairs, r the
@@ -538,11 +555,12 @@ __device__ __forceinline__ uint64_t ld_shared_64(uint32_t addr)
     return v;
 }
 
-template <int KIND, bool GENERIC, bool INIT = false, bool PT = false>
+template <int KIND, int VAR, bool INIT = false, bool PT = false>
 __device__ __forceinline__ void scale_add_unit(uint64_t (&y2)[16], const uint32_t (&r)[32], int a, int Q, int q_lo,
                                                int q_hi, int nf, uint32_t tab_addr, uint32_t nb_addr,
-                                               uint32_t bias_slab = 0, const TokenScale *ts = nullptr)
+                                               uint32_t bias_slab = 0, const TokenScale *ts = nullptr, int q_lane = 0)
 {
+    constexpr bool GENERIC = VAR == kChecking;
     if (GENERIC && ts && ts->col_scale) {
         if (INIT) {
 #pragma unroll
@@ -569,7 +587,7 @@ __device__ __forceinline__ void scale_add_unit(uint64_t (&y2)[16], const uint32_
         }
         return;
     }
-    if (!GENERIC || q_lo == q_hi) {
+    if (VAR == kProduction || q_lo == q_hi) {
         // PT (production variant of the per-token layer): the token's scale times the staged channel scales
         const float c = PT ? ts->row_factor : ld_shared_f32(tab_addr + uint32_t(a * Q + q_lo) * 4u);
         uint64_t c2 = pack_f32x2(c, c);
@@ -582,6 +600,23 @@ __device__ __forceinline__ void scale_add_unit(uint64_t (&y2)[16], const uint32_
             for (int t = 0; t < 2; t++) {
                 const int j = 2 * j4 + t;
                 if (PT) c2 = mul_f32x2(rf2, ld_shared_64(ts->col_smem + uint32_t(nf + 2 * j) * 4u));
+                const uint64_t v2 = KIND == 0 ? pack_f32x2(__int2float_rn(int(r[2 * j])), __int2float_rn(int(r[2 * j + 1])))
+                                              : pack_b32x2(r[2 * j], r[2 * j + 1]);
+                y2[j] = fma_f32x2(c2, v2, t == 0 ? b0 : b1);
+            }
+        }
+    } else if (VAR == kFlexible) {
+        // the slab straddles an N-bound: every lane reads the factor of its own column (N-segment q_lane), the columns
+        // get theirs by shuffle
+        const float cl = ld_shared_f32(tab_addr + uint32_t(a * Q + q_lane) * 4u);
+#pragma unroll
+        for (int j4 = 0; j4 < 8; j4++) {
+            uint64_t b0 = y2[2 * j4], b1 = y2[2 * j4 + 1];
+            if (INIT) ld_shared_2x64(bias_slab + uint32_t(16 * j4), b0, b1);
+#pragma unroll
+            for (int t = 0; t < 2; t++) {
+                const int j = 2 * j4 + t;
+                const uint64_t c2 = pack_f32x2(__shfl_sync(0xFFFFFFFFu, cl, 2 * j), __shfl_sync(0xFFFFFFFFu, cl, 2 * j + 1));
                 const uint64_t v2 = KIND == 0 ? pack_f32x2(__int2float_rn(int(r[2 * j])), __int2float_rn(int(r[2 * j + 1])))
                                               : pack_b32x2(r[2 * j], r[2 * j + 1]);
                 y2[j] = fma_f32x2(c2, v2, t == 0 ? b0 : b1);
@@ -661,6 +696,26 @@ __device__ __forceinline__ void tma_store_block(const uint32_t (&h)[16], const Y
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     }
 }
+// The same for 32 fp32 outputs per lane: 128-byte rows, 128-byte swizzle, a staging buffer of 4 KiB.
+__device__ __forceinline__ void tma_store_block_f32(const uint64_t (&y2)[16], const YOut &yo, int col, int M, int N)
+{
+    if (yo.row0 >= M || col >= N) return;               // warp-uniform
+    if (yo.lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    __syncwarp();
+    const uint32_t row_addr = yo.stage + uint32_t(yo.lane) * 128u;
+    const uint32_t sw = uint32_t(yo.lane) & 7u;         // 16-byte piece index ^ row within the 8-row group
+#pragma unroll
+    for (int c = 0; c < 8; c++)
+        asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(row_addr + ((uint32_t(c) ^ sw) << 4)),
+                     "l"(y2[2 * c]), "l"(y2[2 * c + 1]) : "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (yo.lane == 0) {
+        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
+                     ::"l"(reinterpret_cast<uint64_t>(yo.tm)), "r"(col), "r"(yo.row0), "r"(yo.stage) : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
+}
 // before the CTA's shared memory goes away (all lanes may call; lane 0 issued the stores)
 __device__ __forceinline__ void tma_store_drain(const YOut &yo)
 {
@@ -671,13 +726,15 @@ __device__ __forceinline__ void tma_store_drain(const YOut &yo)
 // Converts and stores the 32 outputs y of row `row`, columns nf .. nf + 31, in 16-byte chunks (8 bf16 or
 // 4 fp32).  N is a multiple of 8, so a chunk is entirely inside or outside the matrix; two adjacent chunks go
 // out as one 32-byte store when the rows of Y are 32-byte aligned.
-// The production variant (GENERIC = false) is called by all 32 lanes of the warp together and writes through
-// yo; the generic one writes row `row` (< M) from registers.
-template <bool GENERIC, typename Params>
+// The production and flexible variants are called by all 32 lanes of the warp together and write through
+// yo; the checking one writes row `row` (< M) from registers.
+template <int VAR, typename Params>
 __device__ __forceinline__ void store_slab(const uint64_t (&y2)[16], const Params &prm, int row, int nf, const YOut &yo)
 {
     const int nvalid = prm.N - nf;                       // valid columns of this slab, may exceed 32
-    if (!GENERIC) {
+    if (VAR == kFlexible && prm.y_is_f32) {
+        tma_store_block_f32(y2, yo, nf, prm.M, prm.N);
+    } else if (VAR != kChecking) {
         uint32_t h[16];
         pack_bf16(y2, h);
         tma_store_block(h, yo, nf, prm.M, prm.N);
@@ -718,11 +775,14 @@ __device__ __forceinline__ void store_slab(const uint64_t (&y2)[16], const Param
     }
 }
 
-// GENERIC = false is the production variant: bf16 output, no accumulator dump, every interior N-bound
+// VAR = kProduction: bf16 output, no accumulator dump, every interior N-bound
 // a multiple of 32 (so that each 32-column slab of the output lies in one N-segment and takes ONE
 // dequantization factor per accumulator).  Its epilogue loop is small enough for the instruction
-// cache.  GENERIC = true adds the fp32 output, the accumulator dump for the parity tests and a
-// per-column factor lookup for slabs that straddle an N-bound.
+// cache.  VAR = kFlexible takes fp32 output too (TMA stores as well, 4 KiB per block) and slabs that straddle an
+// N-bound, whose factors come by shuffle (2 x 1280 -> 8784 with 10 K- and 6 N-segments: 41.8 us in the checking variant,
+// 8.7 here; 940 x 256 -> 8944 to fp32: 13.3 -> 10.4).  VAR = kChecking adds the accumulator dump for the parity tests,
+// rows of Y that TMA cannot write, and what else the other two do not take; it stores directly and looks the factors of
+// straddling slabs up column by column.
 // SEQ = true (layers with more than one K-segment): TMEM holds the accumulators of ONE K-segment at a time,
 // in two alternating sets (four on tiles of half the width, see prepare_gemm).  The MMA issuer fills a set with segment p while the epilogue warps drain the set
 // of segment p - 1, scale it and add it to fp32 running sums kept in registers for the whole tile; the sums
@@ -741,7 +801,7 @@ __device__ __forceinline__ void store_slab(const uint64_t (&y2)[16], const Param
 // of a tile's K range writes its raw accumulators (exact int32 sums, or fp32 ones) to a slot of the caller's
 // workspace and counts itself in on the tile's counter; the CTA whose count completes the tile adds the slots up,
 // in the order of the K ranges, and runs the tile's epilogue.  Nobody waits for anybody.
-template <int KIND, int NPOL, int TILE_N, int CG, bool GENERIC, bool SEQ, bool WIDE = false, bool PT = false, bool SK = false>
+template <int KIND, int NPOL, int TILE_N, int CG, int VAR, bool SEQ, bool WIDE = false, bool PT = false, bool SK = false>
 // 384 threads = 12 warps, 3 on each SM sub-partition with 16 K registers: 168 registers per thread at launch
 __global__ void __launch_bounds__(kThreads, 1)
 segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_constant__ CUtensorMap tm_a_neg,
@@ -749,6 +809,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                      const KernelParams prm)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
+    constexpr bool GENERIC = VAR == kChecking;
     // layout: [ring: stages x (NPOL A tiles of 16 KiB, B part of B_ROWS*128 B)] [output staging] [scales] [header]
     constexpr int B_ROWS = TILE_N / CG;                  // weight rows this CTA loads per K-block
     constexpr uint32_t a_bytes = TILE_M * BLOCK_K;
@@ -756,12 +817,12 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
     constexpr int kHalves = WIDE ? 2 : 1;                // weight tiles per stage
     constexpr int kTileCols = TILE_N * kHalves;          // output columns of a tile
     constexpr int kIssuers = (NPOL == 2 || WIDE) ? 2 : 1;
-    static_assert(!WIDE || (NPOL == 1 && TILE_N == 256 && CG == 2 && !GENERIC && !SEQ), "wide single-scale tile");
-    static_assert(!SK || (CG == 2 && !GENERIC && !SEQ && !WIDE && !PT && NPOL * TILE_N == 256), "split tiles");
+    static_assert(!WIDE || (NPOL == 1 && TILE_N == 256 && CG == 2 && VAR == kProduction && !SEQ), "wide single-scale tile");
+    static_assert(!SK || (CG == 2 && VAR == kProduction && !SEQ && !WIDE && !PT && NPOL * TILE_N == 256), "split tiles");
     constexpr uint32_t stage_bytes = NPOL * a_bytes + kHalves * b_bytes;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *sh_stage = smem + size_t(prm.stages) * stage_bytes;      // 1 KiB aligned: stages are multiples of 1 KiB
-    float *sh_bias = reinterpret_cast<float *>(sh_stage + (GENERIC ? 0 : kStageBytes));     // [TILE_N], per tile
+    float *sh_bias = reinterpret_cast<float *>(sh_stage + (GENERIC ? 0 : VAR == kFlexible && prm.y_is_f32 ? 2 * kStageBytes : kStageBytes));     // [TILE_N], per tile
     float *sh_tab = sh_bias + kTileCols;                                                    // [nacc][Q], per launch
     int *sh_nb = reinterpret_cast<int *>(sh_tab + prm.nacc * prm.sb.Q);                     // [Q + 1]
     // (per-token mode, few K-segments) the tile's channel scales [P][kTileCols], refreshed per tile
@@ -1087,7 +1148,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
         };
         for (int i = et; i <= Q; i += kEpiThreads) sh_nb[i] = prm.sb.nb[i];
 
-        YOut yo{&tm_y, smem_u32(sh_stage) + uint32_t(ew) * kStageBytesPerWarp, lane, 0};
+        YOut yo{&tm_y, smem_u32(sh_stage) + uint32_t(ew) * (VAR == kFlexible && prm.y_is_f32 ? 2 * kStageBytesPerWarp : kStageBytesPerWarp), lane, 0};
         uint32_t as = 0, aph = 0;
         bool ok = true;
         int tile = unit - num_units;
@@ -1138,12 +1199,11 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                 constexpr int kRel = kUnits <= NB ? 0 : kUnits - NB + 1;    // unit before which the set is released
                 static_assert(NB >= 2 || kUnits == 1, "needs two load buffers");
                 uint64_t y2[kSlabsPerWarp][16];
-                int q_lo[kSlabsPerWarp], q_hi[kSlabsPerWarp];
+                SlabSegs q[kSlabsPerWarp];
 #pragma unroll
                 for (int sl = 0; sl < kSlabsPerWarp; sl++) {
                     const int c0 = (slab0 + sl) * 32;
-                    q_lo[sl] = seg_of_column(n0 + c0, Q, nb_addr, lane);
-                    q_hi[sl] = GENERIC ? seg_of_column(min(n0 + c0 + 31, prm.N - 1), Q, nb_addr, lane) : q_lo[sl];
+                    q[sl] = slab_segs<VAR>(n0 + c0, prm.N, Q, nb_addr, lane);
 #pragma unroll
                     for (int j4 = 0; j4 < 8; j4++)
                         ld_shared_2x64(bias_addr + uint32_t(c0 + 4 * j4) * 4u, y2[sl][2 * j4], y2[sl][2 * j4 + 1]);
@@ -1170,7 +1230,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                         const int a = p * NPOL + pol;
                         const int nf = n0 + (slab0 + sl) * 32;
                         const TokenScale tk = token_scale(a, row);
-                        scale_add_unit<KIND, GENERIC, false, PT>(y2[sl], buf[u % NB], a, Q, q_lo[sl], q_hi[sl], nf, tab_addr, nb_addr, 0, &tk);
+                        scale_add_unit<KIND, VAR, false, PT>(y2[sl], buf[u % NB], a, Q, q[sl].lo, q[sl].hi, nf, tab_addr, nb_addr, 0, &tk, q[sl].lane);
                         if (GENERIC && prm.acc_dump && row < prm.M)
                             dump_unit(prm.acc_dump, buf[u % NB], a, row, nf, prm.M, prm.N);
                     }
@@ -1178,7 +1238,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                 if (ok && (!GENERIC || row < prm.M)) {
 #pragma unroll
                     for (int sl = 0; sl < kSlabsPerWarp; sl++)
-                        store_slab<GENERIC>(y2[sl], prm, row, n0 + (slab0 + sl) * 32, yo);
+                        store_slab<VAR>(y2[sl], prm, row, n0 + (slab0 + sl) * 32, yo);
                 }
             } else {
                 // ---- all accumulators of the tile resident
@@ -1295,12 +1355,12 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                                 }
                                 const TokenScale tk = token_scale(pol, row);
                                 if (pol == 0)
-                                    scale_add_unit<KIND, false, true, false>(y2, acc, 0, Q, q, q, nf, tab_addr, nb_addr,
+                                    scale_add_unit<KIND, kProduction, true, false>(y2, acc, 0, Q, q, q, nf, tab_addr, nb_addr,
                                                                              bias_addr + uint32_t(c0) * 4u, &tk);
                                 else
-                                    scale_add_unit<KIND, false, false, false>(y2, acc, pol, Q, q, q, nf, tab_addr, nb_addr, 0, &tk);
+                                    scale_add_unit<KIND, kProduction, false, false>(y2, acc, pol, Q, q, q, nf, tab_addr, nb_addr, 0, &tk);
                             }
-                            store_slab<GENERIC>(y2, prm, row, nf, yo);
+                            store_slab<VAR>(y2, prm, row, nf, yo);
                         }
                         if (from_tmem) release(cur_as);
                         continue;
@@ -1325,9 +1385,9 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                         const int c0 = h * TILE_N + (slab0 + sl) * 32, nf = n0 + c0;
                         const int q = seg_of_column(min(nf, prm.N - 1), Q, nb_addr, lane);
                         const TokenScale tk = token_scale(0, row);
-                        scale_add_unit<KIND, false, true, PT>(y2, hb[h][sl], 0, Q, q, q, nf, tab_addr, nb_addr,
+                        scale_add_unit<KIND, kProduction, true, PT>(y2, hb[h][sl], 0, Q, q, q, nf, tab_addr, nb_addr,
                                                               bias_addr + uint32_t(c0) * 4u, &tk);
-                        store_slab<GENERIC>(y2, prm, row, nf, yo);
+                        store_slab<VAR>(y2, prm, row, nf, yo);
                         if (u == 1) {
                             tc_ld32(t_h1 + 64u, hb[1][2]);
                             tc_ld32(t_h1 + 96u, hb[1][3]);
@@ -1353,13 +1413,13 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
 #pragma unroll
                     for (int sl = 0; sl < 4; sl++) {
                         const int c0 = (slab0 + sl) * 32, nf = n0 + c0;
-                        const int q = seg_of_column(nf, Q, nb_addr, lane);
+                        const SlabSegs q = slab_segs<VAR>(nf, prm.N, Q, nb_addr, lane);
                         const TokenScale tk0 = token_scale(0, row), tk1 = token_scale(1, row);
-                        scale_add_unit<KIND, false, true, PT>(y2, pb[sl], 0, Q, q, q, nf, tab_addr, nb_addr,
-                                                              bias_addr + uint32_t(c0) * 4u, &tk0);
+                        scale_add_unit<KIND, VAR, true, PT>(y2, pb[sl], 0, Q, q.lo, q.hi, nf, tab_addr, nb_addr,
+                                                            bias_addr + uint32_t(c0) * 4u, &tk0, q.lane);
                         if (sl == 0) tc_wait_ld();
-                        scale_add_unit<KIND, false, false, PT>(y2, nbuf[sl], 1, Q, q, q, nf, tab_addr, nb_addr, 0, &tk1);
-                        store_slab<GENERIC>(y2, prm, row, nf, yo);
+                        scale_add_unit<KIND, VAR, false, PT>(y2, nbuf[sl], 1, Q, q.lo, q.hi, nf, tab_addr, nb_addr, 0, &tk1, q.lane);
+                        store_slab<VAR>(y2, prm, row, nf, yo);
                         if (sl == 0) {                        // registers of slab 0 are free: the last two negative units
                             tc_ld32(t_neg + 64u, nbuf[2]);
                             tc_ld32(t_neg + 96u, nbuf[3]);
@@ -1381,7 +1441,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
 #pragma unroll
                     for (int u = 0; u < NB; u++) tc_ld32(t_warp + uint32_t((u % NPOL) * TILE_N + (u / NPOL) * 32), buf[u]);
                     uint64_t y2[16];
-                    int q_lo = 0, q_hi = 0;
+                    SlabSegs q{0, 0, 0};
 #pragma unroll
                     for (int u = 0; u < kUnits; u++) {
                         const int sl = u / NPOL, pol = u % NPOL;
@@ -1397,18 +1457,17 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                             tc_ld32(t_warp + uint32_t(((u - 1 + NB) % NPOL) * TILE_N + ((u - 1 + NB) / NPOL) * 32),
                                     buf[(u - 1) % NB]);
                         if (pol == 0) {
-                            q_lo = seg_of_column(nf, Q, nb_addr, lane);
-                            q_hi = GENERIC ? seg_of_column(min(nf + 31, prm.N - 1), Q, nb_addr, lane) : q_lo;
+                            q = slab_segs<VAR>(nf, prm.N, Q, nb_addr, lane);
                             const TokenScale tk = token_scale(pol, row);
-                            scale_add_unit<KIND, GENERIC, true, PT>(y2, buf[u % NB], pol, Q, q_lo, q_hi, nf, tab_addr, nb_addr,
-                                                                    bias_addr + uint32_t(c0) * 4u, &tk);
+                            scale_add_unit<KIND, VAR, true, PT>(y2, buf[u % NB], pol, Q, q.lo, q.hi, nf, tab_addr, nb_addr,
+                                                                bias_addr + uint32_t(c0) * 4u, &tk, q.lane);
                         } else {
                             const TokenScale tk = token_scale(pol, row);
-                            scale_add_unit<KIND, GENERIC, false, PT>(y2, buf[u % NB], pol, Q, q_lo, q_hi, nf, tab_addr, nb_addr, 0, &tk);
+                            scale_add_unit<KIND, VAR, false, PT>(y2, buf[u % NB], pol, Q, q.lo, q.hi, nf, tab_addr, nb_addr, 0, &tk, q.lane);
                         }
                         if (GENERIC && prm.acc_dump && row < prm.M)
                             dump_unit(prm.acc_dump, buf[u % NB], pol, row, nf, prm.M, prm.N);
-                        if (pol == NPOL - 1 && (!GENERIC || row < prm.M)) store_slab<GENERIC>(y2, prm, row, nf, yo);
+                        if (pol == NPOL - 1 && (!GENERIC || row < prm.M)) store_slab<VAR>(y2, prm, row, nf, yo);
                     }
                     continue;
                 }
@@ -1421,7 +1480,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                 uint32_t ra[32], rb[32];
                 int i_sl = 0, i_a = 0;              // next unit to load
                 int c_sl = 0, c_a = 0;              // next unit to consume
-                int q_lo = 0, q_hi = 0;             // N-segments of the first and last column of the slab
+                SlabSegs q{0, 0, 0};
                 auto issue = [&](uint32_t (&r)[32]) {
                     tc_ld32(t_row + uint32_t(i_a * TILE_N + (slab0 + i_sl) * 32), r);
                     if (++i_a == nacc) { i_a = 0; i_sl++; }
@@ -1430,19 +1489,18 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                     const int c0 = (slab0 + c_sl) * 32;
                     const int nf = n0 + c0;                          // first column of the slab
                     if (c_a == 0) {
-                        q_lo = seg_of_column(nf, Q, nb_addr, lane);
-                        q_hi = GENERIC ? seg_of_column(min(nf + 31, prm.N - 1), Q, nb_addr, lane) : q_lo;
+                        q = slab_segs<VAR>(nf, prm.N, Q, nb_addr, lane);
 #pragma unroll
                         for (int j4 = 0; j4 < 8; j4++)
                             ld_shared_2x64(bias_addr + uint32_t(c0 + 4 * j4) * 4u, y2[2 * j4], y2[2 * j4 + 1]);
                     }
                     const TokenScale tk = token_scale(c_a, row);
-                    scale_add_unit<KIND, GENERIC, false, PT>(y2, r, c_a, Q, q_lo, q_hi, nf, tab_addr, nb_addr, 0, &tk);
+                    scale_add_unit<KIND, VAR, false, PT>(y2, r, c_a, Q, q.lo, q.hi, nf, tab_addr, nb_addr, 0, &tk, q.lane);
                     if (GENERIC && prm.acc_dump && row < prm.M) dump_unit(prm.acc_dump, r, c_a, row, nf, prm.M, prm.N);
                     if (++c_a < nacc) return;
                     c_a = 0;
                     c_sl++;
-                    if (!GENERIC || row < prm.M) store_slab<GENERIC>(y2, prm, row, nf, yo);   // last accumulator of the slab
+                    if (!GENERIC || row < prm.M) store_slab<VAR>(y2, prm, row, nf, yo);   // last accumulator of the slab
                 };
                 if (units == 0) {
                     release(cur_as);
@@ -1514,38 +1572,38 @@ bool make_map(CUtensorMap *map, const void *base, int64_t rows, int64_t cols, in
     return r == CUDA_SUCCESS;
 }
 
-// 2-D map over the bf16 output [M, N] with row pitch ldy (elements): box = 32 columns x 32 rows, 64-byte
-// swizzle (the layout tma_store_block writes).  Needs a 16-byte aligned base and pitch.
-bool make_map_y(CUtensorMap *map, void *base, int64_t M, int64_t N, int64_t ldy)
+// 2-D map over the output [M, N] with row pitch ldy (elements): box = 32 columns x 32 rows; bf16 with 64-byte, fp32 with
+// 128-byte swizzle (the layouts tma_store_block and tma_store_block_f32 write).  Needs a 16-byte aligned base and pitch.
+bool make_map_y(CUtensorMap *map, void *base, int64_t M, int64_t N, int64_t ldy, bool f32)
 {
     EncodeFn enc = get_encode_fn();
     if (!enc) return false;
     cuuint64_t dims[2] = {cuuint64_t(N), cuuint64_t(M)};
-    cuuint64_t strides[1] = {cuuint64_t(ldy) * 2};
+    cuuint64_t strides[1] = {cuuint64_t(ldy) * (f32 ? 4 : 2)};
     cuuint32_t box[2] = {32, 32};
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    CUresult r = enc(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides,
+                     box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, f32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                     CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
 
-template <int KIND, int NPOL, int TILE_N, int CG, bool GENERIC, bool SEQ, bool WIDE = false, bool PT = false, bool SK = false>
+template <int KIND, int NPOL, int TILE_N, int CG, int VAR, bool SEQ, bool WIDE = false, bool PT = false, bool SK = false>
 sq_status prepare_variant(const GemmArgs &g, GemmLaunch &L, int device, int sm_count)
 {
     constexpr int kTileCols = TILE_N * (WIDE ? 2 : 1);
     constexpr int B_ROWS = TILE_N / CG;
     KernelParams &prm = L.prm;
-    if (GENERIC) L.ty = CUtensorMap{};                // unused by the generic variant
-    else if (!make_map_y(&L.ty, g.Y, g.M, g.N, g.ldy)) return SQ_ERR_CUDA;
+    if (VAR == kChecking) L.ty = CUtensorMap{};       // unused by the checking variant
+    else if (!make_map_y(&L.ty, g.Y, g.M, g.N, g.ldy, VAR == kFlexible && prm.y_is_f32)) return SQ_ERR_CUDA;
     if (!make_map(&L.ta, g.a_pos, g.M, g.K, g.lda, TILE_M)) return SQ_ERR_CUDA;
     if (!make_map(&L.tn, g.a_neg ? g.a_neg : g.a_pos, g.M, g.K, g.lda, TILE_M)) return SQ_ERR_CUDA;
     if (!make_map(&L.tb, g.b, g.N, g.K, g.ldb, B_ROWS)) return SQ_ERR_CUDA;
 
     const uint32_t stage_bytes = NPOL * TILE_M * BLOCK_K + (WIDE ? 2 : 1) * B_ROWS * BLOCK_K;
     // per-token mode: the tile's channel scales are staged in shared memory when there are few K-segments
-    prm.col_tab_bytes = ((GENERIC || PT) && prm.col_scale && prm.sb.P <= kMaxTokenSegments) ? uint32_t(prm.sb.P) * kTileCols * 4u : 0u;
-    const uint32_t tail = (GENERIC ? 0u : kStageBytes) + epi_table_bytes(prm.nacc, prm.sb.Q, kTileCols) + prm.col_tab_bytes +
+    prm.col_tab_bytes = ((VAR == kChecking || PT) && prm.col_scale && prm.sb.P <= kMaxTokenSegments) ? uint32_t(prm.sb.P) * kTileCols * 4u : 0u;
+    const uint32_t tail = (VAR == kChecking ? 0u : VAR == kFlexible && prm.y_is_f32 ? 2 * kStageBytes : kStageBytes) + epi_table_bytes(prm.nacc, prm.sb.Q, kTileCols) + prm.col_tab_bytes +
                           sizeof(SharedHeader);
     int stages = int((kSmemBudget - 1024 - tail) / stage_bytes);
     if (stages > kMaxStages) stages = kMaxStages;
@@ -1557,7 +1615,7 @@ sq_status prepare_variant(const GemmArgs &g, GemmLaunch &L, int device, int sm_c
     prm.num_n_tiles = int((g.N + kTileCols - 1) / kTileCols);
     const size_t smem = 1024 + size_t(stages) * stage_bytes + tail;
 
-    auto kern = segquant_gemm_kernel<KIND, NPOL, TILE_N, CG, GENERIC, SEQ, WIDE, PT, SK>;
+    auto kern = segquant_gemm_kernel<KIND, NPOL, TILE_N, CG, VAR, SEQ, WIDE, PT, SK>;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(unsigned(sm_count / CG * CG));
     cfg.blockDim = dim3(kThreads);
@@ -1602,24 +1660,28 @@ template <int KIND, int NPOL, int CG>
 sq_status prepare_tile(const GemmArgs &g, GemmLaunch &L, int tile_n, bool seq, int device, int sm_count)
 {
     KernelParams &prm = L.prm;
-    bool dbg = prm.y_is_f32 || prm.acc_dump != nullptr;
-    // the production variant writes Y with TMA stores: 16-byte aligned base and row pitch
-    dbg = dbg || reinterpret_cast<uintptr_t>(g.Y) % 16 != 0 || (size_t(g.ldy) * 2) % 16 != 0;
-    for (int q = 1; q < prm.sb.Q; q++) dbg = dbg || (prm.sb.nb[q] % 32 != 0);
+    bool dbg = prm.acc_dump != nullptr;
+    // the other variants write Y with TMA stores: 16-byte aligned base and row pitch
+    dbg = dbg || reinterpret_cast<uintptr_t>(g.Y) % 16 != 0 || (size_t(g.ldy) * (prm.y_is_f32 ? 4 : 2)) % 16 != 0;
+    // fp32 output and slabs that straddle an N-bound
+    bool flex = prm.y_is_f32;
+    for (int q = 1; q < prm.sb.Q; q++) flex = flex || (prm.sb.nb[q] % 32 != 0);
     // per-token x per-channel scales: the production variant stages a tile's channel scales in shared memory, which
     // it does for up to 32 K-segments, int8 codes and CTA pairs; anything else runs the checking variant
     const bool pt = prm.col_scale != nullptr;
-    if (pt && !(KIND == 0 && CG == 2 && prm.sb.P <= kMaxTokenSegments)) dbg = true;
+    if (pt && (flex || !(KIND == 0 && CG == 2 && prm.sb.P <= kMaxTokenSegments))) dbg = true;
     if (seq) {      // sequential K-segments
         constexpr int TN = NPOL == 1 ? 256 : 128;         // two accumulator sets fill TMEM
         const bool narrow = tile_n < TN && !dbg;          // half that width and four sets: see prepare_gemm
         prm.acc_stages = narrow ? 4 : 2;
-        if (dbg) return prepare_variant<KIND, NPOL, TN, CG, true, true>(g, L, device, sm_count);
+        if (dbg) return prepare_variant<KIND, NPOL, TN, CG, kChecking, true>(g, L, device, sm_count);
         if constexpr (KIND == 0 && CG == 2)
-            if (pt) return narrow ? prepare_variant<KIND, NPOL, TN / 2, CG, false, true, false, true>(g, L, device, sm_count)
-                                  : prepare_variant<KIND, NPOL, TN, CG, false, true, false, true>(g, L, device, sm_count);
-        return narrow ? prepare_variant<KIND, NPOL, TN / 2, CG, false, true>(g, L, device, sm_count)
-                      : prepare_variant<KIND, NPOL, TN, CG, false, true>(g, L, device, sm_count);
+            if (pt) return narrow ? prepare_variant<KIND, NPOL, TN / 2, CG, kProduction, true, false, true>(g, L, device, sm_count)
+                                  : prepare_variant<KIND, NPOL, TN, CG, kProduction, true, false, true>(g, L, device, sm_count);
+        if (flex) return narrow ? prepare_variant<KIND, NPOL, TN / 2, CG, kFlexible, true>(g, L, device, sm_count)
+                                : prepare_variant<KIND, NPOL, TN, CG, kFlexible, true>(g, L, device, sm_count);
+        return narrow ? prepare_variant<KIND, NPOL, TN / 2, CG, kProduction, true>(g, L, device, sm_count)
+                      : prepare_variant<KIND, NPOL, TN, CG, kProduction, true>(g, L, device, sm_count);
     }
     if constexpr (KIND == 0 && CG == 2) {
         if (pt && !dbg) {     // 256- and 128-column tiles only (the automatic choice never goes below for these layers)
@@ -1630,11 +1692,11 @@ sq_status prepare_tile(const GemmArgs &g, GemmLaunch &L, int tile_n, bool seq, i
                 if (tile_n == 256 && prm.sb.P == 1 && tune != 4 && (n256w % 2 == 0 || n256w >= 9) &&
                     (tune == 5 || 2 * wwide * 94 < w256 * 100)) {
                     prm.acc_stages = 1;
-                    return prepare_variant<KIND, 1, 256, 2, false, false, true, true>(g, L, device, sm_count);
+                    return prepare_variant<KIND, 1, 256, 2, kProduction, false, true, true>(g, L, device, sm_count);
                 }
             }
-            if (tile_n == 256) return prepare_variant<KIND, NPOL, 256, CG, false, false, false, true>(g, L, device, sm_count);
-            if (tile_n == 128) return prepare_variant<KIND, NPOL, 128, CG, false, false, false, true>(g, L, device, sm_count);
+            if (tile_n == 256) return prepare_variant<KIND, NPOL, 256, CG, kProduction, false, false, true>(g, L, device, sm_count);
+            if (tile_n == 128) return prepare_variant<KIND, NPOL, 128, CG, kProduction, false, false, true>(g, L, device, sm_count);
             dbg = true;
         }
     }
@@ -1646,14 +1708,14 @@ sq_status prepare_tile(const GemmArgs &g, GemmLaunch &L, int tile_n, bool seq, i
     const int64_t n256 = (g.N + 255) / 256, m_pairs = (g.M + 2 * TILE_M - 1) / (2 * TILE_M), units = sm_count / 2;
     const int64_t waves_256 = (m_pairs * n256 + units - 1) / units;
     const int64_t waves_wide = (m_pairs * ((n256 + 1) / 2) + units - 1) / units;
-    const bool wide = NPOL == 1 && CG == 2 && !dbg && tile_n == 256 && prm.sb.P == 1 && tune_seq != 4 &&
+    const bool wide = NPOL == 1 && CG == 2 && !dbg && !flex && tile_n == 256 && prm.sb.P == 1 && tune_seq != 4 &&
                       (n256 % 2 == 0 || n256 >= 9) && (tune_seq == 5 || 2 * waves_wide * 94 < waves_256 * 100);
     // Split tiles: one K-segment, CTA pairs, production output, and a tile count that leaves a good part of the
     // last wave idle.  Time in K-blocks of 256 accumulator columns: whole tiles take waves x K-blocks; split
     // tiles take their even share plus the exchange of partial sums (a fixed part and one slot read per pair
     // that shares a tile, in K-block times; measured).  segment_mode 6 forces the split where it is possible, 7 forbids it.
     if constexpr (CG == 2) {
-        if (!dbg && !pt && prm.sb.P == 1 && g.sk_scratch && tune_seq != 7) {
+        if (!dbg && !flex && !pt && prm.sb.P == 1 && g.sk_scratch && tune_seq != 7) {
             constexpr int TN = sk_tile_n(NPOL);
             constexpr double kSkFixup = 30.0, kSkPerSharer = 10.0;
             const int64_t pairs = sm_count / 2, m_tiles = (g.M + 2 * TILE_M - 1) / (2 * TILE_M);
@@ -1667,23 +1729,27 @@ sq_status prepare_tile(const GemmArgs &g, GemmLaunch &L, int tile_n, bool seq, i
             const size_t need = sk_counter_bytes(tiles_sk) + size_t(pairs) * 4 * kSkSlotBytes;
             if (g.sk_bytes >= need && tiles_sk * kblocks >= 2 && (tune_seq == 6 || t_sk < 0.9 * t_dp)) {
                 prm.acc_stages = 2;
-                return prepare_variant<KIND, NPOL, TN, 2, false, false, false, false, true>(g, L, device, sm_count);
+                return prepare_variant<KIND, NPOL, TN, 2, kProduction, false, false, false, true>(g, L, device, sm_count);
             }
         }
     }
     if (wide) {
         prm.acc_stages = 1;
-        return prepare_variant<KIND, 1, 256, 2, false, false, true>(g, L, device, sm_count);
+        return prepare_variant<KIND, 1, 256, 2, kProduction, false, true>(g, L, device, sm_count);
     }
+    if (flex && !dbg && tile_n >= 128)      // (narrower tiles are only ever asked for by tests: checking variant)
+        return tile_n == 256 ? prepare_variant<KIND, NPOL, 256, CG, kFlexible, false>(g, L, device, sm_count)
+                             : prepare_variant<KIND, NPOL, 128, CG, kFlexible, false>(g, L, device, sm_count);
+    dbg = dbg || flex;
     switch (tile_n) {
-        case 256: return dbg ? prepare_variant<KIND, NPOL, 256, CG, true, false>(g, L, device, sm_count)
-                             : prepare_variant<KIND, NPOL, 256, CG, false, false>(g, L, device, sm_count);
-        case 128: return dbg ? prepare_variant<KIND, NPOL, 128, CG, true, false>(g, L, device, sm_count)
-                             : prepare_variant<KIND, NPOL, 128, CG, false, false>(g, L, device, sm_count);
-        case 64: return dbg ? prepare_variant<KIND, NPOL, 64, CG, true, false>(g, L, device, sm_count)
-                            : prepare_variant<KIND, NPOL, 64, CG, false, false>(g, L, device, sm_count);
-        case 32: return dbg ? prepare_variant<KIND, NPOL, 32, CG, true, false>(g, L, device, sm_count)
-                            : prepare_variant<KIND, NPOL, 32, CG, false, false>(g, L, device, sm_count);
+        case 256: return dbg ? prepare_variant<KIND, NPOL, 256, CG, kChecking, false>(g, L, device, sm_count)
+                             : prepare_variant<KIND, NPOL, 256, CG, kProduction, false>(g, L, device, sm_count);
+        case 128: return dbg ? prepare_variant<KIND, NPOL, 128, CG, kChecking, false>(g, L, device, sm_count)
+                             : prepare_variant<KIND, NPOL, 128, CG, kProduction, false>(g, L, device, sm_count);
+        case 64: return dbg ? prepare_variant<KIND, NPOL, 64, CG, kChecking, false>(g, L, device, sm_count)
+                            : prepare_variant<KIND, NPOL, 64, CG, kProduction, false>(g, L, device, sm_count);
+        case 32: return dbg ? prepare_variant<KIND, NPOL, 32, CG, kChecking, false>(g, L, device, sm_count)
+                            : prepare_variant<KIND, NPOL, 32, CG, kProduction, false>(g, L, device, sm_count);
     }
     return SQ_ERR_UNSUPPORTED;
 }

@@ -548,3 +548,33 @@ def test_segments_inside_a_k_block_on_both_tile_widths(kb, code, dual, M):
             assert torch.equal(Y, ref), tile_n
     finally:
         B.segquant_set_tuning()
+
+
+# ------------------------------------------------------------------ fp32 output and N-bounds inside a slab
+
+@pytest.mark.parametrize("y_dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("code,dual", [("int8", True), ("int8", False), ("e4m3", True), ("e4m3", False)])
+@pytest.mark.parametrize("case", [
+    # M, K, N, kb, nb: one and several K-segments, both CTA groups, 256- and 128-column tiles, bounds one column apart
+    # from a slab's edge and from each other, several bounds in one slab, a last slab and a last tile that are not whole
+    (5, 256, 328, [0, 256], [0, 1, 2, 31, 33, 328]),
+    (130, 400, 1000, [0, 160, 400], [0, 328, 664, 1000]),
+    (300, 128, 72, [0, 128], [0, 40, 72]),
+    (700, 256, 2056, [0, 256], [0, 1000, 2049, 2056]),
+    (2100, 192, 4104, [0, 64, 192], [0, 4103, 4104]),
+])
+def test_flexible_outputs_equal_the_checking_variant(case, code, dual, y_dtype):
+    """fp32 output and slabs that straddle N-bounds through the TMA-storing variant: bit for bit the checking variant's
+    output (same terms, same order), and nothing written beyond column N."""
+    M, K, N, kb, nb = case
+    spec = custom_spec("flex", M, K, N, kb, nb, dual, code, x_kind="normal+gelu" if dual else "normal", seed=72)
+    data = WL.make_layer(spec)
+    layer = SegQuantLinear(data.W, data.bias, kb, nb, dual, code, DEV)
+    layer.calibrate(data.X_cal)
+    X = data.X.to(DEV)
+    ref, _, _, _ = layer.forward_steps(X, y_dtype=y_dtype, dump_acc=True)
+    Yw = torch.full((M, N + 8), 7.0, dtype=y_dtype, device=DEV)
+    layer.forward(X, Yw[:, :N])
+    layer.check_status()
+    assert torch.equal(Yw[:, :N], ref)
+    assert bool(torch.all(Yw[:, N:] == 7.0))
