@@ -68,7 +68,7 @@ static_assert(kFrontThreads * kFrontRegs + kEpiThreads * kEpiRegs <= kThreads * 
 static_assert(kFrontRegs % 8 == 0 && kEpiRegs % 8 == 0 && kFrontRegs >= 24 && kEpiRegs <= 256, "setmaxnreg operand");
 [[maybe_unused]] constexpr int kEpiBufRegs = 192;      // of kEpiRegs: accumulator load buffers plus running sums (SEQ)
 [[maybe_unused]] constexpr int kResidentBufs = 4;      // accumulator load buffers of the resident epilogue
-[[maybe_unused]] constexpr int kMaxStages = 8;
+[[maybe_unused]] constexpr int kMaxStages = 32;
 constexpr int kTmemCols = 512;
 [[maybe_unused]] constexpr int kMaxAccSets = 4;        // accumulator sets in TMEM (narrow SEQ tiles; otherwise 1 or 2)
 [[maybe_unused]] constexpr uint32_t kSmemBudget = 227 * 1024;
@@ -810,16 +810,21 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     constexpr bool GENERIC = VAR == kChecking;
-    // layout: [ring: stages x (NPOL A tiles of 16 KiB, B part of B_ROWS*128 B)] [output staging] [scales] [header]
+    // layout: [ring: stages x (B part of B_ROWS*128 B, NPOL A tiles of a_rows*128 B)] [output staging] [scales] [header]
+    // a_rows is 128 for CTA pairs.  One CTA on M <= 128 rows loads only the rows there are (rounded up to 8): the MMA still
+    // reads 128 rows from the tile's address, whatever lies behind the loaded ones (the next tiles; the ring is followed
+    // by at least 16 KiB), but what it makes of them ends up in accumulator rows that nobody stores.  A ring stage of a
+    // small layer thus holds little but weights, and there are more stages: these launches stream the weights once and
+    // are bound by the bytes in flight: 8 x 3072 -> 18432 dual e4m3 20.8 -> 13.5 us (weights at copy bandwidth: 8.5).
     constexpr int B_ROWS = TILE_N / CG;                  // weight rows this CTA loads per K-block
-    constexpr uint32_t a_bytes = TILE_M * BLOCK_K;
+    const uint32_t a_bytes = CG == 2 ? uint32_t(TILE_M * BLOCK_K) : uint32_t(prm.a_rows * BLOCK_K);
     constexpr uint32_t b_bytes = B_ROWS * BLOCK_K;
     constexpr int kHalves = WIDE ? 2 : 1;                // weight tiles per stage
     constexpr int kTileCols = TILE_N * kHalves;          // output columns of a tile
     constexpr int kIssuers = (NPOL == 2 || WIDE) ? 2 : 1;
     static_assert(!WIDE || (NPOL == 1 && TILE_N == 256 && CG == 2 && VAR == kProduction && !SEQ), "wide single-scale tile");
     static_assert(!SK || (CG == 2 && VAR == kProduction && !SEQ && !WIDE && !PT && NPOL * TILE_N == 256), "split tiles");
-    constexpr uint32_t stage_bytes = NPOL * a_bytes + kHalves * b_bytes;
+    const uint32_t stage_bytes = NPOL * a_bytes + kHalves * b_bytes;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *sh_stage = smem + size_t(prm.stages) * stage_bytes;      // 1 KiB aligned: stages are multiples of 1 KiB
     float *sh_bias = reinterpret_cast<float *>(sh_stage + (GENERIC ? 0 : VAR == kFlexible && prm.y_is_f32 ? 2 * kStageBytes : kStageBytes));     // [TILE_N], per tile
@@ -843,20 +848,21 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_b)) : "memory");
         if (!GENERIC) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_y)) : "memory");
     }
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < prm.stages; s++) {
-            mbar_init(smem_u32(&hdr->full[s]), 1);
-            mbar_init(smem_u32(&hdr->empty[s]), kIssuers);      // one arrival per MMA-issuing thread
+    if (warp == 0) {                     // lane s initialises the barriers of ring slot s and accumulator set s
+        static_assert(kMaxStages <= 32 && kMaxAccSets <= 32, "one lane each");
+        if (lane < prm.stages) {
+            mbar_init(smem_u32(&hdr->full[lane]), 1);
+            mbar_init(smem_u32(&hdr->empty[lane]), kIssuers);   // one arrival per MMA-issuing thread
         }
-        for (int s = 0; s < kMaxAccSets; s++) {
-            mbar_init(smem_u32(&hdr->tmem_full[s]), kIssuers);
-            mbar_init(smem_u32(&hdr->tmem_empty[s]), CG * kEpiWarps);
+        if (lane < kMaxAccSets) {
+            mbar_init(smem_u32(&hdr->tmem_full[lane]), kIssuers);
+            mbar_init(smem_u32(&hdr->tmem_empty[lane]), CG * kEpiWarps);
         }
-        hdr->abort_flag = 0;
+        if (lane == 0) hdr->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    // Every thread arrives at the cluster barrier now (thread 0 after its barrier initialisation) and waits for it
+    // Every thread arrives at the cluster barrier now (warp 0 after its barrier initialisation) and waits for it
     // only after the TMEM allocation below, so the barrier's latency overlaps the allocation.
     __syncwarp();
     if (CG == 2) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
@@ -915,9 +921,9 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                         const uint32_t bar = full0_sig + 8 * s;
                         if (elect_one()) {
                             if (rank == 0) mbar_expect_tx(full0 + 8 * s, CG * stage_bytes);
-                            tma_load_2d<CG>(dst, &tm_a_pos, bar, kbi * BLOCK_K, m0);
-                            if (NPOL == 2) tma_load_2d<CG>(dst + a_bytes, &tm_a_neg, bar, kbi * BLOCK_K, m0);
-                            tma_load_2d<CG>(dst + NPOL * a_bytes, &tm_b, bar, kbi * BLOCK_K, n0);
+                            tma_load_2d<CG>(dst + b_bytes, &tm_a_pos, bar, kbi * BLOCK_K, m0);
+                            if (NPOL == 2) tma_load_2d<CG>(dst + b_bytes + a_bytes, &tm_a_neg, bar, kbi * BLOCK_K, m0);
+                            tma_load_2d<CG>(dst, &tm_b, bar, kbi * BLOCK_K, n0);
                         }
                         __syncwarp();
                         issued++;
@@ -937,10 +943,10 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                     const uint32_t bar = full0_sig + 8 * s;
                     if (elect_one()) {
                         if (rank == 0) mbar_expect_tx(full0 + 8 * s, CG * stage_bytes);
-                        tma_load_2d<CG>(dst, &tm_a_pos, bar, k, m0);
-                        if (NPOL == 2) tma_load_2d<CG>(dst + a_bytes, &tm_a_neg, bar, k, m0);
-                        tma_load_2d<CG>(dst + NPOL * a_bytes, &tm_b, bar, k, n0);
-                        if (WIDE) tma_load_2d<CG>(dst + NPOL * a_bytes + b_bytes, &tm_b, bar, k, n0 + TILE_N);
+                        tma_load_2d<CG>(dst + kHalves * b_bytes, &tm_a_pos, bar, k, m0);
+                        if (NPOL == 2) tma_load_2d<CG>(dst + kHalves * b_bytes + a_bytes, &tm_a_neg, bar, k, m0);
+                        tma_load_2d<CG>(dst, &tm_b, bar, k, n0);
+                        if (WIDE) tma_load_2d<CG>(dst + b_bytes, &tm_b, bar, k, n0 + TILE_N);
                     }
                     __syncwarp();
                     issued++;
@@ -972,11 +978,12 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
             constexpr uint32_t idesc = make_idesc(KIND, TILE_N, TILE_M * CG);
             const uint32_t stages = prm.stages, P = prm.sb.P, acc_stages = prm.acc_stages;
             const uint32_t full0 = smem_u32(&hdr->full[0]), empty0 = smem_u32(&hdr->empty[0]);
-            // dual: thread `pol` takes activation tile `pol`; wide: thread `pol` takes weight tile (half) `pol`
-            const uint64_t desc0 = make_smem_desc(smem_u32(smem)) + (WIDE ? 0u : pol) * (uint64_t(a_bytes) >> 4);
-            constexpr uint64_t kStageDesc = uint64_t(stage_bytes) >> 4;
-            const uint64_t b_off = WIDE ? (uint64_t(a_bytes) >> 4) + pol * (uint64_t(b_bytes) >> 4)
-                                        : (uint64_t(NPOL * a_bytes) >> 4) - pol * (uint64_t(a_bytes) >> 4);
+            // dual: warp `pol` takes activation tile `pol`; wide: warp `pol` takes weight tile (half) `pol`
+            const uint64_t desc0 = make_smem_desc(smem_u32(smem) + kHalves * b_bytes + (WIDE ? 0u : pol) * a_bytes);
+            const uint64_t kStageDesc = uint64_t(stage_bytes) >> 4;
+            // from this warp's activation tile to its weight tile, modulo 2^32 in the descriptor's low word
+            const uint32_t b_off = (WIDE ? pol * b_bytes : 0u) / 16u - (kHalves * b_bytes + (WIDE ? 0u : pol) * a_bytes) / 16u;
+            auto b_desc = [&](uint64_t da) { return (da & ~0xFFFFFFFFull) | uint32_t(uint32_t(da) + b_off); };
             uint32_t s = 0, ph = 0, as = 0, aph = 0;
             bool ok = true;
             if constexpr (SK) {
@@ -1000,7 +1007,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                         const int rem = prm.K - kbi * BLOCK_K;
                         const int nk = rem >= BLOCK_K ? BLOCK_K / MMA_K : (rem + MMA_K - 1) / MMA_K;
                         if (elect_one()) {
-                            issue_kblock<KIND, 1, TILE_N, CG>(d0, da, da + b_off, idesc, nk, accumulate);
+                            issue_kblock<KIND, 1, TILE_N, CG>(d0, da, b_desc(da), idesc, nk, accumulate);
                             tc_commit<CG>(empty0 + 8 * s);
                         }
                         accumulate = 1;
@@ -1039,7 +1046,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                         if (k % BLOCK_K != 0) {                    // the block is in the ring: the segment before had its first part
                             const int k_stop = min(k_end, (k + BLOCK_K) / BLOCK_K * BLOCK_K);
                             const uint64_t da = desc0 + s * kStageDesc + uint64_t((k % BLOCK_K) >> 4);
-                            if (elect_one()) issue_kblock<KIND, 1, TILE_N, CG>(d0, da, da + b_off, idesc, (k_stop - k + MMA_K - 1) / MMA_K, 0u);
+                            if (elect_one()) issue_kblock<KIND, 1, TILE_N, CG>(d0, da, b_desc(da), idesc, (k_stop - k + MMA_K - 1) / MMA_K, 0u);
                             accumulate = 1;
                             k = k_stop;
                             if (k % BLOCK_K == 0 || k == prm.K) {
@@ -1059,7 +1066,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                         const int rem = k_end - k;
                         const int nk = rem >= BLOCK_K ? BLOCK_K / MMA_K : (rem + MMA_K - 1) / MMA_K;
                         if (elect_one()) {
-                            issue_kblock<KIND, 1, TILE_N, CG>(d0, da, da + b_off, idesc, nk, accumulate);
+                            issue_kblock<KIND, 1, TILE_N, CG>(d0, da, b_desc(da), idesc, nk, accumulate);
                             tc_commit<CG>(empty0 + 8 * s);         // the slot is free when both threads' MMAs have retired
                         }
                         accumulate = 1;
@@ -1071,7 +1078,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                         } else {
                             tc_fence_after();
                             const uint64_t da = desc0 + s * kStageDesc;
-                            if (elect_one()) issue_kblock<KIND, 1, TILE_N, CG>(d0, da, da + b_off, idesc, (k_end - k) / MMA_K, accumulate);
+                            if (elect_one()) issue_kblock<KIND, 1, TILE_N, CG>(d0, da, b_desc(da), idesc, (k_end - k) / MMA_K, accumulate);
                         }
                     }
                     if (SEQ) {
@@ -1596,15 +1603,17 @@ sq_status prepare_variant(const GemmArgs &g, GemmLaunch &L, int device, int sm_c
     KernelParams &prm = L.prm;
     if (VAR == kChecking) L.ty = CUtensorMap{};       // unused by the checking variant
     else if (!make_map_y(&L.ty, g.Y, g.M, g.N, g.ldy, VAR == kFlexible && prm.y_is_f32)) return SQ_ERR_CUDA;
-    if (!make_map(&L.ta, g.a_pos, g.M, g.K, g.lda, TILE_M)) return SQ_ERR_CUDA;
-    if (!make_map(&L.tn, g.a_neg ? g.a_neg : g.a_pos, g.M, g.K, g.lda, TILE_M)) return SQ_ERR_CUDA;
+    prm.a_rows = CG == 1 && g.M < TILE_M ? int((g.M + 7) / 8 * 8) : TILE_M;
+    if (!make_map(&L.ta, g.a_pos, g.M, g.K, g.lda, prm.a_rows)) return SQ_ERR_CUDA;
+    if (!make_map(&L.tn, g.a_neg ? g.a_neg : g.a_pos, g.M, g.K, g.lda, prm.a_rows)) return SQ_ERR_CUDA;
     if (!make_map(&L.tb, g.b, g.N, g.K, g.ldb, B_ROWS)) return SQ_ERR_CUDA;
 
-    const uint32_t stage_bytes = NPOL * TILE_M * BLOCK_K + (WIDE ? 2 : 1) * B_ROWS * BLOCK_K;
+    const uint32_t stage_bytes = NPOL * prm.a_rows * BLOCK_K + (WIDE ? 2 : 1) * B_ROWS * BLOCK_K;
     // per-token mode: the tile's channel scales are staged in shared memory when there are few K-segments
     prm.col_tab_bytes = ((VAR == kChecking || PT) && prm.col_scale && prm.sb.P <= kMaxTokenSegments) ? uint32_t(prm.sb.P) * kTileCols * 4u : 0u;
-    const uint32_t tail = (VAR == kChecking ? 0u : VAR == kFlexible && prm.y_is_f32 ? 2 * kStageBytes : kStageBytes) + epi_table_bytes(prm.nacc, prm.sb.Q, kTileCols) + prm.col_tab_bytes +
+    uint32_t tail = (VAR == kChecking ? 0u : VAR == kFlexible && prm.y_is_f32 ? 2 * kStageBytes : kStageBytes) + epi_table_bytes(prm.nacc, prm.sb.Q, kTileCols) + prm.col_tab_bytes +
                           sizeof(SharedHeader);
+    if (prm.a_rows < TILE_M && tail < TILE_M * BLOCK_K) tail = TILE_M * BLOCK_K;     // what the MMAs read behind the ring
     int stages = int((kSmemBudget - 1024 - tail) / stage_bytes);
     if (stages > kMaxStages) stages = kMaxStages;
     const int tune_stages = g_tune_stages.load(std::memory_order_relaxed);
@@ -1737,7 +1746,9 @@ sq_status prepare_tile(const GemmArgs &g, GemmLaunch &L, int tile_n, bool seq, i
         prm.acc_stages = 1;
         return prepare_variant<KIND, 1, 256, 2, kProduction, false, true>(g, L, device, sm_count);
     }
-    if (flex && !dbg && tile_n >= 128)      // (narrower tiles are only ever asked for by tests: checking variant)
+    if constexpr (CG == 1)
+        if (flex && !dbg && tile_n == 64) return prepare_variant<KIND, NPOL, 64, CG, kFlexible, false>(g, L, device, sm_count);
+    if (flex && !dbg && tile_n >= 128)      // (the other narrow tiles are only ever asked for by tests: checking variant)
         return tile_n == 256 ? prepare_variant<KIND, NPOL, 256, CG, kFlexible, false>(g, L, device, sm_count)
                              : prepare_variant<KIND, NPOL, 128, CG, kFlexible, false>(g, L, device, sm_count);
     dbg = dbg || flex;
@@ -1908,6 +1919,13 @@ sq_status prepare_gemm(const GemmArgs &g, GemmLaunch *out)
     // only at its end: keep two sets so that it overlaps the next tile's main loop
     const bool pt_generic = g.col_scale && (prm.y_is_f32 || prm.acc_dump || g.code != SQ_CODE_INT8 || cg != 2 || g.sb.P > kMaxTokenSegments);
     if (pt_generic && 2 * tile_n * prm.nacc > kTmemCols && tile_n >= 64) tile_n >>= 1;
+    // One CTA per tile (M <= 128): the launch streams the weights, so the more SMs share in it the better; 64-column
+    // tiles as long as they cost no further wave.  (us, 64 / 128 columns: 8 x 1152 -> 6912 dual, 108 / 54 tiles, 5.3 / 6.0;
+    // 8 x 3072 -> 18432 dual, 288 / 144 tiles for 148 SMs, 15.4 / 13.5.)
+    if (cg == 1 && g.M <= TILE_M && g.sb.P == 1) {
+        auto waves = [&](int tn) { return (((g.N + tn - 1) / tn) + sm_count - 1) / sm_count; };
+        if (waves(64) <= waves(128)) tile_n = 64;
+    }
     if (tune_tile_n >= 32 && tune_tile_n <= tile_max && (tune_tile_n & (tune_tile_n - 1)) == 0)
         tile_n = tune_tile_n;
     prm.acc_stages = (2 * tile_n * prm.nacc <= kTmemCols) ? 2 : 1;

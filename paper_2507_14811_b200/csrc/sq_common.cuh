@@ -130,8 +130,9 @@ struct GemmArgs {
 struct KernelParams {
     int M, N, K;
     int nacc;          // P * npol
-    int acc_stages;    // 1 or 2 accumulator sets in TMEM
+    int acc_stages;    // accumulator sets in TMEM
     int stages;        // shared-memory ring depth
+    int a_rows;        // activation rows a CTA loads per K-block (128; fewer for one CTA on M < 128)
     int num_m_tiles, num_n_tiles;
     SegBounds sb;
     const float *s_pos, *s_neg, *s_w, *bias;

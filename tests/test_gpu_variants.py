@@ -578,3 +578,27 @@ def test_flexible_outputs_equal_the_checking_variant(case, code, dual, y_dtype):
     layer.check_status()
     assert torch.equal(Yw[:, :N], ref)
     assert bool(torch.all(Yw[:, N:] == 7.0))
+
+
+# ------------------------------------------------------------------ few rows: ring stages that hold only the rows there are
+
+@pytest.mark.parametrize("M", [1, 7, 8, 9, 64, 121, 127, 128])
+@pytest.mark.parametrize("code,dual", [("int8", True), ("int8", False), ("e4m3", True), ("e4m3", False)])
+@pytest.mark.parametrize("K,N,kb", [(16, 8, [0, 16]), (4112, 200, [0, 4112]), (1200, 9480, [0, 1200]), (416, 328, [0, 96, 416])])
+def test_few_rows_equal_the_same_rows_of_a_larger_input(M, K, N, kb, code, dual):
+    """Up to 128 rows run on one CTA per tile whose ring stages hold 8 to 128 activation rows; the MMA reads past them, so
+    rows that are not there must not reach any output.  Bit for bit the rows of a 300-row input (CTA pairs, full tiles), on
+    K tails, one stage's worth of K, more K-blocks than stages, 64- and 128-column tiles, and in the checking variant."""
+    nb = [0, N]
+    spec = custom_spec("few_rows", 300, K, N, kb, nb, dual, code, x_kind="normal+gelu" if dual else "normal", seed=73)
+    data = WL.make_layer(spec)
+    layer = SegQuantLinear(data.W, data.bias, kb, nb, dual, code, DEV)
+    layer.calibrate(data.X_cal)
+    X = data.X.to(DEV)
+    full = layer.forward(X)
+    Yw = torch.full((M + 2, N), 7.0, dtype=torch.bfloat16, device=DEV)
+    layer.forward(X[:M], Yw[:M])
+    checked, _, _, _ = layer.forward_steps(X[:M], dump_acc=True)
+    layer.check_status()
+    assert torch.equal(Yw[:M], full[:M]) and torch.equal(checked, full[:M])
+    assert bool(torch.all(Yw[M:] == 7.0))
