@@ -1,4 +1,5 @@
-"""Thin ctypes binding over libsegquant.so: argument marshalling only.
+"""Thin binding over libsegquant.so: argument marshalling only.  The calls that a layer makes at run time go through the
+native module built from csrc/torch_calls.cpp, the offline ones through ctypes.
 
 Function names mirror the C ABI (include/segquant.h).  Tensors are torch CUDA tensors used as
 device memory; every step of the path runs inside the library's kernels.  There is no fallback:
@@ -66,6 +67,19 @@ def lib():
     return _lib
 
 
+_calls_module = None
+
+
+def _calls():
+    """The native module with the run-time calls; like the library, it has to be there."""
+    global _calls_module
+    if _calls_module is None:
+        lib()
+        from . import _calls as module
+        _calls_module = module
+    return _calls_module
+
+
 class SegTable:
     """Host-side segment table: kb[0..P], nb[0..Q]."""
 
@@ -74,6 +88,7 @@ class SegTable:
         self.nb = np.ascontiguousarray(nb, np.int32)
         self._c = _SegTable(len(self.kb) - 1, self.kb.ctypes.data_as(C.POINTER(C.c_int32)),
                             len(self.nb) - 1, self.nb.ctypes.data_as(C.POINTER(C.c_int32)))
+        self.address = C.addressof(self._c)
 
     @property
     def P(self):
@@ -183,9 +198,7 @@ def segquant_quantize_act(X: torch.Tensor, seg: SegTable, s_pos, s_neg, code: st
         c_pos = new_codes(M, K, X.device)
     if s_neg is not None and c_neg is None:
         c_neg = new_codes(M, K, X.device)
-    st = lib().segquant_quantize_act(_ptr(X), C.c_int(_dt(X)), C.c_int64(M), C.c_int64(K), C.c_int64(X.stride(0)),
-                                     seg.ref(), _ptr(s_pos), _ptr(s_neg), C.c_int(SQ_CODE[code]), C.c_uint32(flags),
-                                     _ptr(c_pos), _ptr(c_neg), C.c_int64(c_pos.stride(0)), _stream())
+    st = _calls().quantize_act(X, seg.address, s_pos, s_neg, SQ_CODE[code], flags, c_pos, c_neg)
     _check(st, "segquant_quantize_act")
     return c_pos, (c_neg if s_neg is not None else None)
 
@@ -204,10 +217,7 @@ def segquant_quantize_act_fused(H: torch.Tensor, seg: SegTable, s_pos, s_neg, co
         c_pos = new_codes(M, K, H.device)
     if s_neg is not None and c_neg is None:
         c_neg = new_codes(M, K, H.device)
-    st = lib().segquant_quantize_act_fused(_ptr(H), C.c_int(_dt(H)), C.c_int64(M), C.c_int64(K), C.c_int64(H.stride(0)),
-                                           seg.ref(), _ptr(s_pos), _ptr(s_neg), C.c_int(SQ_CODE[code]), C.c_uint32(flags),
-                                           C.c_int(SQ_ACT[act]), _ptr(mult), _ptr(c_pos), _ptr(c_neg),
-                                           C.c_int64(c_pos.stride(0)), _stream())
+    st = _calls().quantize_act_fused(H, seg.address, s_pos, s_neg, SQ_CODE[code], flags, SQ_ACT[act], mult, c_pos, c_neg)
     _check(st, "segquant_quantize_act_fused")
     return c_pos, (c_neg if s_neg is not None else None)
 
@@ -255,6 +265,9 @@ def segquant_quantize_weight(W: torch.Tensor, seg: SegTable, s_w, code: str, fla
     return Wq
 
 
+_SEGLINEAR, _DUALSCALE, _W4A8 = 0, 1, 2        # GEMM entry points of the native module
+
+
 def _new_y(M, N, y_dtype, device):
     return torch.empty((M, N), dtype=y_dtype, device=device)
 
@@ -270,11 +283,7 @@ def segquant_seglinear_gemm(Xq, Wq, seg: SegTable, code: str, s_x, s_w, bias, wo
     if Y is None:
         Y = _new_y(M, N, y_dtype, Xq.device)
     dump = _new_dump(seg.P, M, N, code, Xq.device) if dump_acc else None
-    st = lib().segquant_seglinear_gemm(_ptr(Xq), C.c_int64(Xq.stride(0)), _ptr(Wq), C.c_int64(Wq.stride(0)),
-                                       C.c_int64(M), C.c_int64(N), C.c_int64(K), seg.ref(), C.c_int(SQ_CODE[code]),
-                                       _ptr(s_x), _ptr(s_w), _ptr(bias), _ptr(Y), C.c_int(_dt(Y)),
-                                       C.c_int64(Y.stride(0)), _ptr(dump), _ptr(workspace),
-                                       C.c_size_t(workspace.numel()), _stream())
+    st = _calls().gemm(Xq, None, Wq, seg.address, SQ_CODE[code], s_x, None, s_w, bias, Y, dump, workspace, _SEGLINEAR)
     _check(st, "segquant_seglinear_gemm")
     return (Y, dump) if dump_acc else Y
 
@@ -287,11 +296,7 @@ def segquant_dualscale_gemm(Xq_pos, Xq_neg, Wq, seg: SegTable, code: str, s_pos,
     if Y is None:
         Y = _new_y(M, N, y_dtype, Xq_pos.device)
     dump = _new_dump(seg.P * 2, M, N, code, Xq_pos.device) if dump_acc else None
-    st = lib().segquant_dualscale_gemm(_ptr(Xq_pos), _ptr(Xq_neg), C.c_int64(Xq_pos.stride(0)), _ptr(Wq),
-                                       C.c_int64(Wq.stride(0)), C.c_int64(M), C.c_int64(N), C.c_int64(K), seg.ref(),
-                                       C.c_int(SQ_CODE[code]), _ptr(s_pos), _ptr(s_neg), _ptr(s_w), _ptr(bias),
-                                       _ptr(Y), C.c_int(_dt(Y)), C.c_int64(Y.stride(0)), _ptr(dump), _ptr(workspace),
-                                       C.c_size_t(workspace.numel()), _stream())
+    st = _calls().gemm(Xq_pos, Xq_neg, Wq, seg.address, SQ_CODE[code], s_pos, s_neg, s_w, bias, Y, dump, workspace, _DUALSCALE)
     _check(st, "segquant_dualscale_gemm")
     return (Y, dump) if dump_acc else Y
 
@@ -304,15 +309,8 @@ def segquant_layer_forward(X, Wq, seg: SegTable, code: str, s_pos, s_neg, s_w, b
                            x_stage=None, y_stage=None, flags: int = 0):
     """Quantize -> GEMM -> epilogue in one call.  X / Y may be (pinned) host tensors, in which case
     x_stage / y_stage are device buffers of the same shape and the copies are part of the call."""
-    M, K = X.shape
-    N = Wq.shape[0]
-    x_host, y_host = not X.is_cuda, not Y.is_cuda
-    st = lib().segquant_layer_forward(
-        _ptr(X), C.c_int(int(x_host)), _ptr(x_stage), C.c_int(_dt(X)), C.c_int64(M), C.c_int64(K),
-        C.c_int64(X.stride(0)), _ptr(Wq), C.c_int64(Wq.stride(0)), C.c_int64(N), seg.ref(), C.c_int(SQ_CODE[code]),
-        _ptr(s_pos), _ptr(s_neg), _ptr(s_w), _ptr(bias), C.c_uint32(flags), _ptr(Y), C.c_int(int(y_host)),
-        _ptr(y_stage), C.c_int(_dt(Y)), C.c_int64(Y.stride(0)), _ptr(scratch), C.c_size_t(scratch.numel()),
-        _ptr(workspace), C.c_size_t(workspace.numel()), _stream())
+    st = _calls().layer_forward(X, Wq, seg.address, SQ_CODE[code], s_pos, s_neg, s_w, bias, Y, scratch, workspace, x_stage,
+                                y_stage, flags)
     _check(st, "segquant_layer_forward")
     return Y
 
@@ -335,14 +333,7 @@ def segquant_layer_forward_pipelined(X, Wq, seg: SegTable, code: str, s_pos, s_n
 
 def segquant_quantize_per_row(X: torch.Tensor, seg: SegTable, dual: bool, bits: int = 8, flags: int = 0):
     """Per-row scales [rows, P] (per token, or per output channel for bits = 4) and the int8 codes made with them."""
-    rows, K = X.shape
-    s_pos = torch.empty((rows, seg.P), dtype=torch.float32, device=X.device)
-    s_neg = torch.empty((rows, seg.P), dtype=torch.float32, device=X.device) if dual else None
-    c_pos = new_codes(rows, K, X.device)
-    c_neg = new_codes(rows, K, X.device) if dual else None
-    st = lib().segquant_quantize_per_row(_ptr(X), C.c_int(_dt(X)), C.c_int64(rows), C.c_int64(K), C.c_int64(X.stride(0)),
-                                         seg.ref(), C.c_int(bits), C.c_uint32(flags), _ptr(s_pos), _ptr(s_neg), _ptr(c_pos),
-                                         _ptr(c_neg), C.c_int64(c_pos.stride(0)), _stream())
+    st, s_pos, s_neg, c_pos, c_neg = _calls().quantize_per_row(X, seg.address, seg.P, dual, bits, flags)
     _check(st, "segquant_quantize_per_row")
     return s_pos, s_neg, c_pos, c_neg
 
@@ -360,8 +351,7 @@ def segquant_unpack_w4(Wq4: torch.Tensor, out=None):
     N, K2 = Wq4.shape
     if out is None:
         out = new_codes(N, 2 * K2, Wq4.device)
-    st = lib().segquant_unpack_w4(_ptr(Wq4), C.c_int64(Wq4.stride(0)), C.c_int64(N), C.c_int64(2 * K2), _ptr(out),
-                                  C.c_int64(out.stride(0)), _stream())
+    st = _calls().unpack_w4(Wq4, out)
     _check(st, "segquant_unpack_w4")
     return out
 
@@ -374,11 +364,7 @@ def segquant_w4a8_gemm(Xq_pos, Xq_neg, Wq8, seg: SegTable, s_pos, s_neg, s_w, bi
     if Y is None:
         Y = _new_y(M, N, y_dtype, Xq_pos.device)
     dump = _new_dump(seg.P * (2 if dual else 1), M, N, "int8", Xq_pos.device) if dump_acc else None
-    st = lib().segquant_w4a8_gemm(_ptr(Xq_pos), _ptr(Xq_neg), C.c_int64(Xq_pos.stride(0)), _ptr(Wq8),
-                                  C.c_int64(Wq8.stride(0)), C.c_int64(M), C.c_int64(N), C.c_int64(K), seg.ref(),
-                                  _ptr(s_pos), _ptr(s_neg), _ptr(s_w), _ptr(bias), _ptr(Y), C.c_int(_dt(Y)),
-                                  C.c_int64(Y.stride(0)), _ptr(dump), _ptr(workspace), C.c_size_t(workspace.numel()),
-                                  _stream())
+    st = _calls().gemm(Xq_pos, Xq_neg, Wq8, seg.address, SQ_CODE["int8"], s_pos, s_neg, s_w, bias, Y, dump, workspace, _W4A8)
     _check(st, "segquant_w4a8_gemm")
     return (Y, dump) if dump_acc else Y
 
@@ -400,11 +386,11 @@ class LayerPlan:
             _ptr(bias), C.c_uint32(flags), _ptr(Y), C.c_int(_dt(Y)), C.c_int64(Y.stride(0)), _ptr(scratch),
             C.c_size_t(scratch.numel()), _ptr(workspace), C.c_size_t(workspace.numel()))
         _check(st, "segquant_plan_layer")
-        self._run = lib().segquant_plan_run
-        self._ref = C.byref(self._buf)
+        self._run = _calls().plan_run
+        self._address = C.addressof(self._buf)
 
     def run(self):
-        st = self._run(self._ref, _stream())
+        st = self._run(self._address)
         if st != SQ_OK:
             _check(st, "segquant_plan_run")
 

@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import os
+import shutil
 import subprocess
 import sys
 from concurrent.futures import ThreadPoolExecutor
@@ -15,14 +16,15 @@ OBJ_DIR = os.path.join(_HERE, "_build")
 UNITS = [(f, f.replace(".cu", ".o"), []) for f in ("api.cu", "calib.cu", "quantize.cu", "zero_point.cu", "gemm_tcgen05.cu")]
 UNITS += [("gemm_tcgen05.cu", f"gemm_kind{k}_npol{n}.o", [f"-DSQ_GEMM_KIND={k}", f"-DSQ_GEMM_NPOL={n}"])
           for k in (0, 1) for n in (1, 2)]
+CALLS_PATH = os.path.join(_HERE, "_calls.so")          # native module over the library, for torch tensors
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC"]
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(CALLS_PATH):
         return True
-    t = os.path.getmtime(LIB_PATH)
+    t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(CALLS_PATH))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(INCLUDE, "segquant.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -44,7 +46,23 @@ def build(force: bool = False, verbose: bool = False) -> str:
         objs = list(pool.map(compile_one, UNITS))
     subprocess.check_call([nvcc, "-shared", "-cudart", "static", "-gencode", "arch=compute_100a,code=sm_100a",
                            "-o", LIB_PATH, *objs])
+    build_calls(nvcc)
     return LIB_PATH
+
+
+def build_calls(nvcc: str) -> None:
+    """Compiles csrc/torch_calls.cpp against torch's headers and links it to the library beside it."""
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(shutil.which(nvcc) or "/usr/local/cuda/bin/nvcc"))), "include")
+    include = [*cpp_extension.include_paths(), sysconfig.get_paths()["include"], cuda]
+    subprocess.check_call([
+        os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+        f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *[f for d in include for f in ("-isystem", d)],
+        "-I", INCLUDE, os.path.join(CSRC, "torch_calls.cpp"), "-o", CALLS_PATH, "-L", _HERE, "-l:libsegquant.so",
+        *[f for d in cpp_extension.library_paths() for f in ("-L", d)], "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+        "-Wl,-rpath,$ORIGIN"])
 
 
 if __name__ == "__main__":

@@ -139,3 +139,20 @@ def test_plan_calls_reject_on_the_host(L):
     # a failed build leaves a plan that does not run
     assert L.segquant_plan_run(C.byref(plan), None) == 5
     assert seg.P == 1 and B.SQ_PLAN_BYTES == 4096
+
+
+@pytest.mark.parametrize("call,args,error", [
+    ("plan_run", (), TypeError),                                            # wrong number of arguments
+    ("plan_run", ("x",), TypeError),                                        # not an address
+    ("unpack_w4", (1, 2), TypeError),                                       # not tensors
+    ("unpack_w4", ("vector", "matrix"), ValueError),                        # not a matrix
+    ("quantize_per_row", ("half", 0, 1, False, 8, 0), TypeError),           # a dtype the library does not take
+    ("quantize_per_row", ("matrix", None, 1, False, 8, 0), TypeError),      # no segment table
+])
+def test_native_calls_turn_bad_arguments_into_exceptions(L, call, args, error):
+    import torch
+    named = {"vector": torch.zeros(8, dtype=torch.uint8), "matrix": torch.zeros(4, 8), "half": torch.zeros(4, 8, dtype=torch.float16)}
+    if call == "plan_run":
+        named = {}
+    with pytest.raises(error):
+        getattr(B._calls(), call)(*[named.get(a, a) if isinstance(a, str) else a for a in args])
