@@ -705,6 +705,9 @@ quantize_table_kernel(const __grid_constant__ QuantParams prm)
 // its extrema per K-segment are reduced in shared memory, the scales (one IEEE division each) are written out,
 // and the codes are made from the registers with the same quantizer as everywhere else.
 constexpr int kRowChunks = 4;                       // K <= 256 threads x 4 chunks x 16 = 16384
+// CHUNKS: chunks a thread may hold.  One where a block covers the row with one per thread (K <= 4096): fewer registers, more
+// rows in flight (us, 4 / 1 chunks: 921 x 1920 dual with 12 segments 8.1 / 4.4, 8858 x 1536 with 24 16.4 / 13.9, 8858 x 3072
+// with 2 21.6 / 20.1).  Two up to K = 8192 were no better on many rows (8858 x 6144 42.8 / 44.5).
 
 __device__ __forceinline__ uint32_t ord_enc(float f)     // monotone map float -> uint32
 {
@@ -740,7 +743,7 @@ __device__ __forceinline__ void chunk_extrema(const Raw16<__nv_bfloat16> &r, flo
     mn = fminf(__low2float(lo), __high2float(lo));
 }
 
-template <typename Tin, bool DUAL>
+template <typename Tin, bool DUAL, int CHUNKS>
 __global__ void __launch_bounds__(kThreads)
 quantize_per_row_kernel(const Tin *__restrict__ X, int K, int64_t ld, const SegBounds sb, float q_max, float q_min_abs,
                         float *__restrict__ s_pos, float *__restrict__ s_neg, uint8_t *__restrict__ c_pos,
@@ -763,10 +766,10 @@ quantize_per_row_kernel(const Tin *__restrict__ X, int K, int64_t ld, const SegB
         __syncthreads();
     }
     const Tin *src = X + row * ld;
-    Raw16<Tin> raw[kRowChunks];
-    int seg[kRowChunks];                            // K-segment of a whole chunk, -1: straddles a bound or the row end
+    Raw16<Tin> raw[CHUNKS];
+    int seg[CHUNKS];                            // K-segment of a whole chunk, -1: straddles a bound or the row end
 #pragma unroll
-    for (int c = 0; c < kRowChunks; c++) {
+    for (int c = 0; c < CHUNKS; c++) {
         const int k0 = (int(threadIdx.x) + c * int(blockDim.x)) * kVec;
         seg[c] = -2;                                // beyond the row
         if (k0 >= K) continue;
@@ -794,7 +797,7 @@ quantize_per_row_kernel(const Tin *__restrict__ X, int K, int64_t ld, const SegB
     if (one) {
         float mx = tail_mx, mn = tail_mn;
 #pragma unroll
-        for (int c = 0; c < kRowChunks; c++) {
+        for (int c = 0; c < CHUNKS; c++) {
             if (seg[c] >= 0) {
                 float cx, cm;
                 chunk_extrema(raw[c], cx, cm);
@@ -826,7 +829,7 @@ quantize_per_row_kernel(const Tin *__restrict__ X, int K, int64_t ld, const SegB
     // reduced with shuffles and one lane updates the shared words; same-address shared atomics from every thread
     // serialise, and were most of this kernel's time.  Every lane takes part in the votes and shuffles.
 #pragma unroll
-    for (int c = 0; c < kRowChunks; c++) {
+    for (int c = 0; c < CHUNKS; c++) {
         float mx = -INFINITY, mn = INFINITY;
         if (seg[c] >= 0) chunk_extrema(raw[c], mx, mn);
         const int s0 = __shfl_sync(0xFFFFFFFFu, seg[c], 0);
@@ -870,7 +873,7 @@ quantize_per_row_kernel(const Tin *__restrict__ X, int K, int64_t ld, const SegB
     SegConst cp, cn;
     int const_seg = -1;
 #pragma unroll
-    for (int c = 0; c < kRowChunks; c++) {
+    for (int c = 0; c < CHUNKS; c++) {
         const int k0 = (int(threadIdx.x) + c * int(blockDim.x)) * kVec;
         if (seg[c] == -2) continue;
         uint8_t *dp = c_pos + row * ldc + k0;
@@ -1100,6 +1103,15 @@ sq_status launch_quantize(const void *X, sq_dtype dt, int64_t M, int64_t K, int6
     return s == SQ_OK ? run_quantize(L, st) : s;
 }
 
+template <typename Tin, bool DUAL, typename... Args>
+static cudaError_t launch_per_row(cudaLaunchConfig_t &cfg, int64_t V, Args... args)
+{
+    const int64_t chunks = V <= kThreads ? 1 : kRowChunks;
+    cfg.blockDim = dim3(unsigned(((V + chunks - 1) / chunks + 31) / 32 * 32));
+    return chunks == 1 ? cudaLaunchKernelEx(&cfg, quantize_per_row_kernel<Tin, DUAL, 1>, args...)
+                       : cudaLaunchKernelEx(&cfg, quantize_per_row_kernel<Tin, DUAL, kRowChunks>, args...);
+}
+
 sq_status launch_quantize_per_row(const void *X, sq_dtype dt, int64_t M, int64_t K, int64_t ld, const SegBounds &sb,
                                   int dual, float q_max, float q_min_abs, float *s_pos, float *s_neg,
                                   void *c_pos, void *c_neg, int64_t ldc, cudaStream_t st)
@@ -1107,12 +1119,8 @@ sq_status launch_quantize_per_row(const void *X, sq_dtype dt, int64_t M, int64_t
     const int64_t V = (K + kVec - 1) / kVec;
     if (V > int64_t(kThreads) * kRowChunks) return SQ_ERR_UNSUPPORTED;      // the row is held in registers
     if (M > 0x7FFFFFFF) return SQ_ERR_SHAPE;
-    int threads = int((V + kRowChunks - 1) / kRowChunks);
-    threads = (threads + 31) / 32 * 32;
-    if (threads < 32) threads = 32;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(unsigned(M));
-    cfg.blockDim = dim3(unsigned(threads));
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1124,12 +1132,12 @@ sq_status launch_quantize_per_row(const void *X, sq_dtype dt, int64_t M, int64_t
     cudaError_t e;
     if (dt == SQ_F32) {
         const float *x = static_cast<const float *>(X);
-        e = dual ? cudaLaunchKernelEx(&cfg, quantize_per_row_kernel<float, true>, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc)
-                 : cudaLaunchKernelEx(&cfg, quantize_per_row_kernel<float, false>, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc);
+        e = dual ? launch_per_row<float, true>(cfg, V, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc)
+                 : launch_per_row<float, false>(cfg, V, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc);
     } else {
         const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(X);
-        e = dual ? cudaLaunchKernelEx(&cfg, quantize_per_row_kernel<__nv_bfloat16, true>, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc)
-                 : cudaLaunchKernelEx(&cfg, quantize_per_row_kernel<__nv_bfloat16, false>, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc);
+        e = dual ? launch_per_row<__nv_bfloat16, true>(cfg, V, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc)
+                 : launch_per_row<__nv_bfloat16, false>(cfg, V, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc);
     }
     count_launch();
     if (e != cudaSuccess) { note_cuda_error(e); return SQ_ERR_CUDA; }

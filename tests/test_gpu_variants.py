@@ -602,3 +602,26 @@ def test_few_rows_equal_the_same_rows_of_a_larger_input(M, K, N, kb, code, dual)
     layer.check_status()
     assert torch.equal(Yw[:M], full[:M]) and torch.equal(checked, full[:M])
     assert bool(torch.all(Yw[M:] == 7.0))
+
+
+# ------------------------------------------------------------------ per-row scales: one or several chunks per thread
+
+@pytest.mark.parametrize("x_dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("dual", [True, False])
+@pytest.mark.parametrize("K,kb", [
+    (16, [0, 16]), (24, [0, 8, 24]), (4080, [0, 4080]), (4088, [0, 1000, 4088]), (4096, [0, 64, 4096]),
+    (4104, [0, 4104]), (4112, [0, 2048, 4112]), (16384, [0, 16384]),
+])
+def test_per_row_scales_and_codes_are_exact(K, kb, dual, x_dtype):
+    """Rows one block holds with one 16-element chunk per thread (K <= 4096) and with four, at the edge between them, with
+    row tails and bounds inside a chunk: scales and codes bit-exact against the oracle."""
+    rs = np.random.default_rng(12)
+    X = torch.from_numpy((rs.standard_normal((37, K)) * np.exp(2 * rs.standard_normal((37, 1)))).astype(np.float32)).to(x_dtype)
+    X[3] = 0.0
+    r_sp, r_sn, r_pos, r_neg = O.quantize_per_row(X.float().numpy(), kb, dual)
+    Xd = torch.full((37, (K + 15) // 16 * 16), 1e6, dtype=x_dtype, device=DEV)
+    Xd[:, :K] = X.to(DEV)
+    g_sp, g_sn, c_pos, c_neg = B.segquant_quantize_per_row(Xd[:, :K], B.SegTable(kb, [0, 8]), dual)
+    assert np.array_equal(g_sp.cpu().numpy(), r_sp) and np.array_equal(c_pos.cpu().numpy().view(np.int8), r_pos)
+    if dual:
+        assert np.array_equal(g_sn.cpu().numpy(), r_sn) and np.array_equal(c_neg.cpu().numpy().view(np.int8), r_neg)
