@@ -2,8 +2,11 @@
 // current stream here costs a fraction of what it costs in Python (an eager 256 x 256 -> 768 layer call: 17.9 us with
 // ctypes objects, 8.5 us from here; the three calls of a 2048 x 4608 -> 1152 W4A8 layer: 50.6 -> 32.8 us).  Argument
 // marshalling only: every check is the C ABI's (include/segquant.h), every function returns its status (with the tensors
-// it allocated, where it did), and the GIL is released around the call.
+// it allocated, where it did), and the GIL is released around the call.  Reading a tensor can throw (a wrapper or sparse
+// tensor without storage, a stride of a 0-dimensional one), so everything is read into locals while the GIL is held; what
+// runs without it is a call of the C ABI, which does not throw.
 #include <Python.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
@@ -63,14 +66,26 @@ sq_dtype dtype_of(const at::Tensor &t)
 
 void *current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
+struct GilRelease {
+    PyThreadState *state = PyEval_SaveThread();
+    ~GilRelease() { PyEval_RestoreThread(state); }
+};
+
 template <typename F>
 sq_status without_gil(F f)
 {
-    PyThreadState *state = PyEval_SaveThread();
-    const sq_status s = f();
-    PyEval_RestoreThread(state);
-    return s;
+    const GilRelease released;
+    return f();
 }
+
+// What the C ABI takes of a tensor with rows: read while the GIL is held.
+struct Rows {
+    void *p;
+    int64_t rows, cols, ld;           // cols: of the last dimension
+    bool on_host;
+    explicit Rows(const at::Tensor &t)
+        : p(t.data_ptr()), rows(t.size(0)), cols(t.size(-1)), ld(t.stride(0)), on_host(!t.is_cuda()) {}
+};
 
 template <typename F>
 PyObject *guarded(const char *name, Py_ssize_t n, Py_ssize_t want, F f)
@@ -83,8 +98,8 @@ PyObject *guarded(const char *name, Py_ssize_t n, Py_ssize_t want, F f)
         return f();
     } catch (const BadArgument &) {
         return nullptr;
-    } catch (const std::exception &e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (...) {                  // torch's own errors, as torch's Python methods raise them
+        torch::translate_exception_to_python(std::current_exception());
         return nullptr;
     }
 }
@@ -100,8 +115,8 @@ PyObject *layer_forward(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     return guarded("layer_forward", n, 14, [&] {
         const Args a{args};
-        const at::Tensor &X = a.matrix(0), &W = a.tensor(1), &Y = a.tensor(8);
-        const sq_dtype dx = dtype_of(X), dy = dtype_of(Y);
+        const sq_dtype dx = dtype_of(a.matrix(0)), dy = dtype_of(a.tensor(8));
+        const Rows X(a.matrix(0)), W(a.tensor(1)), Y(a.tensor(8));
         const sq_segtable *seg = a.seg(2);
         const sq_code code = sq_code(a.integer(3));
         const float *sp = a.f32(4), *sn = a.f32(5), *sw = a.f32(6), *bias = a.f32(7);
@@ -109,9 +124,8 @@ PyObject *layer_forward(PyObject *, PyObject *const *args, Py_ssize_t n)
         void *scratch = a.ptr(9), *ws = a.ptr(10), *xs = a.ptr(11), *ys = a.ptr(12), *stream = current_stream();
         const size_t scratch_bytes = a.bytes(9), ws_bytes = a.bytes(10);
         return PyLong_FromLong(without_gil([&] {
-            return segquant_layer_forward(X.data_ptr(), !X.is_cuda(), xs, dx, X.size(0), X.size(1), X.stride(0), W.data_ptr(),
-                                          W.stride(0), W.size(0), seg, code, sp, sn, sw, bias, flags, Y.data_ptr(),
-                                          !Y.is_cuda(), ys, dy, Y.stride(0), scratch, scratch_bytes, ws, ws_bytes, stream);
+            return segquant_layer_forward(X.p, X.on_host, xs, dx, X.rows, X.cols, X.ld, W.p, W.ld, W.rows, seg, code, sp, sn, sw,
+                                          bias, flags, Y.p, Y.on_host, ys, dy, Y.ld, scratch, scratch_bytes, ws, ws_bytes, stream);
         }));
     });
 }
@@ -121,16 +135,15 @@ PyObject *quantize_act(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     return guarded("quantize_act", n, 8, [&] {
         const Args a{args};
-        const at::Tensor &X = a.matrix(0), &C = a.tensor(6);
-        const sq_dtype dx = dtype_of(X);
+        const sq_dtype dx = dtype_of(a.matrix(0));
+        const Rows X(a.matrix(0)), C(a.tensor(6));
         const sq_segtable *seg = a.seg(1);
         const float *sp = a.f32(2), *sn = a.f32(3);
         const sq_code code = sq_code(a.integer(4));
         const uint32_t flags = uint32_t(a.integer(5));
         void *cn = a.ptr(7), *stream = current_stream();
         return PyLong_FromLong(without_gil([&] {
-            return segquant_quantize_act(X.data_ptr(), dx, X.size(0), X.size(1), X.stride(0), seg, sp, sn, code, flags,
-                                         C.data_ptr(), cn, C.stride(0), stream);
+            return segquant_quantize_act(X.p, dx, X.rows, X.cols, X.ld, seg, sp, sn, code, flags, C.p, cn, C.ld, stream);
         }));
     });
 }
@@ -140,18 +153,17 @@ PyObject *quantize_act_fused(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     return guarded("quantize_act_fused", n, 10, [&] {
         const Args a{args};
-        const at::Tensor &H = a.matrix(0), &C = a.tensor(8);
-        const sq_dtype dh = dtype_of(H);
+        const sq_dtype dh = dtype_of(a.matrix(0));
+        const Rows H(a.matrix(0)), C(a.tensor(8));
         const sq_segtable *seg = a.seg(1);
         const float *sp = a.f32(2), *sn = a.f32(3), *mult = a.f32(7);
         const sq_code code = sq_code(a.integer(4));
         const uint32_t flags = uint32_t(a.integer(5));
         const sq_act act = sq_act(a.integer(6));
-        const int64_t K = act == SQ_ACT_GEGLU ? H.size(1) / 2 : H.size(1);
+        const int64_t K = act == SQ_ACT_GEGLU ? H.cols / 2 : H.cols;
         void *cn = a.ptr(9), *stream = current_stream();
         return PyLong_FromLong(without_gil([&] {
-            return segquant_quantize_act_fused(H.data_ptr(), dh, H.size(0), K, H.stride(0), seg, sp, sn, code, flags, act, mult,
-                                               C.data_ptr(), cn, C.stride(0), stream);
+            return segquant_quantize_act_fused(H.p, dh, H.rows, K, H.ld, seg, sp, sn, code, flags, act, mult, C.p, cn, C.ld, stream);
         }));
     });
 }
@@ -162,24 +174,24 @@ PyObject *gemm(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     return guarded("gemm", n, 13, [&] {
         const Args a{args};
-        const at::Tensor &X = a.matrix(0), &W = a.tensor(2), &Y = a.tensor(9);
-        const sq_dtype dy = dtype_of(Y);
+        const sq_dtype dy = dtype_of(a.tensor(9));
+        const Rows X(a.matrix(0)), W(a.tensor(2)), Y(a.tensor(9));
         const sq_segtable *seg = a.seg(3);
         const sq_code code = sq_code(a.integer(4));
         const float *sp = a.f32(5), *sn = a.f32(6), *sw = a.f32(7), *bias = a.f32(8);
         void *xn = a.ptr(1), *dump = a.ptr(10), *ws = a.ptr(11), *stream = current_stream();
         const size_t ws_bytes = a.bytes(11);
         const int kind = int(a.integer(12));
-        const int64_t M = X.size(0), K = X.size(1), N = W.size(0);
+        const int64_t M = X.rows, K = X.cols, N = W.rows;
         return PyLong_FromLong(without_gil([&] {
             if (kind == kW4a8)
-                return segquant_w4a8_gemm(X.data_ptr(), xn, X.stride(0), W.data_ptr(), W.stride(0), M, N, K, seg, sp, sn, sw, bias,
-                                          Y.data_ptr(), dy, Y.stride(0), dump, ws, ws_bytes, stream);
+                return segquant_w4a8_gemm(X.p, xn, X.ld, W.p, W.ld, M, N, K, seg, sp, sn, sw, bias, Y.p, dy, Y.ld, dump, ws, ws_bytes,
+                                          stream);
             if (kind == kDualscale)
-                return segquant_dualscale_gemm(X.data_ptr(), xn, X.stride(0), W.data_ptr(), W.stride(0), M, N, K, seg, code, sp, sn,
-                                               sw, bias, Y.data_ptr(), dy, Y.stride(0), dump, ws, ws_bytes, stream);
-            return segquant_seglinear_gemm(X.data_ptr(), X.stride(0), W.data_ptr(), W.stride(0), M, N, K, seg, code, sp, sw, bias,
-                                           Y.data_ptr(), dy, Y.stride(0), dump, ws, ws_bytes, stream);
+                return segquant_dualscale_gemm(X.p, xn, X.ld, W.p, W.ld, M, N, K, seg, code, sp, sn, sw, bias, Y.p, dy, Y.ld, dump, ws,
+                                               ws_bytes, stream);
+            return segquant_seglinear_gemm(X.p, X.ld, W.p, W.ld, M, N, K, seg, code, sp, sw, bias, Y.p, dy, Y.ld, dump, ws, ws_bytes,
+                                           stream);
         }));
     });
 }
@@ -189,24 +201,26 @@ PyObject *quantize_per_row(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     return guarded("quantize_per_row", n, 6, [&]() -> PyObject * {
         const Args a{args};
-        const at::Tensor &X = a.matrix(0);
-        const int64_t rows = X.size(0), K = X.size(1), P = a.integer(2);
-        const sq_dtype dx = dtype_of(X);
+        const at::Tensor &x = a.matrix(0);
+        const sq_dtype dx = dtype_of(x);
+        const Rows X(x);
+        const int64_t P = a.integer(2);
         const sq_segtable *seg = a.seg(1);
         const bool dual = a.truth(3);
         const int bits = int(a.integer(4));
         const uint32_t flags = uint32_t(a.integer(5));
-        const auto scales = X.options().dtype(at::kFloat);
-        at::Tensor sp = at::empty({rows, P}, scales), sn, cp = new_codes(rows, K, X), cn;
+        const auto scales = x.options().dtype(at::kFloat);
+        at::Tensor sp = at::empty({X.rows, P}, scales), sn, cp = new_codes(X.rows, X.cols, x), cn;
         if (dual) {
-            sn = at::empty({rows, P}, scales);
-            cn = new_codes(rows, K, X);
+            sn = at::empty({X.rows, P}, scales);
+            cn = new_codes(X.rows, X.cols, x);
         }
+        float *s_pos = sp.data_ptr<float>(), *s_neg = dual ? sn.data_ptr<float>() : nullptr;
+        const Rows C(cp);
+        void *c_neg = dual ? cn.data_ptr() : nullptr;
         void *stream = current_stream();
         const sq_status st = without_gil([&] {
-            return segquant_quantize_per_row(X.data_ptr(), dx, rows, K, X.stride(0), seg, bits, flags, sp.data_ptr<float>(),
-                                             dual ? sn.data_ptr<float>() : nullptr, cp.data_ptr(), dual ? cn.data_ptr() : nullptr,
-                                             cp.stride(0), stream);
+            return segquant_quantize_per_row(X.p, dx, X.rows, X.cols, X.ld, seg, bits, flags, s_pos, s_neg, C.p, c_neg, C.ld, stream);
         });
         return Py_BuildValue("(iNNNN)", int(st), THPVariable_Wrap(sp), THPVariable_Wrap(sn), THPVariable_Wrap(cp), THPVariable_Wrap(cn));
     });
@@ -217,10 +231,10 @@ PyObject *unpack_w4(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     return guarded("unpack_w4", n, 2, [&] {
         const Args a{args};
-        const at::Tensor &W4 = a.matrix(0), &W8 = a.tensor(1);
+        const Rows W4(a.matrix(0)), W8(a.tensor(1));
         void *stream = current_stream();
         return PyLong_FromLong(without_gil([&] {
-            return segquant_unpack_w4(W4.data_ptr(), W4.stride(0), W4.size(0), 2 * W4.size(1), W8.data_ptr(), W8.stride(0), stream);
+            return segquant_unpack_w4(W4.p, W4.ld, W4.rows, 2 * W4.cols, W8.p, W8.ld, stream);
         }));
     });
 }

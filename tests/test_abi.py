@@ -156,3 +156,57 @@ def test_native_calls_turn_bad_arguments_into_exceptions(L, call, args, error):
         named = {}
     with pytest.raises(error):
         getattr(B._calls(), call)(*[named.get(a, a) if isinstance(a, str) else a for a in args])
+
+
+def _gemm_args(X, W, Y, seg):
+    import torch
+    s = torch.ones(1)
+    return X, None, W, seg.address, 0, s, None, s, None, Y, None, torch.zeros(B.workspace_bytes(), dtype=torch.uint8), 0
+
+
+def _layer_args(X, W, Y, seg):
+    import torch
+    s, buf = torch.ones(1), torch.zeros(B.workspace_bytes(), dtype=torch.uint8)
+    return X, W, seg.address, 0, s, None, s, None, Y, buf, buf, None, None, 0
+
+
+@pytest.mark.parametrize("call,bad,error,text", [
+    # (function, what takes the place of a tensor, exception, part of its message)
+    ("gemm", {"Y": "scalar"}, IndexError, "dimension"),
+    ("gemm", {"W": "scalar"}, IndexError, "dimension"),
+    ("gemm", {"X": "sparse"}, RuntimeError, "storage"),
+    ("layer_forward", {"Y": "scalar"}, IndexError, "dimension"),
+    ("layer_forward", {"X": "sparse"}, RuntimeError, "storage"),
+    ("layer_forward", {"X": "vmap"}, RuntimeError, "storage"),
+    ("quantize_act", {"Y": "scalar"}, IndexError, "dimension"),
+    ("quantize_act", {"X": "vmap"}, RuntimeError, "storage"),
+    ("quantize_act_fused", {"Y": "scalar"}, IndexError, "dimension"),
+    ("quantize_act_fused", {"X": "sparse"}, RuntimeError, "storage"),
+    ("quantize_per_row", {"X": "sparse"}, RuntimeError, "storage"),
+    ("quantize_per_row", {"X": "vmap"}, RuntimeError, "storage"),
+    ("unpack_w4", {"X": "sparse"}, RuntimeError, "storage"),
+])
+def test_native_calls_read_tensors_before_they_release_the_gil(L, call, bad, error, text):
+    # a tensor that cannot be read (no rows, no storage) raises what reading it in Python raises; nothing is left to be
+    # read, and to throw, when the GIL has been released
+    import torch
+    seg = B.SegTable([0, 64], [0, 32])
+    s = torch.ones(1)
+
+    def invoke(X):
+        t = {"X": X, "W": torch.zeros(32, 64, dtype=torch.uint8), "Y": torch.zeros(4, 64)}
+        t.update({k: torch.tensor(0.0) for k, v in bad.items() if v == "scalar"})
+        args = {"gemm": lambda: _gemm_args(t["X"], t["W"], t["Y"], seg),
+                "layer_forward": lambda: _layer_args(t["X"], t["W"], t["Y"], seg),
+                "quantize_act": lambda: (t["X"], seg.address, s, None, 0, 0, t["Y"], None),
+                "quantize_act_fused": lambda: (t["X"], seg.address, s, None, 0, 0, 1, None, t["Y"], None),
+                "quantize_per_row": lambda: (t["X"], seg.address, 1, True, 8, 0),
+                "unpack_w4": lambda: (t["X"], t["W"])}[call]()
+        return getattr(B._calls(), call)(*args)
+
+    X = torch.zeros(4, 64)
+    with pytest.raises(error, match=f"(?i){text}"):
+        if bad.get("X") == "vmap":
+            torch.func.vmap(invoke)(torch.zeros(2, 4, 64))
+        else:
+            invoke(X.to_sparse() if bad.get("X") == "sparse" else X)
