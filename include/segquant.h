@@ -149,8 +149,9 @@ sq_status segquant_quantize_act(const void *X, sq_dtype dt, int64_t M, int64_t K
  *   have stored it in), then x = a * mult[k] as one fp32 multiply (mult dev [K] fp32, or NULL), then the codes
  *   of segquant_quantize_act for x.  The activation never goes through device memory.
  *   Accuracy of the activation: evaluated in fp32 with relative error <= (|h| + 8) 2^-23 (SiLU) and
- *   (3 h^2 + 48) 2^-24 (GELU; a result below 2^-100 in magnitude may be zero); where the exact value lies that close to a rounding boundary of dt the stored
- *   value, and with it the code, may be that of the neighbouring dt value.  With SQ_ACT_NONE the codes are exact.
+ *   (3 h^2 + 48) 2^-24 (GELU), plus 2^-143 absolute where the exponential is subnormal (SiLU below h = -87, GELU below
+ *   -13); where the exact value lies that close to a rounding boundary of dt the stored value, and with it the code,
+ *   may be that of the neighbouring dt value.  With SQ_ACT_NONE the codes are exact.
  *   SQ_ACT_GEGLU (gated GELU; App. B names it without a form): H is [M, 2K] with ld >= 2K, value half in columns
  *   [0, K), gate half in [K, 2K), a[k] = H[k] * GELU(H[K + k]) with relative error <= (3 g^2 + 49) 2^-24, g the
  *   gate; K, mult, the segment table and the codes refer to the K outputs.  The gate half must start on a 16-byte

@@ -148,13 +148,14 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
 // first order, so that the rounding of the square, which the exponential would amplify by t^2, does not count.
 // What remains is the hardware exponential's own error (|s| 2^-24 from the product with log2 e, one unit in the
 // last place from the approximation), the fast division's 2 units and a dozen roundings: relative error
-// <= (3 h^2 + 48) 2^-24; in |h| <= 4 it stays below 2^-20.
+// <= (3 h^2 + 48) 2^-24; in |h| <= 4 it stays below 2^-19.  The exponential keeps subnormal results (a GELU of h < -13.2
+// under a small scale, or times a large gated value, is an ordinary number; 2 us of the 8192 x 2560 gated pass).
 // Both are written for TWO elements: the multiplies, FMAs and adds go two per instruction (packed fp32 pairs), each of
 // them rounding exactly as the scalar instruction does, which is what bounds the fused pass (the ALUs, not memory).
 // (8192 x 2560 gated GELU, dual int8, 126 MB: 49.4 us one element at a time with the gate half one row ahead in registers,
 // 35.0 us with pairs and the gate half in the ring; without the table, 54 M elements of GELU 93 -> 72 us.)
 // GELU without branches: with a = min(|h|, 20), v = max(h, 0) - (a / 2) E in one FMA is h - (h / 2) E for h >= 0 and
-// (h / 2) E below; at a = 20 the exponential has long underflowed to zero, so v is h or 0 beyond it and t^2 stays
+// (h / 2) E below; at a = 20 the exponential has long underflowed to zero, so v is h or +0 beyond it and t^2 stays
 // finite for every h.
 __device__ __forceinline__ float rcp_approx(float x)
 {
@@ -162,10 +163,10 @@ __device__ __forceinline__ float rcp_approx(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ float ex2_approx_ftz(float x)
+__device__ __forceinline__ float ex2_approx(float x)         // keeps subnormal results
 {
     float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    asm("ex2.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 __device__ __forceinline__ uint64_t dup2(float v) { return pack2(v, v); }
@@ -197,7 +198,7 @@ __device__ __forceinline__ uint64_t gelu2(float h0, float h1)
     const uint64_t neg_e = fma2(mul2(t, dup2(-1.0f)), t, s);      // t^2 = s - neg_e exactly
     float x0, x1;
     unpack2(mul2(s, dup2(-1.4426950408889634f)), x0, x1);
-    uint64_t E = mul2(pack2(ex2_approx_ftz(x0), ex2_approx_ftz(x1)), g);
+    uint64_t E = mul2(pack2(ex2_approx(x0), ex2_approx(x1)), g);
     E = fma2(E, neg_e, E);                                        // exp(-(s + e)) = exp(-s) (1 - e) to first order
     return fma2(mul2(a, dup2(-0.5f)), E, pack2(fmaxf(h0, 0.0f), fmaxf(h1, 0.0f)));
 }

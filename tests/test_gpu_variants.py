@@ -3,6 +3,7 @@ the act-to-linear prologue (activation function and per-channel multiplier in fr
 against the CPU oracle on the same seeded inputs, through the C ABI."""
 import numpy as np
 import pytest
+import scipy.special
 import torch
 
 import oracle as O
@@ -625,3 +626,38 @@ def test_per_row_scales_and_codes_are_exact(K, kb, dual, x_dtype):
     assert np.array_equal(g_sp.cpu().numpy(), r_sp) and np.array_equal(c_pos.cpu().numpy().view(np.int8), r_pos)
     if dual:
         assert np.array_equal(g_sn.cpu().numpy(), r_sn) and np.array_equal(c_neg.cpu().numpy().view(np.int8), r_neg)
+
+
+@pytest.mark.parametrize("act,dtype,table", [("geglu", "bf16", 0), ("geglu", "f32", 0), ("gelu", "f32", 0), ("gelu", "bf16", 2),
+                                             ("gelu", "bf16", 1), ("silu", "f32", 0)])
+def test_fused_activation_keeps_results_whose_exponential_is_subnormal(act, dtype, table):
+    """GELU below -13.2 and SiLU below -87.3 need an exponential below fp32's smallest normal number.  A large value half, or
+    a large per-channel multiplier, brings the product back to ordinary magnitudes, so a flush to zero shows in the codes."""
+    x = np.linspace(-101.0, -87.5, 17) if act == "silu" else np.arange(-14.25, -13.2, 0.0625)     # exact in bf16
+    x = x.astype(np.float32)
+    K, big = 32, 2.0 ** 120
+    h = np.zeros((2, K), np.float32)
+    h[:, :x.size] = x
+    exact = (h.astype(np.float64) * scipy.special.ndtr(h.astype(np.float64)) if act != "silu"
+             else h.astype(np.float64) / (1.0 + np.exp(-h.astype(np.float64))))
+    stored_step = 2.0 ** -8 if dtype == "bf16" else 2.0 ** -23      # of a normal stored value, relative
+    tol = np.abs(exact) * (3 * 14.25 ** 2 + 49 if act != "silu" else 2 * (101 + 8)) * 2.0 ** -24 + 2.0 ** -143   # the header's bound
+    if act == "geglu":                                              # stored is the product, a normal number
+        H, mult = np.concatenate([np.full_like(h, big), h], axis=1), None
+        tol = tol + np.abs(exact) * stored_step / 2
+    else:                                                           # stored is the activation itself, subnormal
+        H, mult = h, torch.full((K,), big, device=DEV)
+        tol = tol + (2.0 ** -133 if dtype == "bf16" else 2.0 ** -149) / 2 + np.abs(exact) * stored_step / 2
+    s = np.float32(np.abs(exact).max() * big / 128.0)
+    st = torch.tensor([s], device=DEV)
+    Hd = torch.from_numpy(H).to(torch.bfloat16 if dtype == "bf16" else torch.float32).to(DEV)
+    B.segquant_set_quantize_tuning(table)
+    try:
+        c_pos, c_neg = B.segquant_quantize_act_fused(Hd, B.SegTable([0, K], [0, 8]), st, st, "int8", act=act, mult=mult)
+        torch.cuda.synchronize()
+    finally:
+        B.segquant_set_quantize_tuning(0)
+    codes = c_neg.cpu().numpy().view(np.int8).astype(np.float64)
+    assert np.all(c_pos.cpu().numpy() == 0)
+    assert np.all(np.abs(codes - exact * big / s) <= 0.5 + tol * big / s)
+    assert np.count_nonzero(codes) >= 2 * 5
