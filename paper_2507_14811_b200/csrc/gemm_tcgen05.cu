@@ -156,8 +156,8 @@ __device__ __forceinline__ void st_shared_volatile_u32(uint32_t addr, uint32_t v
     asm volatile("st.volatile.shared::cta.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 // abort_flag: shared-memory address of the CTA's abort word
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t abort_flag,
-                                          uint32_t *status, uint32_t where)
+__device__ __forceinline__ bool mbar_wait_lane(uint32_t bar, uint32_t parity, uint32_t abort_flag,
+                                               uint32_t *status, uint32_t where)
 {
     if (mbar_try_wait(bar, parity)) return true;
     long long t0 = 0;
@@ -177,7 +177,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
     return true;
 }
 
-// The same wait by a whole converged warp; every lane returns the same answer.
+// Waits of a whole warp: every lane returns the same answer.  What follows a wait is full of instructions of whole warps
+// (elect, tcgen05.ld, shuffles, votes, named barriers); lanes that disagreed on whether to go on would wait for one another
+// there, without a limit.  The epilogue's form lets the lanes poll on their own and votes once, after at most the limit
+// above (24 K-segments of 64 codes: 65.3 us a layer, with a vote in every poll 66.0); the issuing warps' stays
+// converged through the polls, for elect_one.
+__device__ __forceinline__ bool mbar_wait_agreed(uint32_t bar, uint32_t parity, uint32_t abort_flag,
+                                                 uint32_t *status, uint32_t where)
+{
+    return __all_sync(0xFFFFFFFFu, mbar_wait_lane(bar, parity, abort_flag, status, where));
+}
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint32_t abort_flag,
                                                uint32_t *status, uint32_t where)
 {
@@ -1218,7 +1227,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                 for (int p = 0; p < P; p++) {
                     const uint32_t cur_as = as, cur_aph = aph;
                     if (++as == uint32_t(prm.acc_stages)) { as = 0; aph ^= 1; }
-                    if (ok) ok = mbar_wait(smem_u32(&hdr->tmem_full[cur_as]), cur_aph, abort_flag, prm.status, kWhereEpilogue);
+                    if (ok) ok = mbar_wait_agreed(smem_u32(&hdr->tmem_full[cur_as]), cur_aph, abort_flag, prm.status, kWhereEpilogue);
                     if (!ok) continue;
                     tc_fence_after();
                     const uint32_t t_row = tmem_base + (uint32_t(lane_grp * 32) << 16) + cur_as * acc_cols +
@@ -1251,7 +1260,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                 // ---- all accumulators of the tile resident
                 const uint32_t cur_as = as, cur_aph = aph;
                 if (++as == uint32_t(prm.acc_stages)) { as = 0; aph ^= 1; }
-                if (ok) ok = mbar_wait(smem_u32(&hdr->tmem_full[cur_as]), cur_aph, abort_flag, prm.status, kWhereEpilogue);
+                if (ok) ok = mbar_wait_agreed(smem_u32(&hdr->tmem_full[cur_as]), cur_aph, abort_flag, prm.status, kWhereEpilogue);
                 if constexpr (SK) ok = epilogue_all(ok);    // the barriers below need all 256 threads or none
                 if (!ok) continue;                  // keep the named barriers balanced, do no more work
                 tc_fence_after();

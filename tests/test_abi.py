@@ -210,3 +210,18 @@ def test_native_calls_read_tensors_before_they_release_the_gil(L, call, bad, err
             torch.func.vmap(invoke)(torch.zeros(2, 4, 64))
         else:
             invoke(X.to_sparse() if bad.get("X") == "sparse" else X)
+
+
+def test_gemm_waits_give_a_warp_one_answer():
+    # a bounded wait that expires in some lanes of a warp only would leave the others in a shuffle or a named barrier for
+    # good; such a race cannot be provoked on purpose, so the source is held to the two forms that vote
+    import os
+    import re
+    src = open(os.path.join(os.path.dirname(B.__file__), "csrc", "gemm_tcgen05.cu")).read()
+    kernel = src[src.index("segquant_gemm_kernel(const __grid_constant__"):src.index("// ----------------------------------------------------------------------------- host side")]
+    waits = set(re.findall(r"\b(mbar_wait\w*)\s*\(", kernel))
+    assert waits == {"mbar_wait_warp", "mbar_wait_agreed"}
+    for name in waits:
+        start = src.index(f"bool {name}(")
+        body = src[start:src.index("\n}\n", start)]
+        assert body.count("return") == len(re.findall(r"return (?:true|false|__all_sync)", body)) and "__all_sync" in body
