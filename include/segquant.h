@@ -318,7 +318,7 @@ sq_status segquant_plan_run(const sq_plan *plan, void *stream);
 sq_status segquant_last_device_status(void *workspace, void *stream, uint32_t *detail);
 
 /* Tile plan of the GEMM kernel: tile_n in {0 (automatic), 32, 64, 128, 256}; stages 0 (automatic) or
- * 2..8 (shared-memory ring depth); cta_group 0 (automatic: CTA pairs on 256-row tiles when M > 128),
+ * 2..32 (shared-memory ring depth, at most what fits); cta_group 0 (automatic: CTA pairs on 256-row tiles when M > 128),
  * 1 (one CTA per 128-row tile) or 2; segment_mode for layers with several K-segments: 0 (automatic:
  * segments pass through tensor memory one after the other, running sums in registers), 1 (all
  * accumulators of a tile resident in tensor memory; at most 16 of them), 2 (sequential) or 4

@@ -1760,10 +1760,11 @@ sq_status prepare_kind<SQ_GEMM_KIND, SQ_GEMM_NPOL>(const GemmArgs &g, GemmLaunch
 
 #else   // the dispatch
 
-// What has been found out per (device, kernel instantiation, dynamic shared-memory size): how many CTA pairs can
+// What has been found out per (device, kernel instantiation for CTA pairs, dynamic shared-memory size): how many pairs can
 // be resident; and per (device, kernel instantiation) the largest dynamic shared-memory size the kernel's
 // attribute has been raised to (it is only ever raised, so that earlier plans stay launchable).  Guarded by a
-// mutex; a handful of entries.
+// mutex.  The size of a pair's shared memory depends on the tile width and the length of the factor tables, so there is
+// an entry per instantiation and table length in use; that of a single CTA also depends on M, and has no entries.
 struct KernelFacts { int device; const void *kernel; size_t smem; int clusters; };
 struct KernelSmem { int device; const void *kernel; size_t max_smem; };
 std::mutex g_facts_mu;
@@ -1786,13 +1787,13 @@ sq_status kernel_facts(int device, const void *key, size_t smem, int cg, const c
         if (ks) ks->max_smem = smem;
         else g_smem.push_back({device, key, smem});
     }
+    *clusters = 0;
+    if (cg != 2) return SQ_OK;
     for (const KernelFacts &f : g_facts)
         if (f.device == device && f.kernel == key && f.smem == smem) { *clusters = f.clusters; return SQ_OK; }
     int n = 0;
-    if (cg == 2) {
-        const cudaError_t eo = cudaOccupancyMaxActiveClusters(&n, key, &cfg);
-        if (eo != cudaSuccess || n <= 0) { note_cuda_error(eo != cudaSuccess ? eo : cudaErrorLaunchOutOfResources); return SQ_ERR_CUDA; }
-    }
+    const cudaError_t eo = cudaOccupancyMaxActiveClusters(&n, key, &cfg);
+    if (eo != cudaSuccess || n <= 0) { note_cuda_error(eo != cudaSuccess ? eo : cudaErrorLaunchOutOfResources); return SQ_ERR_CUDA; }
     g_facts.push_back({device, key, smem, n});
     *clusters = n;
     return SQ_OK;
