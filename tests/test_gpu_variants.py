@@ -30,6 +30,9 @@ DEV = "cuda"
     (1000, 1544, [0, 512, 1544], [0, 100, 1000]),
     (2500, 96, [0, 1, 2, 96], [0, 2499, 2500]),
     (130, 4100, list(range(0, 4101, 100)), [0, 64, 130]),
+    # K-bounds on, before and behind the columns at which one block's share ends (128 fp32, 256 bf16); a table of 64 x 64
+    (300, 1029, [0, 1, 127, 128, 129, 255, 256, 257, 511, 512, 1028, 1029], [0, 150, 300]),
+    (640, 2053, [i * 32 for i in range(64)] + [2053], [i * 9 for i in range(64)] + [640]),
 ])
 def test_calibration_scales_are_exact(case, x_dtype):
     """Extrema and one IEEE division per scale: bit-exact against the oracle, twice on one workspace whose contents are
