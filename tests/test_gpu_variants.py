@@ -664,3 +664,22 @@ def test_fused_activation_keeps_results_whose_exponential_is_subnormal(act, dtyp
     assert np.all(c_pos.cpu().numpy() == 0)
     assert np.all(np.abs(codes - exact * big / s) <= 0.5 + tol * big / s)
     assert np.count_nonzero(codes) >= 2 * 5
+
+
+@pytest.mark.parametrize("act", ["silu", "gelu", "geglu", None])
+@pytest.mark.parametrize("code,dual", [("int8", True), ("int8", False), ("e4m3", True)])
+def test_fused_fp32_rows_that_one_thread_walks_equal_single_rows(act, code, dual):
+    """fp32 input of so many rows that a thread handles several of them through its ring: the first and the last rows get the
+    codes they get in a call of their own, where a thread handles one."""
+    M, K = 9000, 512
+    g = torch.Generator(device=DEV).manual_seed(17)
+    H = torch.randn((M, 2 * K if act == "geglu" else K), generator=g, device=DEV) * 2
+    mult = torch.rand((K,), generator=g, device=DEV) + 0.5
+    seg = B.SegTable([0, 192, K], [0, 8])
+    sp = torch.tensor([0.03, 0.05], device=DEV)
+    sn = torch.tensor([0.002, 0.004], device=DEV) if dual else None
+    run = lambda X: B.segquant_quantize_act_fused(X, seg, sp, sn, code, act=act, mult=mult)
+    c_pos, c_neg = run(H)
+    for rows in (slice(0, 300), slice(4000, 4300), slice(M - 300, M)):
+        p, n = run(H[rows].contiguous())
+        assert torch.equal(c_pos[rows], p) and (not dual or torch.equal(c_neg[rows], n))
