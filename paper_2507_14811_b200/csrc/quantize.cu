@@ -718,9 +718,10 @@ quantize_table_kernel(const __grid_constant__ QuantParams prm)
 // its extrema per K-segment are reduced in shared memory, the scales (one IEEE division each) are written out,
 // and the codes are made from the registers with the same quantizer as everywhere else.
 constexpr int kRowChunks = 4;                       // K <= 256 threads x 4 chunks x 16 = 16384
-// CHUNKS: chunks a thread may hold.  One where a block covers the row with one per thread (K <= 4096): fewer registers, more
-// rows in flight (us, 4 / 1 chunks: 921 x 1920 dual with 12 segments 8.1 / 4.4, 8858 x 1536 with 24 16.4 / 13.9, 8858 x 3072
-// with 2 21.6 / 20.1).  Two up to K = 8192 were no better on many rows (8858 x 6144 42.8 / 44.5).
+// CHUNKS: chunks a thread may hold.  One where a block of 256 threads covers the row with one per thread (K <= 4096): fewer
+// registers, more rows in flight (us, 4 / 1 chunks: 921 x 1920 dual with 12 segments 8.1 / 4.4, 8858 x 1536 with 24
+// 16.4 / 13.9, 8858 x 3072 with 2 21.6 / 20.1).  Two up to K = 8192 were no better on many rows (8858 x 6144 42.8 / 44.5);
+// one per thread on larger blocks has not been measured.  Exception, see per_row_chunks: many long rows of one K-segment.
 
 __device__ __forceinline__ uint32_t ord_enc(float f)     // monotone map float -> uint32
 {
@@ -1116,10 +1117,29 @@ sq_status launch_quantize(const void *X, sq_dtype dt, int64_t M, int64_t K, int6
     return s == SQ_OK ? run_quantize(L, st) : s;
 }
 
-template <typename Tin, bool DUAL, typename... Args>
-static cudaError_t launch_per_row(cudaLaunchConfig_t &cfg, int64_t V, Args... args)
+// Chunks per thread for M rows of V chunks in P K-segments.  With several segments one is the better up to V = 256 (time
+// with 1 over time with 4, M 512 .. 32768, K 512 .. 4096: 0.57 .. 1.00).  With one segment a row costs so little beside its
+// loads that, on many rows, four chunks on a quarter of the threads win where these fill their warps reasonably
+// (1 / 4, M = 8858 bf16 single: K = 3072 1.18, 2560 0.99 (40 of 64 threads), 2048 1.16, 1536 1.14, 1024 0.99; M = 16000,
+// K = 2816 1.17; fp32 single, M = 8858: 1.04, 0.93, 1.10, 0.96, 0.95).  On few rows one wins there too (M = 1024:
+// 0.81 .. 1.01).  The lines below are where the ratio crosses 1 (bf16 dual, K = 2048: M = 2048 0.89, 4096 1.05, 6000 1.10;
+// K = 4096: M = 1024 0.93, 2048 1.10).
+template <typename Tin>
+static int64_t per_row_chunks(int64_t M, int64_t V, int P)
 {
-    const int64_t chunks = V <= kThreads ? 1 : kRowChunks;
+    constexpr bool k16 = sizeof(Tin) == 2;
+    if (V > kThreads) return kRowChunks;
+    if (P > 1) return 1;
+    if (V > 160) return M >= 2048 ? kRowChunks : 1;                              // K > 2560: two warps with four chunks a thread
+    if (V <= 128 && V > 96) return M >= (k16 ? 4096 : 6000) ? kRowChunks : 1;    // K > 1536: one warp
+    if (V <= 96 && V > 64) return k16 && M >= 6000 ? kRowChunks : 1;             // K > 1024
+    return 1;
+}
+
+template <typename Tin, bool DUAL, typename... Args>
+static cudaError_t launch_per_row(cudaLaunchConfig_t &cfg, int64_t V, int P, Args... args)
+{
+    const int64_t chunks = per_row_chunks<Tin>(int64_t(cfg.gridDim.x), V, P);
     cfg.blockDim = dim3(unsigned(((V + chunks - 1) / chunks + 31) / 32 * 32));
     return chunks == 1 ? cudaLaunchKernelEx(&cfg, quantize_per_row_kernel<Tin, DUAL, 1>, args...)
                        : cudaLaunchKernelEx(&cfg, quantize_per_row_kernel<Tin, DUAL, kRowChunks>, args...);
@@ -1145,12 +1165,12 @@ sq_status launch_quantize_per_row(const void *X, sq_dtype dt, int64_t M, int64_t
     cudaError_t e;
     if (dt == SQ_F32) {
         const float *x = static_cast<const float *>(X);
-        e = dual ? launch_per_row<float, true>(cfg, V, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc)
-                 : launch_per_row<float, false>(cfg, V, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc);
+        e = dual ? launch_per_row<float, true>(cfg, V, sb.P, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc)
+                 : launch_per_row<float, false>(cfg, V, sb.P, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc);
     } else {
         const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(X);
-        e = dual ? launch_per_row<__nv_bfloat16, true>(cfg, V, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc)
-                 : launch_per_row<__nv_bfloat16, false>(cfg, V, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc);
+        e = dual ? launch_per_row<__nv_bfloat16, true>(cfg, V, sb.P, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc)
+                 : launch_per_row<__nv_bfloat16, false>(cfg, V, sb.P, x, Ki, ld, sb, q_max, q_min_abs, s_pos, s_neg, cp, cn, ldc);
     }
     count_launch();
     if (e != cudaSuccess) { note_cuda_error(e); return SQ_ERR_CUDA; }

@@ -683,3 +683,18 @@ def test_fused_fp32_rows_that_one_thread_walks_equal_single_rows(act, code, dual
     for rows in (slice(0, 300), slice(4000, 4300), slice(M - 300, M)):
         p, n = run(H[rows].contiguous())
         assert torch.equal(c_pos[rows], p) and (not dual or torch.equal(c_neg[rows], n))
+
+
+@pytest.mark.parametrize("x_dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("dual", [True, False])
+@pytest.mark.parametrize("M,K", [(2048, 2561), (2048, 4096), (6000, 1041), (6000, 2048)])
+def test_per_row_many_rows_of_one_segment_equal_few_rows(M, K, dual, x_dtype):
+    """Many rows of one K-segment hold four chunks per thread, few rows one: the same scales and codes."""
+    g = torch.Generator(device=DEV).manual_seed(19)
+    X = torch.zeros((M, (K + 15) // 16 * 16), dtype=x_dtype, device=DEV)[:, :K]
+    X.copy_(torch.randn((M, K), generator=g, device=DEV))
+    seg = B.SegTable([0, K], [0, 8])
+    whole = B.segquant_quantize_per_row(X, seg, dual)
+    for rows in (slice(0, 40), slice(M - 40, M)):
+        part = B.segquant_quantize_per_row(X[rows], seg, dual)
+        assert all((w is None and p is None) or torch.equal(w[rows], p) for w, p in zip(whole, part))
