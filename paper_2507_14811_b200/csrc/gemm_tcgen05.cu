@@ -63,9 +63,15 @@ constexpr int kLaunchRegs = 168;      // per thread at launch: 65536 / 384, roun
 constexpr int kFrontRegs = 56, kEpiRegs = 224;     // per-thread register counts after the role split
 // setmaxnreg.inc waits, without limit, until the CTA's OWN register allocation (made at launch) has that many
 // registers free, so the new counts must fit in what the launch gave the CTA
-static_assert(kFrontThreads * kFrontRegs + kEpiThreads * kEpiRegs <= kThreads * kLaunchRegs,
-              "register counts after the role split exceed the CTA's allocation");
-static_assert(kFrontRegs % 8 == 0 && kEpiRegs % 8 == 0 && kFrontRegs >= 24 && kEpiRegs <= 256, "setmaxnreg operand");
+// The checking variant's epilogue needs fewer and its issuing warps spilled with 56 (with that and two load buffers in the
+// path of run-time unit counts, W4A8 to fp32 had lost 8 to 12 %: 4100 x 1152 -> 6912 dual 92.0 -> 99.9 us, single 60.1 -> 68.5).
+constexpr int kFrontRegsChecking = 72, kEpiRegsChecking = 216;
+constexpr bool role_split_fits(int front, int epi)
+{
+    return kFrontThreads * front + kEpiThreads * epi <= kThreads * kLaunchRegs && front % 8 == 0 && epi % 8 == 0 && front >= 24 && epi <= 256;
+}
+static_assert(role_split_fits(kFrontRegs, kEpiRegs) && role_split_fits(kFrontRegsChecking, kEpiRegsChecking),
+              "setmaxnreg operands, or register counts after the role split exceed the CTA's allocation");
 [[maybe_unused]] constexpr int kEpiBufRegs = 192;      // of kEpiRegs: accumulator load buffers plus running sums (SEQ)
 [[maybe_unused]] constexpr int kResidentBufs = 4;      // accumulator load buffers of the resident epilogue
 [[maybe_unused]] constexpr int kMaxStages = 32;
@@ -877,7 +883,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
     // The producer and the MMA issuer are one warp each: their loops are kept to a few dozen
     // instructions per K-block (ring slot and phase advance incrementally, descriptors by addition).
     if (warp < kFrontThreads / 32) {
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFrontRegs));
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(GENERIC ? kFrontRegsChecking : kFrontRegs));
       if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         {
@@ -1081,7 +1087,7 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
         // Warp w may read TMEM lanes 32 * (w % 4) .. + 31; the two warps of one lane group take one half
         // of the tile's 32-column slabs each.  Per output: y = bias, then y = fma(c[a][q], acc[a], y) over
         // a = (p, polarity) ascending, two outputs per instruction on packed fp32 pairs.
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpiRegs));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(GENERIC ? kEpiRegsChecking : kEpiRegs));
         const int et = threadIdx.x - kFrontThreads;
         const int ew = warp - kFrontThreads / 32;
         const int lane_grp = warp & 3;
@@ -1494,6 +1500,14 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                 };
                 if (units == 0) {
                     release(cur_as);
+                } else if (GENERIC) {                // one load at a time: this path's registers are the whole kernel's (see kFrontRegs)
+#pragma unroll 1
+                    for (int u = 0; u < units; u++) {
+                        issue(ra);
+                        tc_wait_ld();
+                        if (u + 1 == units) release(cur_as);
+                        consume(ra);
+                    }
                 } else {
                     issue(ra);
 #pragma unroll 1
