@@ -1670,8 +1670,18 @@ sq_status prepare_tile(const GemmArgs &g, GemmLaunch &L, int tile_n, bool seq, i
     // the other variants write Y with TMA stores: 16-byte aligned base and row pitch
     dbg = dbg || reinterpret_cast<uintptr_t>(g.Y) % 16 != 0 || (size_t(g.ldy) * (prm.y_is_f32 ? 4 : 2)) % 16 != 0;
     // fp32 output and slabs that straddle an N-bound
-    bool flex = prm.y_is_f32;
-    for (int q = 1; q < prm.sb.Q; q++) flex = flex || (prm.sb.nb[q] % 32 != 0);
+    bool straddles = false;
+    for (int q = 1; q < prm.sb.Q; q++) straddles = straddles || (prm.sb.nb[q] % 32 != 0);
+    const bool flex = prm.y_is_f32 || straddles;
+    // The flexible variant's staging of fp32 blocks (32 KiB) costs dual 128-column tiles the fifth ring stage.  Where the K loop
+    // is long and the epilogue of one tile runs under the next one's, the checking variant, which stores directly, is the
+    // faster one (us, flexible / checking, dual int8: one K-segment 2048 x 12288 -> 3072 110.1 / 96.9, x 6144 51.3 / 48.0,
+    // x 3072 28.6 / 28.4; two K-segments 4100 x 12288 -> 1152 117.1 / 96.6, x 6144 52.2 / 49.4, x 1152 0.78 of its time;
+    // less than one wave of tiles: 500 x 6144 -> 3072 0.97 and 0.96 of its time).
+    if constexpr (NPOL == 2 && CG == 2) {
+        const int64_t tiles_128 = ((g.M + 2 * TILE_M - 1) / (2 * TILE_M)) * ((g.N + 127) / 128);
+        if (prm.y_is_f32 && !straddles && tile_n == 128 && g.K >= 6144 && tiles_128 > sm_count / 2) dbg = true;
+    }
     // per-token x per-channel scales: the production variant stages a tile's channel scales in shared memory, which
     // it does for up to 32 K-segments, int8 codes and CTA pairs; anything else runs the checking variant
     const bool pt = prm.col_scale != nullptr;

@@ -698,3 +698,23 @@ def test_per_row_many_rows_of_one_segment_equal_few_rows(M, K, dual, x_dtype):
     for rows in (slice(0, 40), slice(M - 40, M)):
         part = B.segquant_quantize_per_row(X[rows], seg, dual)
         assert all((w is None and p is None) or torch.equal(w[rows], p) for w, p in zip(whole, part))
+
+
+@pytest.mark.parametrize("code", ["int8", "e4m3"])
+@pytest.mark.parametrize("kb", [[0, 6144], [0, 3072, 6144], [0, 6128]])
+def test_fp32_output_of_long_dual_layers_equals_few_rows(kb, code):
+    """Dual layers with fp32 output and more than a wave of 128-column tiles store directly from K = 6144 on; fewer rows, and
+    shorter rows, go through the staged stores."""
+    M, N, K, P = 2305, 1160, kb[-1], len(kb) - 1
+    g = torch.Generator(device=DEV).manual_seed(23)
+    Xp, Xn, W = B.new_codes(M, K, DEV), B.new_codes(M, K, DEV), B.new_codes(N, K, DEV)
+    for t, hi in ((Xp, 100), (Xn, 100), (W, 100)):           # int8: 0 .. 99; e4m3: finite codes of either size
+        t.copy_(torch.randint(0, hi, t.shape, generator=g, device=DEV, dtype=torch.uint8))
+    seg, ws = B.SegTable(kb, [0, 576, N]), B.new_workspace(DEV)
+    rnd = lambda *s: torch.rand(s, generator=g, device=DEV) * 0.01
+    sp, sn, sw, bias = rnd(P), rnd(P), rnd(P * 2), rnd(N)
+    run = lambda r: B.segquant_dualscale_gemm(Xp[r], Xn[r], W, seg, code, sp, sn, sw, bias, ws, y_dtype=torch.float32)
+    whole = run(slice(0, M))
+    for rows in (slice(0, 200), slice(M - 200, M)):
+        assert torch.equal(whole[rows], run(rows))
+    B.check_device_status(ws)
