@@ -718,6 +718,18 @@ def measure_side_workload(name, dev, args, peaks):
 SIDE_WORKLOADS = ["flux", "dit_xl2", "sdxl_skip", "sdxl_sweep", "sd3_heads", "sdxl_geglu", "modulation_small_m", "sd3_qkv_768x2"]
 
 
+def report_config(workload, specs, world, steps, reps, region_s, step_mode, n_sets, set_bytes):
+    """What was run, in the report's words."""
+    return {"workload": workload,
+            "layers": [f"{s.name} M={s.M} K={s.K} N={s.N} P={s.P} Q={s.Q} {'dual' if s.dual else 'single'} {s.code}" for s in specs],
+            "step": "every layer: quantize_act -> dual/seg GEMM + dequant epilogue (bf16 out)",
+            "timed_region": f"{step_mode}: {reps} x {steps} steps, {region_s:.3f} s between one pair of CUDA events",
+            "ops": "executed tensor ops: 4MNK for dual layers, 2MNK for single-scale layers",
+            "l2": f"inputs larger than L2: step i uses buffer set i mod {n_sets} ({set_bytes / 2**20:.0f} MiB per set, "
+                  f"{n_sets * set_bytes / 2**20:.0f} MiB in all, L2 = {L2_BYTES >> 20} MiB)",
+            "parallelism": f"{world} independent row-sharded replicas, no collective" if world > 1 else "1 GPU"}
+
+
 def run_ours(args):
     from paper_2507_14811_b200 import binding as B
     from paper_2507_14811_b200 import workloads as WL
@@ -839,18 +851,7 @@ def run_ours(args):
             "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(step_ms, 5),
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
             "dtype": "e4m3" if specs[0].code == "e4m3" else "int8", "data": "synthetic",
-            "config": {"workload": args.workload,
-                       "layers": [f"{s.name} M={s.M} K={s.K} N={s.N} P={s.P} Q={s.Q} {'dual' if s.dual else 'single'} {s.code}"
-                                  for s in specs],
-                       "step": "every layer: quantize_act -> dual/seg GEMM + dequant epilogue (bf16 out); steps run "
-                               "back to back between one pair of CUDA events",
-                       "timed_region": f"{step_mode}: {reps} replay(s) x {args.steps} steps = {reps * args.steps} steps, "
-                                       f"{region_s:.3f} s between one pair of CUDA events",
-                       "ops": "executed tensor ops: 4MNK for dual layers, 2MNK for single-scale layers",
-                       "l2": f"inputs larger than L2: step i uses buffer set i mod {n_sets} (weights, inputs, codes, outputs; "
-                             f"{set_bytes / 2**20:.0f} MiB per set, {n_sets * set_bytes / 2**20:.0f} MiB in all, L2 = {L2_BYTES >> 20} MiB); "
-                             "the per-kernel timings rotate over copies of one layer's buffers the same way",
-                       "parallelism": f"{world} independent row-sharded replicas, no collective" if world > 1 else "1 GPU"},
+            "config": report_config(args.workload, specs, world, args.steps, reps, region_s, step_mode, n_sets, set_bytes),
             "timed_region_s": round(region_s, 4), "graph_replays": reps,
             "useful_tops": round(world * useful_ops / (step_ms * 1e-3) / 1e12, 2),
             "whole_step": dict(fractions(step_tops, p8),
@@ -918,6 +919,32 @@ GEMM_DRAM_TRAFFIC = {
                 "from": "ncu --set full of the two GEMM launches of one eager step (bench.py --workload dit_xl2 "
                         "--profile-steps 4); operands partly L2-resident from the quantize pass, Y stays in L2"},
 }
+
+
+# What the one line on standard output carries of the report; the rest (per-layer tables, those of the other workloads, notes)
+# goes to the file that --details names.  A log that keeps the last 3000 characters of the output still has the line.
+LINE_MAX_CHARS = 2600
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline", "dtype",
+             "data", "config", "timed_region_s", "graph_replays", "useful_tops", "ms_per_step_kernels_timed_alone",
+             "ms_per_step_planned_calls_from_host", "frac_of_nominal_4500_tops", "gpu_launches", "clocks")
+LINE_PARTS = {
+    "whole_step": ("of_measured_burst", "of_measured_sustained", "of_nominal_4500"),
+    "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step"),
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "frac_of_sustained_peak", "traffic", "kernel", "launches_per_step"),
+    "quantize_roofline": ("bound", "achieved", "peak", "unit", "frac"),
+    "cpu_baseline": ("value", "unit", "cores", "kind"),
+}
+
+
+def report_line(out):
+    """The report without its tables and notes."""
+    line = {k: out[k] for k in LINE_KEYS if k in out}
+    for part, keys in LINE_PARTS.items():
+        if out.get(part) is not None:
+            line[part] = {k: out[part][k] for k in keys if k in out[part]}
+    if out.get("workloads"):
+        line["ms_per_step_of_workloads"] = {name: w.get("ms_per_step") for name, w in out["workloads"].items()}
+    return line
 
 
 def gemm_source_tag():
@@ -998,6 +1025,7 @@ def main():
     ap.add_argument("--only-headline", action="store_true", help="skip the per-layer tables of the other workloads")
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--details", default=None, metavar="FILE", help="write the whole report, tables and notes included, to FILE")
     ap.add_argument("--tile-n", type=int, default=0)
     ap.add_argument("--stages", type=int, default=0)
     ap.add_argument("--cta-group", type=int, default=0)
@@ -1012,6 +1040,11 @@ def main():
             from paper_2507_14811_b200 import binding as B
             B.segquant_set_tuning(args.tile_n, args.stages, args.cta_group, args.segment_mode)
         out = run_ours(args)
+    if out is not None and args.impl == "ours":
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(out, f)
+        out = report_line(out)
     if out is not None:
         print(json.dumps(out))
 
