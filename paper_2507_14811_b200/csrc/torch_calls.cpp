@@ -83,8 +83,12 @@ struct Rows {
     void *p;
     int64_t rows, cols, ld;           // cols: of the last dimension
     bool on_host;
-    explicit Rows(const at::Tensor &t)
-        : p(t.data_ptr()), rows(t.size(0)), cols(t.size(-1)), ld(t.stride(0)), on_host(!t.is_cuda()) {}
+    explicit Rows(const at::Tensor &t) : p(t.data_ptr()), on_host(!t.is_cuda())
+    {
+        const at::IntArrayRef sizes = t.sizes(), strides = t.strides();
+        if (sizes.empty()) (void)t.size(0);                           // throws the error that t.stride(0) gives in Python
+        rows = sizes.front(), cols = sizes.back(), ld = strides.front();
+    }
 };
 
 template <typename F>
