@@ -153,7 +153,7 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
 // Both are written for TWO elements: the multiplies, FMAs and adds go two per instruction (packed fp32 pairs), each of
 // them rounding exactly as the scalar instruction does, which is what bounds the fused pass (the ALUs, not memory).
 // (8192 x 2560 gated GELU, dual int8, 126 MB: 49.4 us one element at a time with the gate half one row ahead in registers,
-// 35.0 us with pairs and the gate half in the ring; without the table, 54 M elements of GELU 93 -> 72 us.)
+// 37.9 us with pairs and the gate half in the ring; without the table, 54 M elements of GELU 93 -> 80 us.)
 // GELU without branches: with a = min(|h|, 20), v = max(h, 0) - (a / 2) E in one FMA is h - (h / 2) E for h >= 0 and
 // (h / 2) E below; at a = 20 the exponential has long underflowed to zero, so v is h or +0 beyond it and t^2 stays
 // finite for every h.
@@ -604,9 +604,9 @@ quantize_table_kernel(const __grid_constant__ QuantParams prm)
     //   2^-124 <= |h| < 2^-26: both give h / 2 after the rounding to bf16 (the sigmoid / Phi factor is 1/2 to
     //                          far below a bf16 half-step);
     //   h >= 32 (SiLU), h >= 16 (GELU): h itself (exp(-h), erfc(h / sqrt 2) are below fp32's resolution of 1);
-    //   h <= -128 (SiLU), h <= -16 (GELU): -0 (the exponential has underflowed to zero).
-    // NaN and infinities go through the functions.  The test that compares this variant with the arithmetic one
-    // on all 65536 patterns holds these statements to the bit.
+    //   h <= -128 (SiLU), h <= -16 (GELU): -0 and +0 (the exponential has underflowed to zero).
+    // NaN and infinities go through the functions.  A test compares the codes of this variant with those of the arithmetic
+    // one on all 65536 patterns (the sign of a zero does not show in a code).
     const bool is_silu = prm.act == 1;
     for (uint32_t b = threadIdx.x; b < 65536u; b += kTableThreads) {
         const uint32_t e = (b >> 7) & 0xFFu, neg = b >> 15;
@@ -616,7 +616,7 @@ quantize_table_kernel(const __grid_constant__ QuantParams prm)
         } else if (e != 255u && !neg && e >= (is_silu ? 132u : 131u)) {
             out = b;
         } else if (e != 255u && neg && e >= (is_silu ? 134u : 131u)) {
-            out = 0x8000u;
+            out = is_silu ? 0x8000u : 0u;
         } else {
             const float h = __uint_as_float(b << 16);
             float a, a_same;
@@ -1016,9 +1016,10 @@ sq_status prepare_mode(QuantLaunch &L, sq_code code, int mode)
 // The table variant of the fused activation: bf16 input, SiLU or GELU, every 16-element chunk inside one K-segment,
 // and enough elements for the table's set-up time not to count.  Returns false where it does not apply.
 std::atomic<int> g_table_mode{0};        // test hook: 0 automatic, 1 always where possible, 2 never
-// measured break-even points (us, evaluated per element against table): SiLU 16 Mi elements 20.8 / 20.9, 24 Mi 28.5 / 27.2;
-// GELU 8 Mi 14.8 / 15.4, 10 Mi 17.3 / 17.2, 16 Mi 25.5 / 21.6
-constexpr int64_t kTableMinSilu = int64_t(18) << 20, kTableMinGelu = int64_t(10) << 20;
+// measured break-even points (us, evaluated per element against table, K = 1152 and 4608 alike): GELU dual 8 Mi elements
+// 14.4 / 15.2, 9 Mi 16.2 / 16.1, 16 Mi 26.6 / 21.7, single 9 Mi 14.3 / 15.0, 10 Mi 15.8 / 15.7; SiLU dual 18 Mi 21.6 / 22.1,
+// 20 Mi 23.8 / 23.5, 24 Mi 28.0 / 26.8, single 20 Mi 19.6 / 21.8, 24 Mi 23.3 / 24.7 (0.9 / 0.7 us per further Mi)
+constexpr int64_t table_min(bool silu, bool dual) { return int64_t(silu ? (dual ? 20 : 30) : (dual ? 9 : 10)) << 20; }
 bool prepare_table(QuantLaunch &L, sq_dtype dt, sq_code code, int mode)
 {
     QuantParams &prm = L.prm;
@@ -1028,7 +1029,7 @@ bool prepare_table(QuantLaunch &L, sq_dtype dt, sq_code code, int mode)
     if (prm.K % kVec != 0) return false;
     for (int p = 1; p < prm.sb.P; p++)
         if (prm.sb.kb[p] % kVec != 0) return false;
-    if (tm != 1 && prm.M * int64_t(prm.K) < (prm.act == SQ_ACT_SILU ? kTableMinSilu : kTableMinGelu)) return false;
+    if (tm != 1 && prm.M * int64_t(prm.K) < table_min(prm.act == SQ_ACT_SILU, mode == kDual)) return false;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
