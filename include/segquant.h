@@ -234,7 +234,8 @@ size_t segquant_layer_scratch_bytes(int64_t M, int64_t K, int dual);
  *   x_on_host / y_on_host != 0: X / Y are HOST buffers (pinned memory recommended); the call copies
  *   X to `x_stage` (dev, M*ld*sizeof(dt) bytes) before and Y from `y_stage` (dev, M*ldy*sizeof(y_dtype)
  *   bytes) after the kernels, on `stream`.  With device X / Y the stage pointers are ignored.
- *   scratch: dev, segquant_layer_scratch_bytes(M,K,dual) bytes, 256-byte aligned (code matrices). */
+ *   scratch: dev, segquant_layer_scratch_bytes(M,K,dual) bytes, 256-byte aligned (code matrices; a layer of few rows
+ *   may run as one kernel that quantizes its activations itself and leaves the scratch as it is). */
 sq_status segquant_layer_forward(const void *X, int x_on_host, void *x_stage, sq_dtype dt,
                                  int64_t M, int64_t K, int64_t ld,
                                  const void *Wq, int64_t ldw, int64_t N, const sq_segtable *seg, sq_code code,
@@ -295,8 +296,8 @@ sq_status segquant_w4a8_gemm(const void *Xq_pos, const void *Xq_neg, int64_t ldx
 /* A layer call prepared once and replayed.  segquant_plan_layer does everything segquant_layer_forward does on
  * the host for device X and Y -- argument checks, tile plan, kernel choice, tensor-map encoding, attribute set-up --
  * and stores the result in caller-owned memory instead of launching; segquant_plan_run then issues the layer's
- * two kernels (quantize, GEMM + epilogue) on `stream` with no further checks, queries or encoding, for callers
- * that run the same layer on the same buffers again and again (its host cost is two kernel launches).
+ * two kernels (quantize, GEMM + epilogue; one for some layers of few rows) on `stream` with no further checks, queries or
+ * encoding, for callers that run the same layer on the same buffers again and again (its host cost is the launches).
  *   The plan is plain data: it may be copied or freed at will and owns nothing.  It refers to the buffers by
  *   address: X, Wq, the scale tables, bias, Y, scratch and workspace must stay where they were (their CONTENTS
  *   may change between runs); after any pointer, shape or pitch change build a new plan.  A plan belongs to the
@@ -324,7 +325,9 @@ sq_status segquant_last_device_status(void *workspace, void *stream, uint32_t *d
  * accumulators of a tile resident in tensor memory; at most 16 of them), 2 (sequential) or 4
  * (automatic, but single-scale layers keep 256 x 256 tiles instead of 256 x 512 ones) or 5 (256 x 512
  * tiles for single-scale layers even where the automatic choice expects no gain from them), 6 (split
- * tiles wherever the layer and the workspace allow them) or 7 (never split tiles).
+ * tiles wherever the layer and the workspace allow them), 7 (never split tiles), 8 (the GEMM of few rows wherever it
+ * fits; then tile_n is its output channels per tile, 32 .. 128, stages its tokens per tile, 8 .. 256, and cta_group the
+ * CTAs that share a K range, 1, 2, 4 or 8; 0: automatic) or 9 (never that one).
  * Process-wide (atomic words read when a launch or a plan is prepared); meant for benchmarking sweeps and
  * tests only: production callers leave everything automatic.  Values the layer cannot use are replaced by the
  * automatic choice. */

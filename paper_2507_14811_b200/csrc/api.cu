@@ -114,11 +114,41 @@ static sq_status gemm_common(const void *a_pos, const void *a_neg, int dual, int
     return st == SQ_OK ? launch_gemm(g, static_cast<cudaStream_t>(stream)) : st;
 }
 
+static bool overlap(const void *a, size_t a_bytes, const void *b, size_t b_bytes)
+{
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + b_bytes && y < x + a_bytes;
+}
+
+// A layer of few rows as one launch that quantizes its activations itself.  Fills L and returns true if everything is in
+// order and the layer is one that this form takes; otherwise the caller goes on with the two kernels, which also report what
+// is wrong.  An output that overlaps the input stays with the two kernels: there the input has been read when Y is written.
+static bool fused_layer(const void *X, sq_dtype dt, int64_t M, int64_t K, int64_t ld, const void *Wq, int64_t ldw, int64_t N,
+                        const sq_segtable *seg, sq_code code, const float *s_pos, const float *s_neg, const float *s_w,
+                        const float *bias, uint32_t flags, void *Y, sq_dtype y_dtype, int64_t ldy, void *scratch,
+                        void *workspace, size_t ws_bytes, GemmLaunch *L)
+{
+    if (M > kFusedRows || check_matrix(X, M, K, ld, dt_size(dt)) != SQ_OK) return false;
+    const int dual = s_neg != nullptr;
+    GemmArgs g;
+    if (gemm_args(scratch, dual ? scratch : nullptr, dual, (K + 127) & ~int64_t(127), Wq, ldw, M, N, K, seg, code, s_pos, s_neg, s_w,
+                  bias, Y, y_dtype, ldy, nullptr, workspace, ws_bytes, &g) != SQ_OK)
+        return false;
+    if (overlap(X, (size_t(M - 1) * ld + K) * dt_size(dt), Y, (size_t(M - 1) * ldy + N) * dt_size(y_dtype))) return false;
+    g.X = X;
+    g.x_dtype = dt;
+    g.ldx = ld;
+    g.q_hi = int(code_qmax(code));
+    g.q_lo = dual ? -int(code_qmin_abs(code, flags)) : -g.q_hi;
+    return prepare_fused_layer(g, L) == SQ_OK;
+}
+
 // What an sq_plan holds (copied in and out of the caller's storage, which need not be aligned for it).
 struct LayerPlan {
     uint64_t magic;
-    QuantLaunch quant;
+    QuantLaunch quant;        // not launched where the GEMM quantizes its activations itself
     GemmLaunch gemm;
+    int fused;
 };
 constexpr uint64_t kPlanMagic = 0x53514C41594552ull;   // "SQLAYER"
 static_assert(sizeof(LayerPlan) <= sizeof(sq_plan), "sq_plan is too small for a layer plan");
@@ -313,16 +343,23 @@ sq_status segquant_layer_forward(const void *X, int x_on_host, void *x_stage, sq
             return SQ_ERR_CUDA;
         xd = x_stage;
     }
-    const int64_t ldc = (K + 127) & ~int64_t(127);
-    uint8_t *c_pos = static_cast<uint8_t *>(scratch);
-    uint8_t *c_neg = dual ? c_pos + ((size_t(M) * ldc + 255) & ~size_t(255)) : nullptr;
-    sq_status r = segquant_quantize_act(xd, dt, M, K, ld, seg, s_pos, s_neg, code, flags, c_pos, c_neg, ldc, stream);
-    if (r != SQ_OK) return r;
     void *yd = y_on_host ? y_stage : Y;
-    r = dual ? segquant_dualscale_gemm(c_pos, c_neg, ldc, Wq, ldw, M, N, K, seg, code, s_pos, s_neg, s_w, bias, yd,
-                                       y_dtype, ldy, nullptr, workspace, ws_bytes, stream)
-             : segquant_seglinear_gemm(c_pos, ldc, Wq, ldw, M, N, K, seg, code, s_pos, s_w, bias, yd, y_dtype, ldy,
-                                       nullptr, workspace, ws_bytes, stream);
+    GemmLaunch one;
+    sq_status r;
+    if (fused_layer(xd, dt, M, K, ld, Wq, ldw, N, seg, code, s_pos, s_neg, s_w, bias, flags, yd, y_dtype, ldy, scratch, workspace,
+                    ws_bytes, &one)) {
+        r = run_gemm(one, st);
+    } else {
+        const int64_t ldc = (K + 127) & ~int64_t(127);
+        uint8_t *c_pos = static_cast<uint8_t *>(scratch);
+        uint8_t *c_neg = dual ? c_pos + ((size_t(M) * ldc + 255) & ~size_t(255)) : nullptr;
+        r = segquant_quantize_act(xd, dt, M, K, ld, seg, s_pos, s_neg, code, flags, c_pos, c_neg, ldc, stream);
+        if (r != SQ_OK) return r;
+        r = dual ? segquant_dualscale_gemm(c_pos, c_neg, ldc, Wq, ldw, M, N, K, seg, code, s_pos, s_neg, s_w, bias, yd,
+                                           y_dtype, ldy, nullptr, workspace, ws_bytes, stream)
+                 : segquant_seglinear_gemm(c_pos, ldc, Wq, ldw, M, N, K, seg, code, s_pos, s_w, bias, yd, y_dtype, ldy,
+                                           nullptr, workspace, ws_bytes, stream);
+    }
     if (r != SQ_OK) return r;
     if (y_on_host &&
         cudaMemcpyAsync(Y, y_stage, size_t(M) * ldy * dt_size(y_dtype), cudaMemcpyDeviceToHost, st) != cudaSuccess)
@@ -480,6 +517,13 @@ sq_status segquant_plan_layer(sq_plan *plan, const void *X, sq_dtype dt, int64_t
                         nullptr, workspace, ws_bytes, &g)) != SQ_OK)
         return st;
     LayerPlan lp{};
+    if (fused_layer(X, dt, M, K, ld, Wq, ldw, N, seg, code, s_pos, s_neg, s_w, bias, flags, Y, y_dtype, ldy, scratch, workspace,
+                    ws_bytes, &lp.gemm)) {
+        lp.fused = 1;
+        lp.magic = kPlanMagic;
+        std::memcpy(plan, &lp, sizeof(lp));
+        return SQ_OK;
+    }
     if ((st = prepare_quantize(X, dt, M, K, ld, g.sb, s_pos, s_neg, nullptr, 0, code, code_qmax(code),
                                code_qmin_abs(code, flags), 0, nullptr, c_pos, c_neg, ldc, &lp.quant)) != SQ_OK)
         return st;
@@ -499,7 +543,7 @@ sq_status segquant_plan_run(const sq_plan *plan, void *stream)
     if (cudaGetDevice(&dev) != cudaSuccess) return SQ_ERR_CUDA;
     if (dev != lp.gemm.device) return SQ_ERR_UNSUPPORTED;      // plans belong to the device they were built on
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const sq_status r = run_quantize(lp.quant, st);
+    const sq_status r = lp.fused ? SQ_OK : run_quantize(lp.quant, st);
     return r == SQ_OK ? run_gemm(lp.gemm, st) : r;
 }
 

@@ -36,7 +36,10 @@
 #include <mutex>
 #include <vector>
 #include <cuda_bf16.h>
-#include "sq_common.cuh"
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+#include "quant_codes.cuh"
 
 namespace sq {
 
@@ -47,6 +50,10 @@ extern std::atomic<int> g_tune_tile_n, g_tune_stages, g_tune_cta_group, g_tune_s
 template <int KIND, int NPOL>
 sq_status prepare_kind(const GemmArgs &g, GemmLaunch &L, int cg, int tile_n, bool seq, int device, int sm_count);
 
+// The same for the GEMM of few rows (gemm_rows.cuh); SQ_ERR_UNSUPPORTED where it does not take the layer, or is not expected to
+// take less than `limit` microseconds.
+template <int KIND, int NPOL>
+sq_status prepare_rows(const GemmArgs &g, GemmLaunch &L, double limit, int device, int sm_count);
 // Raises the kernel's dynamic shared-memory limit if need be; *clusters: how many CTA pairs can be resident (cg == 2).
 sq_status kernel_facts(int device, const void *kern, size_t smem, int cg, const cudaLaunchConfig_t &cfg, int *clusters);
 
@@ -81,6 +88,11 @@ constexpr int kTmemCols = 512;
 [[maybe_unused]] constexpr long long kWaitLimitCycles = 4000000000ll;   // about 2 s
 constexpr uint32_t kStageBytesPerWarp = 32 * 64;       // one 32 x 32 bf16 output block per epilogue warp
 [[maybe_unused]] constexpr uint32_t kStageBytes = kEpiWarps * kStageBytesPerWarp;
+// The GEMM of few rows is taken below this share of the expected time of the tile form (the models' margin; beyond 128 rows that
+// of the tile form is off by up to a quarter), for the GEMM alone or for a whole layer whose activations it quantizes itself
+// against a quantize kernel (1.9 us on a few rows) and the better of the two GEMMs.
+[[maybe_unused]] constexpr double kQuantizeLaunch = 1.9;
+[[maybe_unused]] inline double rows_gain(int64_t M) { return M > TILE_M ? 0.70 : 0.92; }
 constexpr int kMaxTokenSegments = 32;                  // per-token layers: channel scales of up to 32 K-segments (32 KiB at 256 columns) are staged per tile
 [[maybe_unused]] constexpr int kMaxFactorTable = 2048;                  // (K-segments x polarities) x N-segments factors in shared memory
 
@@ -1772,7 +1784,15 @@ sq_status prepare_tile(const GemmArgs &g, GemmLaunch &L, int tile_n, bool seq, i
     return SQ_ERR_UNSUPPORTED;
 }
 
+#include "gemm_rows.cuh"
+
 }  // namespace
+
+template <>
+sq_status prepare_rows<SQ_GEMM_KIND, SQ_GEMM_NPOL>(const GemmArgs &g, GemmLaunch &L, double limit, int device, int sm_count)
+{
+    return prepare_rows_t<SQ_GEMM_KIND, SQ_GEMM_NPOL>(g, L, limit, device, sm_count);
+}
 
 template <>
 sq_status prepare_kind<SQ_GEMM_KIND, SQ_GEMM_NPOL>(const GemmArgs &g, GemmLaunch &L, int cg, int tile_n, bool seq, int device,
@@ -1824,9 +1844,13 @@ sq_status kernel_facts(int device, const void *key, size_t smem, int cg, const c
 }
 
 extern template sq_status prepare_kind<0, 1>(const GemmArgs &, GemmLaunch &, int, int, bool, int, int);
+extern template sq_status prepare_rows<0, 1>(const GemmArgs &, GemmLaunch &, double, int, int);
 extern template sq_status prepare_kind<0, 2>(const GemmArgs &, GemmLaunch &, int, int, bool, int, int);
+extern template sq_status prepare_rows<0, 2>(const GemmArgs &, GemmLaunch &, double, int, int);
 extern template sq_status prepare_kind<1, 1>(const GemmArgs &, GemmLaunch &, int, int, bool, int, int);
+extern template sq_status prepare_rows<1, 1>(const GemmArgs &, GemmLaunch &, double, int, int);
 extern template sq_status prepare_kind<1, 2>(const GemmArgs &, GemmLaunch &, int, int, bool, int, int);
+extern template sq_status prepare_rows<1, 2>(const GemmArgs &, GemmLaunch &, double, int, int);
 
 static sq_status prepare_for(const GemmArgs &g, GemmLaunch &L, int npol, int cg, int tile_n, bool seq, int device, int sm_count)
 {
@@ -1835,6 +1859,14 @@ static sq_status prepare_for(const GemmArgs &g, GemmLaunch &L, int npol, int cg,
                          : prepare_kind<0, 1>(g, L, cg, tile_n, seq, device, sm_count);
     return npol == 2 ? prepare_kind<1, 2>(g, L, cg, tile_n, seq, device, sm_count)
                      : prepare_kind<1, 1>(g, L, cg, tile_n, seq, device, sm_count);
+}
+
+// Few rows: gemm_rows.cuh.  Nothing is decided by the process-wide tuning words unless they ask for this form.
+static sq_status prepare_few_rows(const GemmArgs &g, GemmLaunch &L, double limit, int device, int sm_count)
+{
+    if (g.code == SQ_CODE_INT8)
+        return g.a_neg ? prepare_rows<0, 2>(g, L, limit, device, sm_count) : prepare_rows<0, 1>(g, L, limit, device, sm_count);
+    return g.a_neg ? prepare_rows<1, 2>(g, L, limit, device, sm_count) : prepare_rows<1, 1>(g, L, limit, device, sm_count);
 }
 
 size_t gemm_split_scratch_bytes(int64_t M, int64_t N, int dual)
@@ -1853,6 +1885,104 @@ void set_gemm_tuning(int tile_n, int stages, int cta_group, int segment_mode)
     g_tune_stages.store(stages, std::memory_order_relaxed);
     g_tune_cta_group.store(cta_group, std::memory_order_relaxed);
     g_tune_seq.store(segment_mode, std::memory_order_relaxed);
+}
+
+// Tile of the other form of the kernel: CTAs that share it, columns (0: none fits), segments one after the other.
+struct TilePlan { int cg, tile_n; bool seq; };
+static TilePlan tile_plan(const GemmArgs &g, int npol, int sm_count)
+{
+    const int tune_tile_n = g_tune_tile_n.load(std::memory_order_relaxed);
+    const int tune_cta_group = g_tune_cta_group.load(std::memory_order_relaxed);
+    const int tune_seq = g_tune_seq.load(std::memory_order_relaxed);
+    const int nacc = g.sb.P * npol;
+
+    // CTA pairs whenever a tile has more than 128 rows to work on
+    int cg = g.M > TILE_M ? 2 : 1;
+    if (tune_cta_group == 1 || tune_cta_group == 2) cg = tune_cta_group;
+    if (sm_count < 2) cg = 1;
+
+    // More than one K-segment: segments go through TMEM one after the other (SEQ) unless the caller asks for
+    // all accumulators of a tile to stay resident, which needs 32 columns for each of them.
+    bool seq = g.sb.P > 1;
+    if (tune_seq == 1 && nacc * 32 <= kTmemCols) seq = false;
+    if (tune_seq == 2) seq = true;
+    if (seq) {
+        const int wide_n = npol == 1 ? 256 : 128;
+        int tile_n = wide_n;
+        // The tile of half the width, with four accumulator sets in flight, is the better one as long as it costs no
+        // further wave: its epilogue handles half the columns per segment.  (us, wide / narrow, K-segments of 64 codes:
+        // 1024 x 1536 -> 1536 on 24 / 48 of 74 CTA pairs 20.2 / 17.0; 8858 rows, 210 / 420 tiles, 55.4 / 83.9.)
+        const int64_t m_tiles = (g.M + TILE_M * cg - 1) / (TILE_M * cg), units = sm_count / cg;
+        auto waves = [&](int tn) { return (m_tiles * ((g.N + tn - 1) / tn) + units - 1) / units; };
+        if (waves(wide_n / 2) <= waves(wide_n)) tile_n = wide_n / 2;
+        if (tune_tile_n == wide_n || tune_tile_n == wide_n / 2) tile_n = tune_tile_n;
+        return {cg, tile_n, true};
+    }
+
+    // Tile width: the widest tile whose accumulators fit the 512 TMEM columns, unless half that width
+    // fills the machine so much better that it outweighs the narrower tile's higher operand traffic
+    // per MMA (weights 1 : 0.75; a double-buffered accumulator set counts 10 % extra).
+    int tile_max = 256;
+    while (tile_max * nacc > kTmemCols) tile_max >>= 1;
+    if (tile_max < 32) return {cg, 0, false};
+    int tile_n = tile_max;
+    if (tile_max >= 128) {
+        const int64_t units = sm_count / cg;
+        auto score = [&](int tn, double weight) {
+            const int64_t tiles = ((g.M + TILE_M * cg - 1) / (TILE_M * cg)) * ((g.N + tn - 1) / tn);
+            const int64_t waves = (tiles + units - 1) / units;
+            const double dbuf = (2 * tn * nacc <= kTmemCols) ? 1.1 : 1.0;
+            return weight * dbuf * double(tiles) / double(waves * units);
+        };
+        if (score(tile_max / 2, 0.75) > score(tile_max, 1.0)) tile_n = tile_max / 2;
+    }
+    // per-(token, channel) factors run in the checking variant, whose epilogue releases a full-TMEM accumulator set
+    // only at its end: keep two sets so that it overlaps the next tile's main loop
+    const bool pt_generic = g.col_scale && (g.y_dtype == SQ_F32 || g.acc_dump || g.code != SQ_CODE_INT8 || cg != 2 || g.sb.P > kMaxTokenSegments);
+    if (pt_generic && 2 * tile_n * nacc > kTmemCols && tile_n >= 64) tile_n >>= 1;
+    // One CTA per tile (M <= 128): the launch streams the weights, so the more SMs share in it the better; 64-column
+    // tiles as long as they cost no further wave.  (us, 64 / 128 columns: 8 x 1152 -> 6912 dual, 108 / 54 tiles, 5.3 / 6.0;
+    // 8 x 3072 -> 18432 dual, 288 / 144 tiles for 148 SMs, 15.4 / 13.5.)
+    if (cg == 1 && g.M <= TILE_M && g.sb.P == 1) {
+        auto waves = [&](int tn) { return (((g.N + tn - 1) / tn) + sm_count - 1) / sm_count; };
+        if (waves(64) <= waves(128)) tile_n = 64;
+    }
+    if (tune_tile_n >= 32 && tune_tile_n <= tile_max && (tune_tile_n & (tune_tile_n - 1)) == 0)
+        tile_n = tune_tile_n;
+    return {cg, tile_n, false};
+}
+
+// Microseconds that form takes on few rows, a model fitted to 110 layers (M 1 .. 300; nine in ten within 13 %); 0, so that it is
+// taken, for more than 128 rows in more than one wave of tiles: there it is busy and the model too coarse (470 x 6512 -> 15096
+// dual 74.3 us, 79.2 in the form of few rows).
+static double tile_form_cost(const GemmArgs &g, int npol, const TilePlan &t, int sm_count)
+{
+    if (t.tile_n < 32) return 1e9;
+    const int64_t m_tiles = (g.M + TILE_M * t.cg - 1) / (TILE_M * t.cg), units = sm_count / t.cg;
+    const double waves = double((m_tiles * ((g.N + t.tile_n - 1) / t.tile_n) + units - 1) / units);
+    if (g.M > TILE_M && waves > 1.0) return 0.0;
+    const double kblocks = double((g.K + 127) / 128), w = npol * t.tile_n / 256.0;
+    return 2.27 + std::max(0.234e-6 * double(g.N) * double(g.K), waves * kblocks * std::max(0.2347, 0.14 * w)) +
+           (t.seq ? waves * g.sb.P * (0.308 + 0.159 * w) : waves * g.sb.P * w * 0.905) + (t.cg == 2 ? 1.57 : 0.0);
+}
+
+constexpr int kFewRows = 512;          // rows up to which the GEMM of few rows is considered at all
+
+sq_status prepare_fused_layer(const GemmArgs &g, GemmLaunch *out)
+{
+    int dev = 0, sm_count = 0;
+    const int tune_seq = g_tune_seq.load(std::memory_order_relaxed);
+    const bool automatic = !tune_seq && !g_tune_tile_n.load(std::memory_order_relaxed) && !g_tune_cta_group.load(std::memory_order_relaxed) &&
+                           !g_tune_stages.load(std::memory_order_relaxed);
+    if (!(tune_seq == kSegmentModeRows || (automatic && g.M <= kFusedRows))) return SQ_ERR_UNSUPPORTED;
+    if (cudaGetDevice(&dev) != cudaSuccess) return SQ_ERR_CUDA;
+    if (cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sm_count <= 0)
+        return SQ_ERR_CUDA;
+    const int npol = g.a_neg ? 2 : 1;
+    const double other = automatic ? tile_form_cost(g, npol, tile_plan(g, npol, sm_count), sm_count) : 1e9;
+    if (other == 0.0) return SQ_ERR_UNSUPPORTED;
+    const double limit = automatic ? rows_gain(g.M) * (other + kQuantizeLaunch) : other;
+    return prepare_few_rows(g, *out, limit, dev, sm_count);
 }
 
 // Everything a GEMM launch needs that can be worked out ahead of it: tile plan, kernel instantiation, tensor
@@ -1878,67 +2008,20 @@ sq_status prepare_gemm(const GemmArgs &g, GemmLaunch *out)
     if (cudaGetDevice(&dev) != cudaSuccess) return SQ_ERR_CUDA;
     if (cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sm_count <= 0)
         return SQ_ERR_CUDA;
-    const int tune_tile_n = g_tune_tile_n.load(std::memory_order_relaxed);
-    const int tune_cta_group = g_tune_cta_group.load(std::memory_order_relaxed);
-    const int tune_seq = g_tune_seq.load(std::memory_order_relaxed);
-
-    // CTA pairs whenever a tile has more than 128 rows to work on
-    int cg = g.M > TILE_M ? 2 : 1;
-    if (tune_cta_group == 1 || tune_cta_group == 2) cg = tune_cta_group;
-    if (sm_count < 2) cg = 1;
-
-    // More than one K-segment: segments go through TMEM one after the other (SEQ) unless the caller asks for
-    // all accumulators of a tile to stay resident, which needs 32 columns for each of them.
-    bool seq = g.sb.P > 1;
-    if (tune_seq == 1 && prm.nacc * 32 <= kTmemCols) seq = false;
-    if (tune_seq == 2) seq = true;
+    L.few_rows = 0;
+    L.threads = kThreads;
     if (prm.nacc * g.sb.Q > kMaxFactorTable) return SQ_ERR_UNSUPPORTED;
-    if (seq) {
-        const int wide_n = npol == 1 ? 256 : 128;
-        int tile_n = wide_n;
-        // The tile of half the width, with four accumulator sets in flight, is the better one as long as it costs no
-        // further wave: its epilogue handles half the columns per segment.  (us, wide / narrow, K-segments of 64 codes:
-        // 1024 x 1536 -> 1536 on 24 / 48 of 74 CTA pairs 20.2 / 17.0; 8858 rows, 210 / 420 tiles, 55.4 / 83.9.)
-        const int64_t m_tiles = (g.M + TILE_M * cg - 1) / (TILE_M * cg), units = sm_count / cg;
-        auto waves = [&](int tn) { return (m_tiles * ((g.N + tn - 1) / tn) + units - 1) / units; };
-        if (waves(wide_n / 2) <= waves(wide_n)) tile_n = wide_n / 2;
-        if (tune_tile_n == wide_n || tune_tile_n == wide_n / 2) tile_n = tune_tile_n;
-        return prepare_for(g, L, npol, cg, tile_n, true, dev, sm_count);
+    const TilePlan t = tile_plan(g, npol, sm_count);
+    const int tune_seq = g_tune_seq.load(std::memory_order_relaxed);
+    const bool automatic = !tune_seq && !g_tune_tile_n.load(std::memory_order_relaxed) && !g_tune_cta_group.load(std::memory_order_relaxed);
+    if (tune_seq == kSegmentModeRows || (automatic && g.M <= kFewRows)) {
+        const double limit = automatic ? rows_gain(g.M) * tile_form_cost(g, npol, t, sm_count) : 1e9;
+        const sq_status fr = limit > 0.0 ? prepare_few_rows(g, L, limit, dev, sm_count) : SQ_ERR_UNSUPPORTED;
+        if (fr != SQ_ERR_UNSUPPORTED) return fr;
     }
-
-    // Tile width: the widest tile whose accumulators fit the 512 TMEM columns, unless half that width
-    // fills the machine so much better that it outweighs the narrower tile's higher operand traffic
-    // per MMA (weights 1 : 0.75; a double-buffered accumulator set counts 10 % extra).
-    int tile_max = 256;
-    while (tile_max * prm.nacc > kTmemCols) tile_max >>= 1;
-    if (tile_max < 32) return SQ_ERR_UNSUPPORTED;
-    int tile_n = tile_max;
-    if (tile_max >= 128) {
-        const int64_t units = sm_count / cg;
-        auto score = [&](int tn, double weight) {
-            const int64_t tiles = ((g.M + TILE_M * cg - 1) / (TILE_M * cg)) * ((g.N + tn - 1) / tn);
-            const int64_t waves = (tiles + units - 1) / units;
-            const double dbuf = (2 * tn * prm.nacc <= kTmemCols) ? 1.1 : 1.0;
-            return weight * dbuf * double(tiles) / double(waves * units);
-        };
-        if (score(tile_max / 2, 0.75) > score(tile_max, 1.0)) tile_n = tile_max / 2;
-    }
-    // per-(token, channel) factors run in the checking variant, whose epilogue releases a full-TMEM accumulator set
-    // only at its end: keep two sets so that it overlaps the next tile's main loop
-    const bool pt_generic = g.col_scale && (prm.y_is_f32 || prm.acc_dump || g.code != SQ_CODE_INT8 || cg != 2 || g.sb.P > kMaxTokenSegments);
-    if (pt_generic && 2 * tile_n * prm.nacc > kTmemCols && tile_n >= 64) tile_n >>= 1;
-    // One CTA per tile (M <= 128): the launch streams the weights, so the more SMs share in it the better; 64-column
-    // tiles as long as they cost no further wave.  (us, 64 / 128 columns: 8 x 1152 -> 6912 dual, 108 / 54 tiles, 5.3 / 6.0;
-    // 8 x 3072 -> 18432 dual, 288 / 144 tiles for 148 SMs, 15.4 / 13.5.)
-    if (cg == 1 && g.M <= TILE_M && g.sb.P == 1) {
-        auto waves = [&](int tn) { return (((g.N + tn - 1) / tn) + sm_count - 1) / sm_count; };
-        if (waves(64) <= waves(128)) tile_n = 64;
-    }
-    if (tune_tile_n >= 32 && tune_tile_n <= tile_max && (tune_tile_n & (tune_tile_n - 1)) == 0)
-        tile_n = tune_tile_n;
-    prm.acc_stages = (2 * tile_n * prm.nacc <= kTmemCols) ? 2 : 1;
-
-    return prepare_for(g, L, npol, cg, tile_n, false, dev, sm_count);
+    if (t.tile_n < 32) return SQ_ERR_UNSUPPORTED;
+    prm.acc_stages = (2 * t.tile_n * prm.nacc <= kTmemCols) ? 2 : 1;       // (one segment after the other: set by prepare_tile)
+    return prepare_for(g, L, npol, t.cg, t.tile_n, t.seq, dev, sm_count);
 }
 
 // One launch from a prepared plan: no queries, no encoding.
@@ -1946,7 +2029,7 @@ sq_status run_gemm(const GemmLaunch &L, cudaStream_t st)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(L.grid);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(L.threads);
     cfg.dynamicSmemBytes = L.smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -1956,10 +2039,11 @@ sq_status run_gemm(const GemmLaunch &L, cudaStream_t st)
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = L.cluster == 2 ? attr : attr + 1;          // the cluster attribute only for CTA pairs
-    cfg.numAttrs = L.cluster == 2 ? 2 : 1;
+    cfg.attrs = L.cluster > 1 ? attr : attr + 1;           // the cluster attribute only where there are clusters
+    cfg.numAttrs = L.cluster > 1 ? 2 : 1;
     void *args[5] = {const_cast<CUtensorMap *>(&L.ta), const_cast<CUtensorMap *>(&L.tn), const_cast<CUtensorMap *>(&L.tb),
                      const_cast<CUtensorMap *>(&L.ty), const_cast<KernelParams *>(&L.prm)};
+    if (L.few_rows) args[3] = const_cast<RowsParams *>(&L.rows);
     const cudaError_t e = cudaLaunchKernelExC(&cfg, L.kernel, args);
     count_launch();
     if (e != cudaSuccess) { note_cuda_error(e); return SQ_ERR_CUDA; }

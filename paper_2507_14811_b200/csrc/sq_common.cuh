@@ -123,6 +123,10 @@ struct GemmArgs {
     int64_t ldy;
     void *acc_dump;
     uint32_t *status;
+    const void *X;               // few rows: quantize these activations (then a_pos / a_neg are not read), or nullptr
+    sq_dtype x_dtype;
+    int64_t ldx;
+    int q_lo, q_hi;              // their code range
     void *sk_scratch;            // split tiles: zero-filled device scratch behind the workspace's fixed part, or nullptr
     size_t sk_bytes;
 };
@@ -149,16 +153,49 @@ struct KernelParams {
     int sk_kblocks;              // split tiles: K-blocks per tile (0: tiles are not split)
 };
 
+// Parameters of the GEMM of few rows (gemm_rows.cuh).
+struct RowsParams {
+    int M, N, K;
+    int tile_tokens, tile_rows;  // tokens (MMA columns per polarity) and output channels (MMA rows) of a tile
+    int ncols;                   // columns of one K-segment's accumulators: tokens padded x polarities
+    int num_m, num_n;            // tiles
+    int split;                   // CTAs (one cluster) that share the K range of a tile
+    int kblocks, stages;
+    int ahead;                   // K-blocks of a CTA's first tile fetched into L2 ahead of the dependency wait
+    int acc_sets, tmem_cols;
+    int rank_p0[8], rank_p1[8];  // first and last K-segment of a CTA's K range
+    uint32_t act_bytes, x_bytes, tab_bytes, red_bytes;    // shared memory: quantized activations, their inputs, factors, partial sums
+    uint32_t x_pitch;
+    int red_alias;               // the partial sums take the ring's place
+    SegBounds sb;
+    const float *s_pos, *s_neg, *s_w, *bias;
+    const float *row_pos, *row_neg, *col_scale;
+    void *Y;
+    long long ldy;
+    int y_is_f32;
+    void *acc_dump;
+    uint32_t *status;
+    const void *X;               // activations to quantize, or nullptr: code matrices
+    long long ldx;
+    int q_lo, q_hi;
+};
+constexpr int kSegmentModeRows = 8, kSegmentModeNoRows = 9;     // segquant_set_tuning
+
 // A GEMM launch worked out ahead of time: kernel instantiation, tensor maps, parameters, grid.
 struct GemmLaunch {
     CUtensorMap ta, tn, tb, ty;
     KernelParams prm;
+    RowsParams rows;             // few_rows: parameters of that kernel, with the maps ta, tn, tb
+    int few_rows;
     const void *kernel;
-    unsigned grid, cluster;
+    unsigned grid, cluster, threads;
     size_t smem;
     int device;
 };
 sq_status prepare_gemm(const GemmArgs &g, GemmLaunch *out);    // launches nothing
+// The whole layer in one launch from g.X, where the GEMM of few rows takes it and gains by that; SQ_ERR_UNSUPPORTED where not.
+constexpr int kFusedRows = 256;
+sq_status prepare_fused_layer(const GemmArgs &g, GemmLaunch *out);
 sq_status run_gemm(const GemmLaunch &l, cudaStream_t st);      // one launch, no queries
 sq_status launch_gemm(const GemmArgs &g, cudaStream_t st);     // prepare + run
 void set_gemm_tuning(int tile_n, int stages, int cta_group, int segment_mode);

@@ -1,0 +1,111 @@
+"""The GEMM of few rows (output channels on the MMA's rows, tokens on its columns, K ranges split over clusters, activations
+quantized inside): bit for bit the results of the tile form, which the parity tests hold to the oracle.  Both add the same
+terms in the same order: int8 sums are exact however a K range is split, e4m3 ones are never split."""
+import pytest
+import torch
+
+from paper_2507_14811_b200 import binding as B
+from paper_2507_14811_b200.layer import SegQuantLinear
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+BF16, F32 = torch.bfloat16, torch.float32
+TILE_FORM, ROWS_FORM = 9, 8
+
+
+def make(M, K, N, kb, nb, dual, code, x_dtype):
+    g = torch.Generator(device=DEV).manual_seed(M + K + N)
+    layer = SegQuantLinear(torch.randn((N, K), generator=g, device=DEV) * 0.02, torch.randn((N,), generator=g, device=DEV), kb, nb, dual, code)
+    X = torch.randn((M, K), generator=g, device=DEV).to(x_dtype)
+    layer.calibrate(X * 0.9)                             # the largest inputs are clipped
+    return layer, X
+
+
+def gemm(layer, codes, y_dtype, dump=False):
+    c_pos, c_neg = codes
+    if layer.dual:
+        return B.segquant_dualscale_gemm(c_pos, c_neg, layer.Wq, layer.seg, layer.code, layer.s_pos, layer.s_neg, layer.s_w,
+                                         layer.bias, layer.workspace, y_dtype=y_dtype, dump_acc=dump)
+    return B.segquant_seglinear_gemm(c_pos, layer.Wq, layer.seg, layer.code, layer.s_pos, layer.s_w, layer.bias, layer.workspace,
+                                     y_dtype=y_dtype, dump_acc=dump)
+
+
+@pytest.mark.parametrize("case", [
+    # M, K, N, kb, nb, x, y: one 16-code step; a K tail; one channel past a tile; every token count around 8 and 16; segments
+    # inside a K-block and across the cut of a split K range; more segments than CTAs; N-bounds anywhere; several token tiles
+    (1, 16, 8, [0, 16], [0, 8], BF16, BF16),
+    (7, 1040, 136, [0, 1040], [0, 136], F32, BF16),
+    (9, 2064, 264, [0, 32, 96, 1056, 2064], [0, 1, 130, 264], BF16, F32),
+    (17, 528, 1000, [0, 160, 528], [0, 328, 1000], F32, F32),
+    (40, 1152, 96, [0, 64, 128, 192, 256, 1024, 1152], [0, 96], BF16, BF16),
+    (128, 384, 72, [0, 384], [0, 40, 72], BF16, F32),
+    (250, 640, 392, [0, 320, 640], [0, 392], BF16, BF16),
+])
+@pytest.mark.parametrize("code,dual", [("int8", True), ("int8", False), ("e4m3", True), ("e4m3", False)])
+def test_every_shape_equals_the_tile_form(case, code, dual):
+    M, K, N, kb, nb, x_dtype, y_dtype = case
+    layer, X = make(M, K, N, kb, nb, dual, code, x_dtype)
+    codes = B.segquant_quantize_act(X, layer.seg, layer.s_pos, layer.s_neg, code)
+    try:
+        B.segquant_set_tuning(segment_mode=TILE_FORM)
+        ref, ref_acc = gemm(layer, codes, y_dtype, dump=True)
+        for rows, tokens, split in ((0, 0, 0), (128, 8, 1), (32, 16, 2), (64, 256, 4), (96, 32, 8), (128, 128, 1), (32, 8, 8)):
+            B.segquant_set_tuning(rows, tokens, split, ROWS_FORM)        # shapes that do not fit run the tile form
+            Y = torch.full((M + 1, N), 7.0, dtype=y_dtype, device=DEV)
+            layer.forward(X, Y[:M])                                      # quantized inside
+            y, acc = gemm(layer, codes, y_dtype, dump=True)
+            layer.check_status()
+            shape = (rows, tokens, split)
+            assert torch.equal(Y[:M], ref) and torch.equal(y, ref) and torch.equal(acc, ref_acc), shape
+            assert torch.equal(gemm(layer, codes, y_dtype), ref) and bool(torch.all(Y[M:] == 7.0)), shape
+    finally:
+        B.segquant_set_tuning()
+
+
+@pytest.mark.parametrize("dual", [True, False])
+@pytest.mark.parametrize("M,K,N,kb", [(1, 4096, 264, [0, 4096]), (5, 1056, 1000, [0, 96, 1056]), (100, 512, 136, [0, 512])])
+def test_per_token_scales(M, K, N, kb, dual):
+    P = len(kb) - 1
+    g = torch.Generator(device=DEV).manual_seed(5)
+    seg, ws = B.SegTable(kb, [0, N]), B.new_workspace(DEV)
+    s_pos, s_neg, c_pos, c_neg = B.segquant_quantize_per_row(torch.randn((M, K), generator=g, device=DEV), seg, dual)
+    s_w, _, w, _ = B.segquant_quantize_per_row(torch.randn((N, K), generator=g, device=DEV), seg, False, bits=4)
+    bias = torch.randn((N,), generator=g, device=DEV)
+    run = lambda: B.segquant_w4a8_gemm(c_pos, c_neg, w, seg, s_pos, s_neg, s_w, bias, ws, y_dtype=F32)
+    try:
+        B.segquant_set_tuning(segment_mode=TILE_FORM)
+        ref = run()
+        for shape in ((0, 0, 0), (32, 8, 1), (128, 32, 8), (64, 16, 2)):
+            B.segquant_set_tuning(*shape, ROWS_FORM)
+            assert torch.equal(run(), ref), shape
+    finally:
+        B.segquant_set_tuning()
+    B.check_device_status(ws)
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -90, 2.0 ** 105])
+@pytest.mark.parametrize("code,dual", [("int8", True), ("int8", False), ("e4m3", True)])
+def test_scales_outside_the_fast_quantizer(scale, code, dual):
+    layer, X = make(6, 288, 40, [0, 288], [0, 40], dual, code, F32)
+    X = X * scale
+    layer.calibrate(X)
+    outs = []
+    try:
+        for mode in (TILE_FORM, ROWS_FORM):
+            B.segquant_set_tuning(segment_mode=mode)
+            outs.append(layer.forward(X, y_dtype=F32))
+    finally:
+        B.segquant_set_tuning()
+    assert torch.equal(*outs)
+
+
+def test_output_in_place_of_the_input():
+    """X is read before Y is written wherever the two share memory."""
+    layer, X = make(24, 256, 256, [0, 256], [0, 256], True, "int8", F32)
+    ref = layer.forward(X, y_dtype=F32)
+    n = B.segquant_launch_count()
+    layer.forward(X.clone(), y_dtype=F32)
+    assert B.segquant_launch_count() == n + 1                            # apart, this layer is one launch
+    Y = X.clone()
+    layer.forward(Y, Y)
+    assert torch.equal(Y, ref)
