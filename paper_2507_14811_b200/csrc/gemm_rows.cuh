@@ -18,10 +18,10 @@
 // has: one would wait for the other, and with clusters round in a circle.  Hence smem_for_columns: shared memory grows with
 // the columns so that what fits in shared memory fits in tensor memory, too.
 // Measured against the tile form, which takes one CTA per 64 or 128 output columns (us, tile form / here, device time in a graph
-// over rotating buffers; GEMM alone): 1 x 10912 -> 2320 dual int8 23.0 / 10.9, 9 x 6720 -> 1336 three segments 15.5 / 8.6,
-// 54 x 6688 -> 504 eleven segments 19.7 / 9.7, 283 x 9248 -> 384 24.2 / 11.0, 8 x 3072 -> 18432 dual e4m3 13.5 / 11.9 (weights at copy
-// bandwidth 8.8); whole layers, where the quantizer's launch goes as well: 8 x 3072 -> 18432 15.9 / 14.2, 256 x 256 -> 768 5.9 / 4.7.
-// 120 random layers of 1 .. 128 rows: GEMM 0.81 of its time, layer 0.865.
+// over rotating buffers; GEMM alone): 1 x 10912 -> 2320 dual int8 23.0 / 9.2, 9 x 6720 -> 1336 three segments 15.5 / 8.2,
+// 283 x 9248 -> 384 24.2 / 10, 1 x 4672 -> 288 dual e4m3 11.4 / 7.5; whole layers, where the quantizer's launch goes as well (a
+// call): 8 x 3072 -> 18432 dual e4m3 18.1 / 12.2 (weights at copy bandwidth 8.8), 256 x 256 -> 768 7.7 / 5.3.  120 random layers of 1 .. 128
+// rows: GEMM 0.79, layer 0.79 of its time.
 
 constexpr int kRowsWarps = 8;                          // quantizer / epilogue
 constexpr int kRowsThreads = (kRowsWarps + 2) * 32;
@@ -70,7 +70,8 @@ segquant_rows_kernel(const __grid_constant__ CUtensorMap tm_pos, const __grid_co
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t w_bytes = uint32_t(prm.tile_rows) * BLOCK_K, act_block = uint32_t(prm.ncols) * BLOCK_K;
-    const uint32_t stage_bytes = w_bytes + (SRC == 0 ? act_block : 0u);
+    const uint32_t block_bytes = w_bytes + (SRC == 0 ? act_block : 0u), stage_bytes = uint32_t(prm.stage_blocks) * block_bytes;
+    const int stage_blocks = prm.stage_blocks;
     // [ring] [(SRC != 0) codes of the tokens' K range] [(SRC != 0) their inputs] [factors] [partial sums of the cluster] [header]
     const uint32_t ring0 = smem_u32(smem);
     const uint32_t act0 = ring0 + uint32_t(prm.stages) * stage_bytes;
@@ -154,18 +155,23 @@ segquant_rows_kernel(const __grid_constant__ CUtensorMap tm_pos, const __grid_co
         }
         uint32_t s = 0, ph = 0, issued = 0;
         for (int nt = unit / prm.num_m; nt < prm.num_n && ok; nt += units / prm.num_m) {
-            for (int kb = kb0; kb < kb1; kb++) {
+            for (int kb = kb0; kb < kb1; kb += stage_blocks) {
                 if (!mbar_wait_warp(empty0 + 8 * s, ph ^ 1, abort_flag, prm.status, kWhereRowsProducer)) {
                     ok = false;
                     break;
                 }
-                const uint32_t dst = ring0 + s * stage_bytes, bar = full0 + 8 * s;
+                const uint32_t bar = full0 + 8 * s;
+                const int blocks = min(stage_blocks, kb1 - kb);
                 if (elect_one()) {
-                    mbar_expect_tx(bar, stage_bytes);
-                    tma_load_2d<1>(dst, &tm_w, bar, kb * BLOCK_K, nt * prm.tile_rows);
-                    if (SRC == 0) {
-                        tma_load_2d<1>(dst + w_bytes, &tm_pos, bar, kb * BLOCK_K, m0);
-                        if (NPOL == 2) tma_load_2d<1>(dst + w_bytes + act_block / 2, &tm_neg, bar, kb * BLOCK_K, m0);
+                    mbar_expect_tx(bar, uint32_t(blocks) * block_bytes);
+                    for (int b = 0; b < blocks; b++) {
+                        const uint32_t dst = ring0 + s * stage_bytes + uint32_t(b) * block_bytes;
+                        const int k = (kb + b) * BLOCK_K;
+                        tma_load_2d<1>(dst, &tm_w, bar, k, nt * prm.tile_rows);
+                        if (SRC == 0) {
+                            tma_load_2d<1>(dst + w_bytes, &tm_pos, bar, k, m0);
+                            if (NPOL == 2) tma_load_2d<1>(dst + w_bytes + act_block / 2, &tm_neg, bar, k, m0);
+                        }
                     }
                 }
                 __syncwarp();
@@ -193,44 +199,58 @@ segquant_rows_kernel(const __grid_constant__ CUtensorMap tm_pos, const __grid_co
         const uint64_t w_desc0 = make_smem_desc(ring0), act_desc0 = make_smem_desc(SRC == 0 ? ring0 + w_bytes : act0);
         const uint32_t hi = uint32_t(w_desc0 >> 32);
         uint32_t s = 0, ph = 0, as = 0, aph = 0;
-        int act_groups = 0;                                        // groups of activations known to be there
+        int act_groups = 0, act_have = 0;                          // groups and chunks of activations known to be there
         for (int nt = unit / prm.num_m; nt < prm.num_n && ok; nt += units / prm.num_m) {
             if (!mbar_wait_warp(acc_empty0 + 8 * as, aph ^ 1, abort_flag, prm.status, kWhereRowsAcc)) {
                 ok = false;
                 break;
             }
             tc_fence_after();
-            int p = p_first;
+            int p = p_first, k_end = prm.sb.kb[p + 1];
             uint32_t accumulate = 0, d = tmem_base + as * set_cols;
-            for (int kb = kb0; kb < kb1; kb++) {
+            for (int kb = kb0; kb < kb1; kb += stage_blocks) {
                 if (!mbar_wait_warp(full0 + 8 * s, ph, abort_flag, prm.status, kWhereRowsFull)) {
                     ok = false;
                     break;
                 }
+                const int blocks = min(stage_blocks, kb1 - kb);
                 if (SRC != 0) {
-                    const int need = min((kb - kb0 + 1) * rows * 8 - 1, act_chunks - 1) / act_group + 1;
-                    while (act_groups < need && ok)
+                    const int need = (kb + blocks - kb0) * per_block;
+                    while (act_have < need && ok) {
                         ok = mbar_wait_warp(smem_u32(&hdr->act_ready[act_groups++]), 0, abort_flag, prm.status, kWhereRowsAct);
+                        act_have += act_group;
+                    }
                     if (!ok) break;
                 }
                 tc_fence_after();
-                const uint32_t a_lo = uint32_t(w_desc0) + s * (stage_bytes >> 4);
-                const uint32_t b_lo = uint32_t(act_desc0) + (SRC == 0 ? s * (stage_bytes >> 4) : uint32_t(kb - kb0) * (act_block >> 4));
-                const int k = kb * BLOCK_K;
-                if (k + BLOCK_K <= prm.sb.kb[p + 1]) {             // the whole block lies in one K-segment
-                    if (elect_one()) issue_full_kblock<KIND, 1>(d, a_lo, b_lo, hi, idesc, accumulate);
-                    accumulate = 1;
-                } else {                                           // K-steps lie in one segment each (bounds are multiples of 32)
-                    for (int kk = k; kk < min(k + BLOCK_K, prm.K); kk += MMA_K) {
-                        if (kk >= prm.sb.kb[p + 1]) { p++; d += prm.ncols; accumulate = 0; }
-                        const uint32_t off = uint32_t(kk - k) >> 4;
-                        if (elect_one())
-                            tc_mma<KIND, 1>(d, uint64_t(hi) << 32 | (a_lo + off), uint64_t(hi) << 32 | (b_lo + off), idesc, accumulate);
-                        accumulate = 1;
+                uint32_t a_lo = uint32_t(w_desc0) + s * (stage_bytes >> 4);
+                uint32_t b_lo = uint32_t(act_desc0) + (SRC == 0 ? s * (stage_bytes >> 4) : uint32_t(kb - kb0) * (act_block >> 4));
+                int k = kb * BLOCK_K;
+                const uint32_t b_step = (SRC == 0 ? block_bytes : act_block) >> 4;
+                if (k + blocks * BLOCK_K <= k_end) {               // whole blocks of one K-segment
+                    if (elect_one()) {
+#pragma unroll 1
+                        for (int b = 0; b < blocks; b++, a_lo += block_bytes >> 4, b_lo += b_step) {
+                            issue_full_kblock<KIND, 1>(d, a_lo, b_lo, hi, idesc, accumulate);
+                            accumulate = 1;
+                        }
+                        tc_commit<1>(empty0 + 8 * s);
                     }
+                    accumulate = 1;
+                    k += blocks * BLOCK_K;
+                } else {                                           // K-steps lie in one segment each (bounds are multiples of 32)
+                    for (int b = 0; b < blocks; b++, a_lo += block_bytes >> 4, b_lo += b_step) {
+                        const int stop = min(k + BLOCK_K, prm.K);
+                        for (uint32_t off = 0; k < stop; k += MMA_K, off += MMA_K >> 4) {
+                            if (k >= k_end) { k_end = prm.sb.kb[++p + 1]; d += prm.ncols; accumulate = 0; }
+                            if (elect_one())
+                                tc_mma<KIND, 1>(d, uint64_t(hi) << 32 | (a_lo + off), uint64_t(hi) << 32 | (b_lo + off), idesc, accumulate);
+                            accumulate = 1;
+                        }
+                    }
+                    if (elect_one()) tc_commit<1>(empty0 + 8 * s);
                 }
-                if (k + BLOCK_K == prm.sb.kb[p + 1] && p < p_last) { p++; d += prm.ncols; accumulate = 0; }
-                if (elect_one()) tc_commit<1>(empty0 + 8 * s);
+                if (k >= k_end && p < p_last) { k_end = prm.sb.kb[++p + 1]; d += prm.ncols; accumulate = 0; }
                 if (++s == uint32_t(prm.stages)) { s = 0; ph ^= 1; }
             }
             if (ok && elect_one()) tc_commit<1>(acc_full0 + 8 * as);
@@ -545,31 +565,43 @@ bool rows_layout(const GemmArgs &g, const RowsShape &sh, int sm_count, RowsParam
     r.x_bytes = (r.x_pitch * r.tile_tokens + 127u) & ~127u;
     r.red_bytes = split > 1 ? uint32_t(pieces * NPOL * ((r.tile_tokens + split - 1) / split) * r.tile_rows) * 4u : 0u;
     r.red_alias = r.red_bytes > 16 * 1024;
-    const size_t stage = size_t(r.tile_rows) * BLOCK_K + (fused ? 0u : act_block);
-    const size_t fixed = 1024 + r.act_bytes + r.x_bytes + r.tab_bytes + (r.red_alias ? 0u : r.red_bytes) + sizeof(RowsHeader);
-    // two CTAs per SM where that leaves a ring of four stages; the last stage is followed by what an MMA reads behind a tile of
-    // fewer than 128 rows
-    auto stages_in = [&](size_t budget) -> int {
-        if (fixed + 2 * stage > budget) return 0;
-        return int(std::min<size_t>((budget - fixed) / stage, kRowsStages));
+    const size_t block = size_t(r.tile_rows) * BLOCK_K + (fused ? 0u : act_block);
+    // behind the ring: what follows, and at least what an MMA reads behind a tile of fewer than 128 rows
+    const size_t fixed = 1024 + std::max<size_t>(r.act_bytes + r.x_bytes + r.tab_bytes + (r.red_alias ? 0u : r.red_bytes) + sizeof(RowsHeader),
+                                                 size_t(TILE_M - r.tile_rows) * BLOCK_K);
+    // K-blocks per ring stage: a wait, an election and a commit per stage cost the issuing loop some 75 ns (ns per block with 1, 2 and
+    // 4 blocks a stage: 233, 146, 115); as many as the length of the K range and three stages allow.  Two CTAs per SM where three
+    // stages fit half of its shared memory.
+    auto ring = [&](size_t budget) {
+        for (r.stage_blocks = longest >= 16 ? 4 : longest >= 4 ? 2 : 1; r.stage_blocks > 0; r.stage_blocks /= 2) {
+            const int turns = (longest + r.stage_blocks - 1) / r.stage_blocks;
+            const size_t stage = r.stage_blocks * block;
+            r.stages = fixed + 2 * stage > budget ? 0 : int(std::min<size_t>((budget - fixed) / stage, kRowsStages));
+            if (r.stages >= std::min(3, turns)) return turns;
+        }
+        return 0;
     };
     constexpr size_t kTwo = 113 * 1024, kOne = kSmemBudget;
-    int per_sm = 2;
-    r.stages = stages_in(kTwo);
-    if (r.stages < std::min(4, longest)) { r.stages = stages_in(kOne); per_sm = 1; }
-    if (r.stages < 2) return false;
+    int per_sm = 2, turns = ring(kTwo);
+    if (!turns) { turns = ring(kOne); per_sm = 1; }
+    if (!turns) return false;
     const int64_t slots = int64_t(sm_count) * per_sm / split;
     if (slots < 1) return false;
     const int64_t per_m = split > 1 ? r.num_n : std::min<int64_t>(r.num_n, std::max<int64_t>(1, slots / r.num_m));
     *grid = unsigned(per_m * r.num_m * split);
     const int tiles_per_cta = int((r.num_n + per_m - 1) / per_m);
-    if (tiles_per_cta == 1 && r.stages > longest) r.stages = std::max(2, longest);
+    if (per_sm == 2 && int(*grid) <= sm_count && turns * tiles_per_cta > r.stages) {
+        // a CTA per SM and more blocks than that ring holds: a deeper one counts for more than the next launch's early start
+        turns = ring(kOne);
+        per_sm = 1;
+    }
+    const size_t stage = r.stage_blocks * block;
+    if (tiles_per_cta == 1 && r.stages > turns) r.stages = std::max(2, turns);
     if (r.red_alias && r.red_bytes > r.stages * stage + r.act_bytes + r.x_bytes) return false;
     r.acc_sets = tiles_per_cta > 1 && 2 * most * r.ncols <= kTmemCols / per_sm ? 2 : 1;
     r.tmem_cols = 32;
     while (r.tmem_cols < r.acc_sets * most * r.ncols) r.tmem_cols *= 2;
-    const size_t behind = (r.stages - 1) * stage + size_t(TILE_M) * BLOCK_K;         // what the last stage's MMAs may read
-    *smem = std::max(std::max(r.stages * stage + fixed, 1024 + behind), smem_for_columns(r.tmem_cols));
+    *smem = std::max(r.stages * stage + fixed, smem_for_columns(r.tmem_cols));
     if (*smem > kOne) return false;
 
     // microseconds, a model fitted to some 5000 timings of forced shapes (M 1 .. 300, K 256 .. 12288, N 256 .. 18432, up to 24
@@ -581,12 +613,15 @@ bool rows_layout(const GemmArgs &g, const RowsShape &sh, int sm_count, RowsParam
     const int resident = std::min(int(*grid), capacity), waves = (int(*grid) + capacity - 1) / capacity;
     const double per_sm_now = (resident + sm_count - 1) / sm_count, blocks = double(waves) * tiles_per_cta * longest;
     const double bytes = double(r.tile_rows + (fused ? 0 : r.ncols)) * BLOCK_K, g16 = (r.tile_tokens + 15) / 16;
-    const double block = std::max(std::max(0.2442, 0.4505e-3 * 4.0 * std::max(32.0, r.ncols / 2.0) * per_sm_now), 6.3e-6 * bytes * per_sm_now);
-    const double stream = std::max(std::max(0.1776e-6 * double(g.N) * double(g.K), blocks * block), 0.0457e-6 * resident * blocks * bytes);
-    const double quant = fused ? (KIND == 0 ? 0.58 : 1.2) + (KIND == 0 ? 0.51 : 0.6) * ((r.tile_tokens * longest * 8 + 255) / 256) * (per_sm_now > 1 ? 1.62 : 1.0) : 0.0;
-    const double epi = 0.12 * most * NPOL * g16 * (per_sm_now > 1 ? 1.41 : 1.0) + 0.21 * g16;
-    const double comb = split > 1 ? 0.93 + 0.128 * pieces * NPOL * (((r.tile_tokens + split - 1) / split + 7) / 8) + 0.074 * most * NPOL * g16 : 0.0;
-    *cost = 2.39 + stream + waves * (quant + tiles_per_cta * epi + comb) + (waves - 1) * 2.7;
+    const double busy = per_sm_now > 1 ? 1.62 : 1.0, busy_half = per_sm_now > 1 ? 1.41 : 1.0;        // two CTAs on an SM
+    const double quant = fused ? (KIND == 0 ? 0.31 : 0.49) + 0.4675 * ((r.tile_tokens * longest * 8 + 255) / 256) * busy : 0.0;
+    const double per_block = std::max((r.stage_blocks == 4 ? 0.133 : r.stage_blocks == 2 ? 0.164 : 0.262) + 1.75e-4 * r.ncols * per_sm_now,
+                                      6.8e-6 * bytes * per_sm_now);
+    const double chain = blocks * per_block + waves * quant, memory = 0.183e-6 * double(g.N) * double(g.K) + (fused ? 0.27 : 0.0);
+    const double stream = std::max(std::max(memory, chain), 0.04e-6 * resident * blocks * bytes + quant);
+    const double epi = 0.148 * most * NPOL * g16 * busy_half + 0.157 * g16;
+    const double comb = split > 1 ? 0.894 + 0.129 * pieces * NPOL * (((r.tile_tokens + split - 1) / split + 7) / 8) + 0.082 * most * NPOL * g16 : 0.0;
+    *cost = 2.64 + stream + waves * (tiles_per_cta * epi + comb) + (waves - 1) * 2.95;
     r.ahead = int(std::min<double>(longest, std::max(0.0, std::ceil(kRowsAheadBytes / (double(*grid) * r.tile_rows * BLOCK_K)))));
     return true;
 }
@@ -661,7 +696,7 @@ sq_status prepare_rows_t(const GemmArgs &g, GemmLaunch &L, double limit, int dev
         GemmArgs codes = g;
         codes.X = nullptr;
         double apart = 0.0;
-        if (rows_plan<KIND, NPOL>(codes, sm_count, &shape, &apart) && cost >= rows_gain(g.M) * (apart + kQuantizeLaunch)) return SQ_ERR_UNSUPPORTED;
+        if (rows_plan<KIND, NPOL>(codes, sm_count, &shape, &apart) && cost >= rows_gain(g.M, g.K, true) * (apart + kQuantizeLaunch)) return SQ_ERR_UNSUPPORTED;
         rows_plan<KIND, NPOL>(g, sm_count, &shape, &cost);
     }
     rows_layout<KIND, NPOL>(g, shape, sm_count, &r, &L.smem, &L.grid, &cost);

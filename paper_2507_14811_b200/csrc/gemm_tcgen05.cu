@@ -92,7 +92,7 @@ constexpr uint32_t kStageBytesPerWarp = 32 * 64;       // one 32 x 32 bf16 outpu
 // of the tile form is off by up to a quarter), for the GEMM alone or for a whole layer whose activations it quantizes itself
 // against a quantize kernel (1.9 us on a few rows) and the better of the two GEMMs.
 [[maybe_unused]] constexpr double kQuantizeLaunch = 1.9;
-[[maybe_unused]] inline double rows_gain(int64_t M) { return M > TILE_M ? 0.70 : 0.92; }
+[[maybe_unused]] inline double rows_gain(int64_t M, int64_t K, bool fused) { return M <= TILE_M ? 0.92 : fused && K <= 512 ? 0.80 : 0.70; }
 constexpr int kMaxTokenSegments = 32;                  // per-token layers: channel scales of up to 32 K-segments (32 KiB at 256 columns) are staged per tile
 [[maybe_unused]] constexpr int kMaxFactorTable = 2048;                  // (K-segments x polarities) x N-segments factors in shared memory
 
@@ -1981,7 +1981,7 @@ sq_status prepare_fused_layer(const GemmArgs &g, GemmLaunch *out)
     const int npol = g.a_neg ? 2 : 1;
     const double other = automatic ? tile_form_cost(g, npol, tile_plan(g, npol, sm_count), sm_count) : 1e9;
     if (other == 0.0) return SQ_ERR_UNSUPPORTED;
-    const double limit = automatic ? rows_gain(g.M) * (other + kQuantizeLaunch) : other;
+    const double limit = automatic ? rows_gain(g.M, g.K, true) * (other + kQuantizeLaunch) : other;
     return prepare_few_rows(g, *out, limit, dev, sm_count);
 }
 
@@ -2015,7 +2015,7 @@ sq_status prepare_gemm(const GemmArgs &g, GemmLaunch *out)
     const int tune_seq = g_tune_seq.load(std::memory_order_relaxed);
     const bool automatic = !tune_seq && !g_tune_tile_n.load(std::memory_order_relaxed) && !g_tune_cta_group.load(std::memory_order_relaxed);
     if (tune_seq == kSegmentModeRows || (automatic && g.M <= kFewRows)) {
-        const double limit = automatic ? rows_gain(g.M) * tile_form_cost(g, npol, t, sm_count) : 1e9;
+        const double limit = automatic ? rows_gain(g.M, g.K, false) * tile_form_cost(g, npol, t, sm_count) : 1e9;
         const sq_status fr = limit > 0.0 ? prepare_few_rows(g, L, limit, dev, sm_count) : SQ_ERR_UNSUPPORTED;
         if (fr != SQ_ERR_UNSUPPORTED) return fr;
     }

@@ -160,7 +160,8 @@ struct RowsParams {
     int ncols;                   // columns of one K-segment's accumulators: tokens padded x polarities
     int num_m, num_n;            // tiles
     int split;                   // CTAs (one cluster) that share the K range of a tile
-    int kblocks, stages;
+    int kblocks;
+    int stages, stage_blocks;    // ring: stages of so many K-blocks
     int ahead;                   // K-blocks of a CTA's first tile fetched into L2 ahead of the dependency wait
     int acc_sets, tmem_cols;
     int rank_p0[8], rank_p1[8];  // first and last K-segment of a CTA's K range
