@@ -334,10 +334,11 @@ sq_status segquant_last_device_status(void *workspace, void *stream, uint32_t *d
 sq_status segquant_set_tuning(int tile_n, int stages, int cta_group, int segment_mode);
 
 /* The fused activation of segquant_quantize_act_fused has two implementations with identical results: one that
- * evaluates SiLU / GELU per element, and, for bf16 inputs, one that looks the stored activation up in a table of
- * all 65536 bf16 values which every thread block builds in shared memory first (about 9 us per launch, then one
- * load per element).  fused_table_mode: 0 automatic (the table from 9 Mi elements up for GELU and 20 Mi
- * for SiLU with dual codes, from 10 Mi and 30 Mi with single-scale ones), 1 the table wherever it applies, 2 never.  Process-wide and for tests and sweeps, like segquant_set_tuning. */
+ * evaluates SiLU / GELU per element, and, for bf16 inputs, one that looks up a table which every thread block builds in
+ * shared memory first: SiLU the stored activation of all 65536 bf16 values (about 9 us per launch), GELU and gated GELU the
+ * 3841 values of erfc(|h| / sqrt 2) that differ (about 1 us).  fused_table_mode: 0 automatic (from 20 Mi elements up for SiLU with dual
+ * codes and 30 Mi with single-scale ones, from 0.5 Mi for GELU, 10 and 12 Mi for gated GELU), 1 the table wherever it
+ * applies, 2 never.  Process-wide and for tests and sweeps, like segquant_set_tuning. */
 sq_status segquant_set_quantize_tuning(int fused_table_mode);
 
 /* Text of the CUDA error behind the most recent SQ_ERR_CUDA of a GEMM launch ("no error" if none). */

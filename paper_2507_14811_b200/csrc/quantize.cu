@@ -66,9 +66,9 @@ __device__ __forceinline__ uint64_t silu2(float h0, float h1)
     unpack2(mul2(pack2(h0, h1), pack2(z0, z1)), n0, n1);
     return mul2(pack2(h0 >= 0.0f ? h0 : n0, h1 >= 0.0f ? h1 : n1), pack2(rcp_approx(d0), rcp_approx(d1)));
 }
-__device__ __forceinline__ uint64_t gelu2(float h0, float h1)
+// erfc(a / sqrt 2) for 0 <= a <= 20
+__device__ __forceinline__ uint64_t gelu_tail2(uint64_t a)
 {
-    const uint64_t a = pack2(fminf(fabsf(h0), 20.0f), fminf(fabsf(h1), 20.0f));
     const uint64_t t = mul2(a, dup2(0.70710678118654752440f));
     float d0, d1;
     unpack2(add2(t, dup2(2.5f)), d0, d1);
@@ -86,13 +86,21 @@ __device__ __forceinline__ uint64_t gelu2(float h0, float h1)
     const uint64_t neg_e = fma2(mul2(t, dup2(-1.0f)), t, s);      // t^2 = s - neg_e exactly
     float x0, x1;
     unpack2(mul2(s, dup2(-1.4426950408889634f)), x0, x1);
-    uint64_t E = mul2(pack2(ex2_approx(x0), ex2_approx(x1)), g);
-    E = fma2(E, neg_e, E);                                        // exp(-(s + e)) = exp(-s) (1 - e) to first order
+    const uint64_t E = mul2(pack2(ex2_approx(x0), ex2_approx(x1)), g);
+    return fma2(E, neg_e, E);                                     // exp(-(s + e)) = exp(-s) (1 - e) to first order
+}
+__device__ __forceinline__ uint64_t gelu_from_tail2(float h0, float h1, uint64_t a, uint64_t E)
+{
     return fma2(mul2(a, dup2(-0.5f)), E, pack2(fmaxf(h0, 0.0f), fmaxf(h1, 0.0f)));
 }
-// two activations as the unfused graph would have stored them, times the per-channel multipliers (one fp32 multiply)
+__device__ __forceinline__ uint64_t gelu2(float h0, float h1)
+{
+    const uint64_t a = pack2(fminf(fabsf(h0), 20.0f), fminf(fabsf(h1), 20.0f));
+    return gelu_from_tail2(h0, h1, a, gelu_tail2(a));
+}
+// two activations as the unfused graph would have stored them
 template <typename Tin>
-__device__ __forceinline__ uint64_t stored2(uint64_t a, uint64_t mult)
+__device__ __forceinline__ uint64_t rounded2(uint64_t a)
 {
     if (sizeof(Tin) == 2) {
         float a0, a1;
@@ -101,8 +109,11 @@ __device__ __forceinline__ uint64_t stored2(uint64_t a, uint64_t mult)
         const uint32_t w = *reinterpret_cast<const uint32_t *>(&r);
         a = pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
     }
-    return mul2(a, mult);
+    return a;
 }
+// times the per-channel multipliers (one fp32 multiply)
+template <typename Tin>
+__device__ __forceinline__ uint64_t stored2(uint64_t a, uint64_t mult) { return mul2(rounded2<Tin>(a), mult); }
 template <typename Tin>
 __device__ __forceinline__ uint64_t pre2(float h0, float h1, int act, uint64_t mult)
 {
@@ -317,14 +328,13 @@ quantize_kernel(const __grid_constant__ QuantParams prm)
     asm volatile("cp.async.wait_group 0;" ::: "memory");     // nothing of this thread's is in flight when it leaves
 }
 
-// ----------------------------------------------------------------------------- fused activation by table (bf16 inputs)
-// A bf16 pre-activation has 65536 possible values, so the stored activation bf16(act(h)) is a table of 128 KiB.
-// Every CTA (1024 threads, one per SM) builds the table in its shared memory with the same silu2 / gelu2 as
+// ----------------------------------------------------------------------------- fused SiLU by table (bf16 inputs)
+// A bf16 pre-activation has 65536 possible values, so the stored activation bf16(silu(h)) is a table of 128 KiB.
+// Every CTA (1024 threads, one per SM) builds the table in its shared memory with the same silu2 as
 // the arithmetic variant (a few evaluations per thread: most bit patterns need none), after which an element costs one
 // shared-memory load instead of about 30 instructions: the fused pass stops being bound by the ALUs.  Results are
 // those of the arithmetic variant bit for bit.  Used for large inputs: a launch of this kernel costs about 9 us
 // more than the other's (the table, and a CTA that fills the SM cannot start under the previous kernel's tail).
-// (Not for the gated form: its product is rounded once, from the unrounded GELU, which a bf16 table does not hold.)
 // The rest is quantize_kernel's scheme: thread g owns column chunk g % V of rows g / V, g / V + R, ...; the rows
 // travel through a thread-private ring of kTableDepth slots behind the table.
 constexpr int kTableThreads = 1024;
@@ -334,34 +344,31 @@ constexpr size_t kTableSmem = kTableBytes + size_t(kTableDepth) * 2 * kTableThre
 
 template <int CODE, int MODE>
 __global__ void __launch_bounds__(kTableThreads, 1)
-quantize_table_kernel(const __grid_constant__ QuantParams prm)
+quantize_silu_table_kernel(const __grid_constant__ QuantParams prm)
 {
     constexpr bool DUAL = MODE == kDual;
     extern __shared__ __align__(16) uint8_t table_smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t tab0 = uint32_t(__cvta_generic_to_shared(table_smem));
-    // Most bit patterns need no evaluation, because silu2 / gelu2 return a value known in advance there
+    // Most bit patterns need no evaluation, because silu2 returns a value known in advance there
     // (a warp's 32 consecutive patterns share sign and exponent, so the branch is uniform):
-    //   2^-124 <= |h| < 2^-26: both give h / 2 after the rounding to bf16 (the sigmoid / Phi factor is 1/2 to
-    //                          far below a bf16 half-step);
-    //   h >= 32 (SiLU), h >= 16 (GELU): h itself (exp(-h), erfc(h / sqrt 2) are below fp32's resolution of 1);
-    //   h <= -128 (SiLU), h <= -16 (GELU): -0 and +0 (the exponential has underflowed to zero).
-    // NaN and infinities go through the functions.  A test compares the codes of this variant with those of the arithmetic
+    //   2^-124 <= |h| < 2^-26: h / 2 after the rounding to bf16 (the sigmoid is 1/2 to far below a bf16 half-step);
+    //   h >= 32: h itself (exp(-h) is below fp32's resolution of 1);  h <= -128: -0 (the exponential has underflowed to zero).
+    // NaN and infinities go through the function.  A test compares the codes of this variant with those of the arithmetic
     // one on all 65536 patterns (the sign of a zero does not show in a code).
-    const bool is_silu = prm.act == 1;
     for (uint32_t b = threadIdx.x; b < 65536u; b += kTableThreads) {
         const uint32_t e = (b >> 7) & 0xFFu, neg = b >> 15;
         uint32_t out;
         if (e >= 3u && e <= 100u) {
             out = b - 0x80u;                                  // exponent - 1
-        } else if (e != 255u && !neg && e >= (is_silu ? 132u : 131u)) {
+        } else if (e != 255u && !neg && e >= 132u) {
             out = b;
-        } else if (e != 255u && neg && e >= (is_silu ? 134u : 131u)) {
-            out = is_silu ? 0x8000u : 0u;
+        } else if (e != 255u && neg && e >= 134u) {
+            out = 0x8000u;
         } else {
             const float h = __uint_as_float(b << 16);
             float a, a_same;
-            unpack2(is_silu ? silu2(h, h) : gelu2(h, h), a, a_same);
+            unpack2(silu2(h, h), a, a_same);
             const __nv_bfloat16 r = __float2bfloat16_rn(a);
             out = *reinterpret_cast<const unsigned short *>(&r);
         }
@@ -444,6 +451,137 @@ quantize_table_kernel(const __grid_constant__ QuantParams prm)
                 }
             }
         }
+        *reinterpret_cast<uint4 *>(dp) = make_uint4(wp[0], wp[1], wp[2], wp[3]);
+        if (DUAL) *reinterpret_cast<uint4 *>(dn) = make_uint4(wn[0], wn[1], wn[2], wn[3]);
+        src += src_step;
+        dp += dst_step;
+        if (DUAL) dn += dst_step;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// ----------------------------------------------------------------------------- GELU by a table of its tail (bf16 inputs)
+// GELU(h) = max(h, 0) - (a / 2) E(a) with a = |h|, E = erfc(a / sqrt 2), in one FMA (gelu_from_tail2).  Of a bf16 value a the tail needs
+// few: below 2^-26 E does not change any more (t + 2.5 and t - 2.5 have rounded to the same values since 2^-23), from 16 on it
+// is zero, and between them lie 30 binades of 128 values.  A table of E as fp32, 15 KiB, built by every block in its shared memory
+// with the same instructions, so leaves about ten instructions of thirty, with the bits of the arithmetic variant, and serves
+// the gated form too, whose product is rounded once, from the unrounded GELU.  One block of 1024 threads per SM: the table is
+// built once per SM (about four entries a thread), ahead of the dependency wait.  Rows travel as in quantize_kernel.
+// Bound by the load unit: 16 scattered loads a chunk, on average three and a half of a warp's in one bank, while instructions issue in
+// 59 % (gated) and 70 % of the cycles.  us, evaluated per element / by a table of all 65536 stored values, which this replaces / here,
+// dual int8: GELU 8858 x 6144 80.0 / 47.3 / 45.8, 8192 x 2560 32.5 / 23.9 / 21.0, 1024 x 2560 7.4 / 9.0 / 6.2; gated 8858 x 6144
+// 90.3 / - / 64.1, 8192 x 2560 37.8 / - / 29.7.
+constexpr uint32_t kTailLo = 101u << 7, kTailHi = 0x4180u;            // bf16 patterns of 2^-26 and 16
+constexpr int kTailEntries = int(kTailHi - kTailLo) + 1;
+constexpr size_t kTailBytes = (size_t(kTailEntries) * 4 + 127) / 128 * 128;
+__host__ __device__ constexpr int tail_depth(bool gated) { return gated ? 3 : 4; }
+__host__ __device__ constexpr size_t tail_smem(bool gated) { return size_t(tail_depth(gated)) * (gated ? 4 : 2) * kTableThreads * 16; }
+
+template <int CODE, int MODE, bool GATED, bool MULT>
+__global__ void __launch_bounds__(kTableThreads, 1)
+quantize_tail_kernel(const __grid_constant__ QuantParams prm)
+{
+    constexpr bool DUAL = MODE == kDual;
+    __shared__ __align__(16) float table[kTailBytes / 4];                // (static: its address is part of the load instructions)
+    extern __shared__ __align__(16) uint8_t tail_ring[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int i = 2 * int(threadIdx.x); i < kTailEntries; i += 2 * kTableThreads) {
+        const uint32_t b = kTailLo + uint32_t(i);
+        float e0, e1;
+        unpack2(gelu_tail2(pack2(__uint_as_float(b << 16), __uint_as_float(min(b + 1, kTailHi) << 16))), e0, e1);
+        *reinterpret_cast<float2 *>(table + i) = make_float2(e0, e1);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    __syncthreads();
+
+    const SegBounds &sb = prm.sb;
+    const int64_t M = prm.M;
+    const int R = prm.R;
+    const uint32_t g = blockIdx.x * kTableThreads + threadIdx.x;
+    const uint32_t r0 = g / uint32_t(prm.V);
+    if (r0 >= uint32_t(R) || int64_t(r0) >= M) return;
+    const int k0 = int(g - r0 * uint32_t(prm.V)) * kVec;                 // the host checked: every chunk lies in one K-segment
+    int p = 0;
+    while (p + 1 < sb.P && k0 >= sb.kb[p + 1]) p++;
+
+    using Tin = __nv_bfloat16;
+    const Tin *src = static_cast<const Tin *>(prm.X) + int64_t(r0) * prm.ld + k0;
+    uint8_t *dp = prm.c_pos + int64_t(r0) * prm.ldc + k0;
+    uint8_t *dn = DUAL ? prm.c_neg + int64_t(r0) * prm.ldc + k0 : nullptr;
+    const int64_t src_step = int64_t(R) * prm.ld, dst_step = int64_t(R) * prm.ldc;
+    uint64_t mreg[MULT ? kVec / 2 : 1];
+    if (MULT) {
+#pragma unroll
+        for (int i = 0; i < kVec; i += 2) mreg[i / 2] = pack2(__ldg(prm.mult + k0 + i), __ldg(prm.mult + k0 + i + 1));
+    }
+    const SegConst cp = seg_const(__ldg(prm.s_pos + p));
+    const SegConst cn = seg_const(DUAL ? __ldg(prm.s_neg + p) : 1.0f);
+    const bool fast = cp.fast && cn.fast && !(DUAL && CODE == SQ_CODE_INT8 && prm.lo != -128);
+
+    constexpr int NS = GATED ? 4 : 2, kDepth = tail_depth(GATED);        // 16-byte pieces per slot, value half first
+    const uint32_t ring0 = uint32_t(__cvta_generic_to_shared(tail_ring)) + threadIdx.x * 16u;
+    auto slot_addr = [&](int slot, int v) { return ring0 + uint32_t((slot * NS + v) * kTableThreads) * 16u; };
+    auto copy_row = [&](const Tin *row_src, int slot, bool valid) {          // one commit group per call, always
+        if (valid) {
+#pragma unroll
+            for (int v = 0; v < NS; v++)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(slot_addr(slot, v)),
+                             "l"(reinterpret_cast<const char *>(v < 2 ? row_src : row_src + prm.K) + 16 * (v & 1)) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto read_piece = [&](int slot, int v, uint32_t (&w)[4]) {
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                     : "r"(slot_addr(slot, v)) : "memory");
+    };
+    auto tail = [&](uint32_t byte_offset) -> float {
+        return *reinterpret_cast<const float *>(reinterpret_cast<const uint8_t *>(table) + byte_offset);
+    };
+#pragma unroll
+    for (int d = 0; d < kDepth - 1; d++) copy_row(src + int64_t(d) * src_step, d, int64_t(r0) + int64_t(d) * R < M);
+    int slot = 0;
+    for (int64_t row = r0; row < M; row += R) {
+        const int ahead = slot == 0 ? kDepth - 1 : slot - 1;
+        copy_row(src + int64_t(kDepth - 1) * src_step, ahead, row + int64_t(kDepth - 1) * R < M);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kDepth - 1) : "memory");
+        uint32_t wp[4], wn[4];
+#pragma unroll
+        for (int half = 0; half < 2; half++) {
+            uint32_t w[4], wg[4];
+            read_piece(slot, half, w);
+            if (GATED) read_piece(slot, 2 + half, wg);
+#pragma unroll
+            for (int q = 0; q < 2; q++) {                                // four elements
+                const int g4 = 2 * half + q;
+                float x[4];
+#pragma unroll
+                for (int i = 0; i < 2; i++) {
+                    const uint32_t h = GATED ? wg[2 * q + i] : w[2 * q + i];
+                    const uint32_t a = __vminu2(h & 0x7FFF7FFFu, kTailHi * 0x10001u), at = __vmaxu2(a, kTailLo * 0x10001u);
+                    const uint32_t off = (at - kTailLo * 0x10001u) << 2;         // byte offsets of both entries, 14 bits each
+                    const uint64_t E = pack2(tail(off & 0xFFFFu), tail(off >> 16));
+                    uint64_t v = gelu_from_tail2(__uint_as_float(h << 16), __uint_as_float(h & 0xFFFF0000u),
+                                                 pack2(__uint_as_float(a << 16), __uint_as_float(a & 0xFFFF0000u)), E);
+                    if (GATED) v = mul2(pack2(__uint_as_float(w[2 * q + i] << 16), __uint_as_float(w[2 * q + i] & 0xFFFF0000u)), v);
+                    v = rounded2<Tin>(v);
+                    if (MULT) v = mul2(v, mreg[MULT ? 2 * g4 + i : 0]);
+                    unpack2(v, x[2 * i], x[2 * i + 1]);
+                }
+                if (fast) {
+                    quant4<CODE, MODE>(x, cp, cn, float(prm.hi), 0, wp[g4], wn[g4]);
+                } else {
+                    wp[g4] = wn[g4] = 0u;
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        uint32_t a, b;
+                        quant1<CODE, MODE>(x[i], cp.s, cn.s, 0, prm.lo, prm.hi, a, b);
+                        wp[g4] |= (a & 0xFFu) << (8 * i);
+                        wn[g4] |= (b & 0xFFu) << (8 * i);
+                    }
+                }
+            }
+        }
+        slot = slot + 1 == kDepth ? 0 : slot + 1;
         *reinterpret_cast<uint4 *>(dp) = make_uint4(wp[0], wp[1], wp[2], wp[3]);
         if (DUAL) *reinterpret_cast<uint4 *>(dn) = make_uint4(wn[0], wn[1], wn[2], wn[3]);
         src += src_step;
@@ -754,23 +892,40 @@ sq_status prepare_mode(QuantLaunch &L, sq_code code, int mode)
     return mode == kDual ? prepare_t<Tin, SQ_CODE_E4M3, kDual>(L) : prepare_t<Tin, SQ_CODE_E4M3, kSingle>(L);
 }
 
-// The table variant of the fused activation: bf16 input, SiLU or GELU, every 16-element chunk inside one K-segment,
-// and enough elements for the table's set-up time not to count.  Returns false where it does not apply.
+// The table variants of the fused activation: bf16 input, every 16-element chunk inside one K-segment, and enough elements for
+// the table's set-up time not to count.  prepare_table returns false where they do not apply.
 std::atomic<int> g_table_mode{0};        // test hook: 0 automatic, 1 always where possible, 2 never
-// measured break-even points (us, evaluated per element against table, K = 1152 and 4608 alike): GELU dual 8 Mi elements
-// 14.4 / 15.2, 9 Mi 16.2 / 16.1, 16 Mi 26.6 / 21.7, single 9 Mi 14.3 / 15.0, 10 Mi 15.8 / 15.7; SiLU dual 18 Mi 21.6 / 22.1,
-// 20 Mi 23.8 / 23.5, 24 Mi 28.0 / 26.8, single 20 Mi 19.6 / 21.8, 24 Mi 23.3 / 24.7 (0.9 / 0.7 us per further Mi)
-constexpr int64_t table_min(bool silu, bool dual) { return int64_t(silu ? (dual ? 20 : 30) : (dual ? 9 : 10)) << 20; }
+// measured break-even points (us, evaluated per element against table): SiLU dual 18 Mi 21.6 / 22.1, 20 Mi 23.8 / 23.5, 24 Mi
+// 28.0 / 26.8, single 20 Mi 19.6 / 21.8, 24 Mi 23.3 / 24.7 (0.9 / 0.7 us per further Mi); GELU dual 0.31 Mi 3.7 / 4.0, 0.62 Mi
+// 4.3 / 4.1, single 0.31 Mi 3.1 / 3.4, 0.62 Mi 3.7 / 3.5; gated GELU dual 5 Mi 11.2 / 12.7, 10 Mi 19.5 / 19.2, single 10 Mi 16.9 / 17.3,
+// 20 Mi 31.1 / 26.8.
+int64_t table_min(int act, bool dual)
+{
+    if (act == SQ_ACT_SILU) return int64_t(dual ? 20 : 30) << 20;
+    return act == SQ_ACT_GELU ? int64_t(1) << 19 : int64_t(dual ? 10 : 12) << 20;
+}
+template <bool MULT>
+const void *tail_kernel(sq_code code, int mode, bool gated)
+{
+    auto pick = [&](auto k_int8_dual, auto k_int8, auto k_e4m3_dual, auto k_e4m3) {
+        return reinterpret_cast<const void *>(code == SQ_CODE_INT8 ? (mode == kDual ? k_int8_dual : k_int8) : (mode == kDual ? k_e4m3_dual : k_e4m3));
+    };
+    return gated ? pick(quantize_tail_kernel<SQ_CODE_INT8, kDual, true, MULT>, quantize_tail_kernel<SQ_CODE_INT8, kSingle, true, MULT>,
+                        quantize_tail_kernel<SQ_CODE_E4M3, kDual, true, MULT>, quantize_tail_kernel<SQ_CODE_E4M3, kSingle, true, MULT>)
+                 : pick(quantize_tail_kernel<SQ_CODE_INT8, kDual, false, MULT>, quantize_tail_kernel<SQ_CODE_INT8, kSingle, false, MULT>,
+                        quantize_tail_kernel<SQ_CODE_E4M3, kDual, false, MULT>, quantize_tail_kernel<SQ_CODE_E4M3, kSingle, false, MULT>);
+}
 bool prepare_table(QuantLaunch &L, sq_dtype dt, sq_code code, int mode)
 {
     QuantParams &prm = L.prm;
     const int tm = g_table_mode.load(std::memory_order_relaxed);
     if (tm == 2 || dt != SQ_BF16 || mode == kZeroPoint || prm.row_segments) return false;
-    if (prm.act != SQ_ACT_SILU && prm.act != SQ_ACT_GELU) return false;
+    if (prm.act != SQ_ACT_SILU && prm.act != SQ_ACT_GELU && prm.act != SQ_ACT_GEGLU) return false;
+    const bool silu = prm.act == SQ_ACT_SILU, gated = prm.act == SQ_ACT_GEGLU;
     if (prm.K % kVec != 0) return false;
     for (int p = 1; p < prm.sb.P; p++)
         if (prm.sb.kb[p] % kVec != 0) return false;
-    if (tm != 1 && prm.M * int64_t(prm.K) < table_min(prm.act == SQ_ACT_SILU, mode == kDual)) return false;
+    if (tm != 1 && prm.M * int64_t(prm.K) < table_min(prm.act, mode == kDual)) return false;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
@@ -779,17 +934,20 @@ bool prepare_table(QuantLaunch &L, sq_dtype dt, sq_code code, int mode)
     const int64_t threads = int64_t(sms) * kTableThreads;                 // one CTA per SM
     int64_t iters = (prm.M * V + threads - 1) / threads;
     if (iters < 1) iters = 1;
-    const int64_t R = (prm.M + iters - 1) / iters;
+    const int64_t R = silu ? (prm.M + iters - 1) / iters : std::min<int64_t>(prm.M, std::max<int64_t>(1, threads / V));
     const int64_t blocks = (R * V + kTableThreads - 1) / kTableThreads;
     if (blocks > 0x7FFFFFFF || R * V > 0xFFFFFFFFll || V > 0x7FFFFFFF || R > 0x7FFFFFFF) return false;
-    const void *kern = nullptr;
-    if (code == SQ_CODE_INT8)
-        kern = mode == kDual ? reinterpret_cast<const void *>(quantize_table_kernel<SQ_CODE_INT8, kDual>)
-                             : reinterpret_cast<const void *>(quantize_table_kernel<SQ_CODE_INT8, kSingle>);
+    const size_t smem = silu ? kTableSmem : tail_smem(gated);
+    const void *kern;
+    if (!silu)
+        kern = prm.mult ? tail_kernel<true>(code, mode, gated) : tail_kernel<false>(code, mode, gated);
+    else if (code == SQ_CODE_INT8)
+        kern = mode == kDual ? reinterpret_cast<const void *>(quantize_silu_table_kernel<SQ_CODE_INT8, kDual>)
+                             : reinterpret_cast<const void *>(quantize_silu_table_kernel<SQ_CODE_INT8, kSingle>);
     else
-        kern = mode == kDual ? reinterpret_cast<const void *>(quantize_table_kernel<SQ_CODE_E4M3, kDual>)
-                             : reinterpret_cast<const void *>(quantize_table_kernel<SQ_CODE_E4M3, kSingle>);
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTableSmem)) != cudaSuccess) {
+        kern = mode == kDual ? reinterpret_cast<const void *>(quantize_silu_table_kernel<SQ_CODE_E4M3, kDual>)
+                             : reinterpret_cast<const void *>(quantize_silu_table_kernel<SQ_CODE_E4M3, kSingle>);
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
     }
@@ -798,7 +956,7 @@ bool prepare_table(QuantLaunch &L, sq_dtype dt, sq_code code, int mode)
     L.blocks = unsigned(blocks);
     L.kernel = kern;
     L.threads = kTableThreads;
-    L.smem = unsigned(kTableSmem);
+    L.smem = unsigned(smem);
     return true;
 }
 
