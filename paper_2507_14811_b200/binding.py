@@ -1,5 +1,5 @@
-"""Thin binding over libsegquant.so: argument marshalling only.  The calls that a layer makes at run time go through the
-native module built from csrc/torch_calls.cpp, the offline ones through ctypes.
+"""Thin binding over libsegquant.so: argument marshalling only.  The calls that a layer makes at run time or when it is built go
+through the native module built from csrc/torch_calls.cpp, the others through ctypes.
 
 Function names mirror the C ABI (include/segquant.h).  Tensors are torch CUDA tensors used as
 device memory; every step of the path runs inside the library's kernels.  There is no fallback:
@@ -41,7 +41,7 @@ class SegquantError(RuntimeError):
 
 
 class _SegTable(C.Structure):
-    _fields_ = [("P", C.c_int32), ("kb", C.POINTER(C.c_int32)), ("Q", C.c_int32), ("nb", C.POINTER(C.c_int32))]
+    _fields_ = [("P", C.c_int32), ("kb", C.c_void_p), ("Q", C.c_int32), ("nb", C.c_void_p)]
 
 
 _lib = None
@@ -86,8 +86,7 @@ class SegTable:
     def __init__(self, kb, nb):
         self.kb = np.ascontiguousarray(kb, np.int32)
         self.nb = np.ascontiguousarray(nb, np.int32)
-        self._c = _SegTable(len(self.kb) - 1, self.kb.ctypes.data_as(C.POINTER(C.c_int32)),
-                            len(self.nb) - 1, self.nb.ctypes.data_as(C.POINTER(C.c_int32)))
+        self._c = _SegTable(len(self.kb) - 1, self.kb.ctypes.data, len(self.nb) - 1, self.nb.ctypes.data)
         self.address = C.addressof(self._c)
 
     @property
@@ -151,14 +150,8 @@ def new_workspace(device="cuda", split_for=None) -> torch.Tensor:
 def segquant_calib_scales(X: torch.Tensor, seg: SegTable, code: str, is_weight: bool, dual: bool,
                           workspace: torch.Tensor, flags: int = 0):
     """Returns (s_pos, s_neg|None) for activations, (s_w [P*Q], None) for weights."""
-    rows, K = X.shape
     n = seg.P * (seg.Q if is_weight else 1)
-    s_pos = torch.empty(n, dtype=torch.float32, device=X.device)
-    s_neg = torch.empty(n, dtype=torch.float32, device=X.device) if (dual and not is_weight) else None
-    st = lib().segquant_calib_scales(_ptr(X), C.c_int(_dt(X)), C.c_int64(rows), C.c_int64(K), C.c_int64(X.stride(0)),
-                                     seg.ref(), C.c_int(SQ_CODE[code]), C.c_int(int(is_weight)), C.c_int(int(dual)),
-                                     C.c_uint32(flags), _ptr(s_pos), _ptr(s_neg), _ptr(workspace),
-                                     C.c_size_t(workspace.numel()), _stream())
+    st, s_pos, s_neg = _calls().calib_scales(X, seg.address, n, SQ_CODE[code], is_weight, dual, workspace, flags)
     _check(st, "segquant_calib_scales")
     return s_pos, s_neg
 
@@ -255,12 +248,7 @@ def segquant_fold_zero_point(Wq: torch.Tensor, seg: SegTable, s_x, z_x, s_w, bia
 
 
 def segquant_quantize_weight(W: torch.Tensor, seg: SegTable, s_w, code: str, flags: int = 0, Wq=None):
-    N, K = W.shape
-    if Wq is None:
-        Wq = new_codes(N, K, W.device)
-    st = lib().segquant_quantize_weight(_ptr(W), C.c_int(_dt(W)), C.c_int64(N), C.c_int64(K), C.c_int64(W.stride(0)),
-                                        seg.ref(), _ptr(s_w), C.c_int(SQ_CODE[code]), C.c_uint32(flags),
-                                        _ptr(Wq), C.c_int64(Wq.stride(0)), _stream())
+    st, Wq = _calls().quantize_weight(W, seg.address, s_w, SQ_CODE[code], flags, Wq)
     _check(st, "segquant_quantize_weight")
     return Wq
 

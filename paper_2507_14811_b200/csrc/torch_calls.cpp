@@ -1,4 +1,4 @@
-// The calls a layer makes at run time, as functions that take torch tensors: reading shapes, strides, pointers and the
+// The calls a layer makes at run time and when it is built, as functions that take torch tensors: reading shapes, strides, pointers and the
 // current stream here costs a fraction of what it costs in Python (an eager 256 x 256 -> 768 layer call: 17.9 us with
 // ctypes objects, 8.5 us from here; the three calls of a 2048 x 4608 -> 1152 W4A8 layer: 50.6 -> 32.8 us).  Argument
 // marshalling only: every check is the C ABI's (include/segquant.h), every function returns its status (with the tensors
@@ -172,6 +172,54 @@ PyObject *quantize_act_fused(PyObject *, PyObject *const *args, Py_ssize_t n)
     });
 }
 
+// X, seg, number of scales, code, is_weight, dual, workspace, flags -> (status, s_pos, s_neg | None)
+PyObject *calib_scales(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    return guarded("calib_scales", n, 8, [&]() -> PyObject * {
+        const Args a{args};
+        const at::Tensor &x = a.matrix(0);
+        const sq_dtype dx = dtype_of(x);
+        const Rows X(x);
+        const sq_segtable *seg = a.seg(1);
+        const int64_t scales = a.integer(2);
+        const sq_code code = sq_code(a.integer(3));
+        const bool is_weight = a.truth(4), dual = a.truth(5);
+        void *ws = a.ptr(6), *stream = current_stream();
+        const size_t ws_bytes = a.bytes(6);
+        const uint32_t flags = uint32_t(a.integer(7));
+        const auto f32 = x.options().dtype(at::kFloat);
+        at::Tensor sp = at::empty({scales}, f32), sn;
+        if (dual && !is_weight) sn = at::empty({scales}, f32);
+        float *s_pos = sp.data_ptr<float>(), *s_neg = sn.defined() ? sn.data_ptr<float>() : nullptr;
+        const sq_status st = without_gil([&] {
+            return segquant_calib_scales(X.p, dx, X.rows, X.cols, X.ld, seg, code, is_weight, dual, flags, s_pos, s_neg, ws, ws_bytes, stream);
+        });
+        return Py_BuildValue("(iNN)", int(st), THPVariable_Wrap(sp), THPVariable_Wrap(sn));
+    });
+}
+
+// W, seg, s_w, code, flags, Wq | None -> (status, Wq)
+PyObject *quantize_weight(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    return guarded("quantize_weight", n, 6, [&]() -> PyObject * {
+        const Args a{args};
+        const at::Tensor &w = a.matrix(0);
+        const sq_dtype dw = dtype_of(w);
+        const Rows W(w);
+        const sq_segtable *seg = a.seg(1);
+        const float *sw = a.f32(2);
+        const sq_code code = sq_code(a.integer(3));
+        const uint32_t flags = uint32_t(a.integer(4));
+        const at::Tensor q = a.none(5) ? new_codes(W.rows, W.cols, w) : a.tensor(5);
+        const Rows C(q);
+        void *stream = current_stream();
+        const sq_status st = without_gil([&] {
+            return segquant_quantize_weight(W.p, dw, W.rows, W.cols, W.ld, seg, sw, code, flags, C.p, C.ld, stream);
+        });
+        return Py_BuildValue("(iN)", int(st), THPVariable_Wrap(q));
+    });
+}
+
 // Xq_pos, Xq_neg | None, Wq, seg, code, s_pos, s_neg | None, s_w, bias, Y, acc_dump | None, workspace, kind
 enum GemmCall : int { kSeglinear = 0, kDualscale = 1, kW4a8 = 2 };
 PyObject *gemm(PyObject *, PyObject *const *args, Py_ssize_t n)
@@ -256,7 +304,7 @@ PyObject *plan_run(PyObject *, PyObject *const *args, Py_ssize_t n)
 
 #define SQ_METHOD(f) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(f)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {SQ_METHOD(layer_forward), SQ_METHOD(quantize_act), SQ_METHOD(quantize_act_fused), SQ_METHOD(gemm),
-                         SQ_METHOD(quantize_per_row), SQ_METHOD(unpack_w4), SQ_METHOD(plan_run), {nullptr, nullptr, 0, nullptr}};
+                         SQ_METHOD(quantize_per_row), SQ_METHOD(calib_scales), SQ_METHOD(quantize_weight), SQ_METHOD(unpack_w4), SQ_METHOD(plan_run), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
