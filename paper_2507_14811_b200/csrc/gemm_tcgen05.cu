@@ -38,6 +38,7 @@
 #include <cuda_bf16.h>
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <type_traits>
 #include "quant_codes.cuh"
 
@@ -984,6 +985,8 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
             const uint64_t kStageDesc = uint64_t(stage_bytes) >> 4;
             // from this warp's activation tile to its weight tile, modulo 2^32 in the descriptor's low word
             const uint32_t b_off = (WIDE ? pol * b_bytes : 0u) / 16u - (kHalves * b_bytes + (WIDE ? 0u : pol) * a_bytes) / 16u;
+            const uint32_t stage16 = stage_bytes >> 4, desc_hi = uint32_t(desc0 >> 32);
+            constexpr uint32_t empty_off = uint32_t(offsetof(SharedHeader, empty) - offsetof(SharedHeader, full));
             auto b_desc = [&](uint64_t da) { return (da & ~0xFFFFFFFFull) | uint32_t(uint32_t(da) + b_off); };
             uint32_t s = 0, ph = 0, as = 0, aph = 0;
             bool ok = true;
@@ -1056,30 +1059,37 @@ segquant_gemm_kernel(const __grid_constant__ CUtensorMap tm_a_pos, const __grid_
                             }
                         }
                     }
-                    const int k_loop = P == 1 || k_end == prm.K ? k_end : k_end / BLOCK_K * BLOCK_K;
-                    for (; k < k_loop; k += BLOCK_K) {
-                        if (!mbar_wait_warp(full0 + 8 * s, ph, abort_flag, prm.status, kWhereMmaFull)) {
+                    // The loop of whole blocks: what an iteration needs is in registers and goes on by addition.  With the descriptor
+                    // multiplied out, the K-steps counted and the parameters read per block it bounded tiles that give the pipe less
+                    // than some 400 cycles per block (us: 2048 x 4608 -> 1152 single 12.7 -> 11.2, 600 x 3072 -> 1024 single 8.3 -> 7.3, 1689 x 1920
+                    // -> 4224 dual in 15 segments 46.5 -> 42, 8858 x 1536 -> 1536 in 24 segments 54.1 -> 52.4).
+                    uint32_t a_lo = uint32_t(desc0) + s * stage16, bar_empty = empty0 + 8 * s;
+                    for (; k + BLOCK_K <= k_end; k += BLOCK_K) {
+                        if (!mbar_wait_warp(bar_empty - empty_off, ph, abort_flag, prm.status, kWhereMmaFull)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
-                        const uint64_t da = desc0 + s * kStageDesc;
-                        const int rem = k_end - k;
-                        const int nk = rem >= BLOCK_K ? BLOCK_K / MMA_K : (rem + MMA_K - 1) / MMA_K;
                         if (elect_one()) {
-                            issue_kblock<KIND, CG>(d0, da, b_desc(da), idesc, nk, accumulate);
-                            tc_commit<CG>(empty0 + 8 * s);         // the slot is free when both threads' MMAs have retired
+                            issue_full_kblock<KIND, CG>(d0, a_lo, a_lo + b_off, desc_hi, idesc, accumulate);
+                            tc_commit<CG>(bar_empty);              // the slot is free when both threads' MMAs have retired
                         }
                         accumulate = 1;
-                        if (++s == stages) { s = 0; ph ^= 1; }
+                        a_lo += stage16;
+                        bar_empty += 8;
+                        if (++s == stages) { s = 0; ph ^= 1; a_lo = uint32_t(desc0); bar_empty = empty0; }
                     }
-                    if (P > 1 && ok && k < k_end) {                // the segment ends inside this block
+                    if (ok && k < k_end) {                         // the segment, or K, ends inside this block
                         if (!mbar_wait_warp(full0 + 8 * s, ph, abort_flag, prm.status, kWhereMmaFull)) {
                             ok = false;
                         } else {
                             tc_fence_after();
                             const uint64_t da = desc0 + s * kStageDesc;
-                            if (elect_one()) issue_kblock<KIND, CG>(d0, da, b_desc(da), idesc, (k_end - k) / MMA_K, accumulate);
+                            if (elect_one()) issue_kblock<KIND, CG>(d0, da, b_desc(da), idesc, (k_end - k + MMA_K - 1) / MMA_K, accumulate);
+                            if (k_end == prm.K) {                  // nobody else uses it
+                                if (elect_one()) tc_commit<CG>(empty0 + 8 * s);
+                                if (++s == stages) { s = 0; ph ^= 1; }
+                            }
                         }
                     }
                     if (SEQ) {
