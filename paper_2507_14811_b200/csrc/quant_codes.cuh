@@ -176,8 +176,9 @@ constexpr int kMagicBits = 0x4B400000;       // its bit pattern: bits(v + magic)
 // 4 elements of one K-segment -> one word of packed codes per matrix.
 // int8, dual: both polarities are quantized as non-negative numbers, max(x, 0) and max(-x, 0) = max(x, 0) - x,
 //   each with its own constants.  Adding the magic constant rounds half to even; the integer is the distance of
-//   the sum's bit pattern from the constant's, taken with the sign of the polarity, and a saturating pack clips
-//   it to [-128, 127].  A quotient beyond the range of the magic constant, infinity, or the NaN of an overflowed
+//   the sum's bit pattern from the constant's, one of the two is zero, so the difference of the two bit patterns is the signed
+//   code, a saturating pack clips it to [-128, 127] and its sign says whose it is (one subtraction and one pack for both
+//   polarities: 1111 x 1072 fp32 3.5 -> 3.0 us, 8858 x 1536 15.2 -> 14.5; bf16 inputs are bound by memory or latency).  A quotient beyond the range of the magic constant, infinity, or the NaN of an overflowed
 //   chain all have bit patterns above the constant's, so they saturate to the end of the code range as the
 //   clip demands; nothing has to be bounded beforehand.  (A negative bound of -127 takes the division path.)
 // int8, single scale: |x| is quantized, clipped in fp32 (clip-then-round equals round-then-clip for integer
@@ -211,19 +212,21 @@ __device__ __forceinline__ void quant4(const float (&x)[4], const SegConst &cp, 
         const uint64_t rp2 = pack2(cp.r, cp.r), nsp2 = pack2(-cp.s, -cp.s);
         const uint64_t rn2 = pack2(cn.r, cn.r), nsn2 = pack2(-cn.s, -cn.s);
         const uint64_t minus1 = pack2(-1.0f, -1.0f);
-        int kp[4], kn[4];
+        int k[4];
 #pragma unroll
         for (int i = 0; i < 4; i += 2) {
             const uint64_t xp2 = pack2(fmaxf(x[i], 0.0f), fmaxf(x[i + 1], 0.0f));
             const uint64_t xn2 = fma2(pack2(x[i], x[i + 1]), minus1, xp2);          // max(x, 0) - x, exact
-            uint32_t a, b;
-            unpack2u(add2(div2_rn_fast(xp2, nsp2, rp2), magic2), a, b);
-            kp[i] = int(a) - kMagicBits; kp[i + 1] = int(b) - kMagicBits;
-            unpack2u(add2(div2_rn_fast(xn2, nsn2, rn2), magic2), a, b);
-            kn[i] = kMagicBits - int(a); kn[i + 1] = kMagicBits - int(b);
+            uint32_t p0, p1, n0, n1;
+            unpack2u(add2(div2_rn_fast(xp2, nsp2, rp2), magic2), p0, p1);
+            unpack2u(add2(div2_rn_fast(xn2, nsn2, rn2), magic2), n0, n1);
+            k[i] = int(p0 - n0); k[i + 1] = int(p1 - n1);
         }
-        wp = pack_sat_s8(kp[1], kp[0], pack_sat_s8(kp[3], kp[2], 0u));
-        wn = pack_sat_s8(kn[1], kn[0], pack_sat_s8(kn[3], kn[2], 0u));
+        const uint32_t w = pack_sat_s8(k[1], k[0], pack_sat_s8(k[3], k[2], 0u));
+        uint32_t negative;                              // 0xFF in the bytes below zero
+        asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(negative) : "r"(w));
+        wp = w & ~negative;
+        wn = w & negative;
         return;
     }
     uint32_t bp[4], bn[4];
