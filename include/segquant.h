@@ -337,7 +337,7 @@ sq_status segquant_set_tuning(int tile_n, int stages, int cta_group, int segment
  * evaluates SiLU / GELU per element, and, for bf16 inputs, one that looks up a table which every thread block builds in
  * shared memory first: SiLU the stored activation of all 65536 bf16 values (about 9 us per launch), GELU and gated GELU the
  * 3841 values of erfc(|h| / sqrt 2) that differ (about 1 us).  fused_table_mode: 0 automatic (from 20 Mi elements up for SiLU with dual
- * codes and 30 Mi with single-scale ones, from 0.5 Mi for GELU, 10 and 12 Mi for gated GELU), 1 the table wherever it
+ * codes and 30 Mi with single-scale ones, from 1.25 Mi for GELU, 10 and 12 Mi for gated GELU), 1 the table wherever it
  * applies, 2 never.  Process-wide and for tests and sweeps, like segquant_set_tuning. */
 sq_status segquant_set_quantize_tuning(int fused_table_mode);
 

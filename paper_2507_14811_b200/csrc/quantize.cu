@@ -328,6 +328,79 @@ quantize_kernel(const __grid_constant__ QuantParams prm)
     asm volatile("cp.async.wait_group 0;" ::: "memory");     // nothing of this thread's is in flight when it leaves
 }
 
+// ----------------------------------------------------------------------------- small inputs
+// A launch of few elements lasts as long as one thread's chain of loads, evaluation and stores: sixteen elements of gated GELU
+// are some 700 dependent instructions.  Here a thread has four elements and nothing to walk.  Used while every thread of the
+// grid can be resident at once, roughly (few_limit).  us, 16 elements a thread / 4: 8 x 3072 dual int8 1.8 / 1.3, 400 x 2560 2.9 / 2.3, GELU 64 x
+// 2048 2.9 / 1.8, gated fp32 24 x 5632 4.2 / 1.6.
+constexpr int kFewVec = 4;
+__device__ __forceinline__ void load4(const float *p, float (&x)[4])
+{
+    const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
+    x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+}
+__device__ __forceinline__ void load4(const __nv_bfloat16 *p, float (&x)[4])
+{
+    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p));
+    x[0] = __uint_as_float(v.x << 16); x[1] = __uint_as_float(v.x & 0xFFFF0000u);
+    x[2] = __uint_as_float(v.y << 16); x[3] = __uint_as_float(v.y & 0xFFFF0000u);
+}
+
+template <typename Tin, int CODE, int MODE, int PRE>
+__global__ void __launch_bounds__(kThreads)
+quantize_few_kernel(const __grid_constant__ QuantParams prm)
+{
+    constexpr bool DUAL = MODE == kDual, GATED = PRE == 2;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const SegBounds &sb = prm.sb;
+    const uint32_t g = blockIdx.x * kThreads + threadIdx.x;
+    const uint32_t row = g / uint32_t(prm.V);
+    const int k0 = int(g - row * uint32_t(prm.V)) * kFewVec, K = prm.K;
+    int p = 0;
+    while (p + 1 < sb.P && k0 >= sb.kb[p + 1]) p++;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (int64_t(row) >= prm.M) return;
+    const Tin *src = static_cast<const Tin *>(prm.X) + int64_t(row) * prm.ld + k0;
+    uint8_t *dp = prm.c_pos + int64_t(row) * prm.ldc + k0;
+    uint8_t *dn = DUAL ? prm.c_neg + int64_t(row) * prm.ldc + k0 : nullptr;
+    const float sp = __ldg(prm.s_pos + p), sn = DUAL ? __ldg(prm.s_neg + p) : 1.0f;
+    if (k0 + kFewVec <= sb.kb[p + 1]) {
+        float x[4], gate[4], m[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+        load4(src, x);
+        if (GATED) load4(src + K, gate);
+        if (PRE && prm.mult) {
+#pragma unroll
+            for (int i = 0; i < 4; i++) m[i] = __ldg(prm.mult + k0 + i);
+        }
+        const int zp = MODE == kZeroPoint ? __ldg(prm.zp + p) : 0;
+        const SegConst cp = seg_const(sp), cn = seg_const(sn);
+        if (cp.fast && cn.fast && !(DUAL && CODE == SQ_CODE_INT8 && prm.lo != -128)) {
+#pragma unroll
+            for (int i = 0; i < 4 && PRE != 0; i += 2) {
+                const uint64_t m2 = pack2(m[i], m[i + 1]);
+                unpack2(GATED ? pre_gated2<Tin>(x[i], x[i + 1], gate[i], gate[i + 1], m2) : pre2<Tin>(x[i], x[i + 1], prm.act, m2), x[i], x[i + 1]);
+            }
+            uint32_t wp, wn;
+            quant4<CODE, MODE>(x, cp, cn, float(prm.hi), zp, wp, wn);
+            *reinterpret_cast<uint32_t *>(dp) = wp;
+            if (DUAL) *reinterpret_cast<uint32_t *>(dn) = wn;
+            return;
+        }
+    }
+    const int n = min(kFewVec, K - k0);                  // a segment bound or the row's end among the four, or an extreme scale
+    for (int i = 0; i < n; i++) {
+        while (p + 1 < sb.P && k0 + i >= sb.kb[p + 1]) p++;
+        uint32_t a, b;
+        float x = load1(src + i);
+        if (GATED) x = pre_gated<Tin>(x, load1(src + K + i), prm.mult ? __ldg(prm.mult + k0 + i) : 1.0f);
+        else if (PRE) x = pre1<Tin>(x, prm.act, prm.mult ? __ldg(prm.mult + k0 + i) : 1.0f);
+        quant1<CODE, MODE>(x, __ldg(prm.s_pos + p), DUAL ? __ldg(prm.s_neg + p) : 0.0f, MODE == kZeroPoint ? __ldg(prm.zp + p) : 0,
+                           prm.lo, prm.hi, a, b);
+        dp[i] = uint8_t(a);
+        if (DUAL) dn[i] = uint8_t(b);
+    }
+}
+
 // ----------------------------------------------------------------------------- fused SiLU by table (bf16 inputs)
 // A bf16 pre-activation has 65536 possible values, so the stored activation bf16(silu(h)) is a table of 128 KiB.
 // Every CTA (1024 threads, one per SM) builds the table in its shared memory with the same silu2 as
@@ -848,6 +921,17 @@ pack_w4_kernel(uint8_t *__restrict__ w8, int64_t ld8, int64_t N, int K, uint8_t 
     }
 }
 
+std::atomic<int> g_table_mode{0};        // test hook: 0 automatic, 1 a table wherever possible, 2 never
+// Threads of four elements per SM up to which quantize_few_kernel is the faster one: about as many as an SM holds, more where
+// sixteen elements a thread cost most (us, 16 / 4 elements, dual int8, Mi elements: plain bf16 0.98 2.87 / 2.29, 1.25 3.0 / 3.1; fp32 1.56
+// 4.1 / 3.7, 2.44 4.6 / 4.8; SiLU bf16 1.25 3.9 / 3.8, 1.56 3.9 / 4.1; fp32 SiLU 2.44 6.1 / 5.9, GELU 2.44 7.5 / 6.8, 4.39 9.7 / 10.5; gated bf16 2.44
+// 8.3 / 7.2, 4.39 10.7 / 11.2; gated fp32 4.39 16.0 / 11.1, 40 91.3 / 86.2: up to any ordinary size).
+int64_t few_limit(bool f32, int act, bool pre)
+{
+    if (act == SQ_ACT_GEGLU) return f32 ? 1 << 20 : 4400;
+    return f32 ? (pre ? 4400 : 2800) : (pre ? 2048 : 1800);
+}
+
 template <typename Tin, int CODE, int MODE>
 sq_status prepare_t(QuantLaunch &L)
 {
@@ -860,6 +944,17 @@ sq_status prepare_t(QuantLaunch &L)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
         return SQ_ERR_CUDA;
     const bool pre = prm.act != 0 || prm.mult != nullptr;
+    if (!prm.row_segments) {
+        const int64_t V4 = (prm.K + kFewVec - 1) / kFewVec;
+        if (prm.M * V4 <= few_limit(sizeof(Tin) == 4, prm.act, pre) * sms) {
+            prm.V = int(V4);
+            L.blocks = unsigned((prm.M * V4 + kThreads - 1) / kThreads);
+            L.kernel = prm.act == SQ_ACT_GEGLU ? reinterpret_cast<const void *>(quantize_few_kernel<Tin, CODE, MODE, 2>)
+                       : pre                   ? reinterpret_cast<const void *>(quantize_few_kernel<Tin, CODE, MODE, 1>)
+                                               : reinterpret_cast<const void *>(quantize_few_kernel<Tin, CODE, MODE, 0>);
+            return SQ_OK;
+        }
+    }
     const int64_t V = (prm.K + kVec - 1) / kVec;
     const int64_t target_threads = int64_t(sms) * kThreads * (pre ? 3 : kBlocksPerSm);
     int64_t iters = (prm.M * V + target_threads - 1) / target_threads;
@@ -894,15 +989,14 @@ sq_status prepare_mode(QuantLaunch &L, sq_code code, int mode)
 
 // The table variants of the fused activation: bf16 input, every 16-element chunk inside one K-segment, and enough elements for
 // the table's set-up time not to count.  prepare_table returns false where they do not apply.
-std::atomic<int> g_table_mode{0};        // test hook: 0 automatic, 1 always where possible, 2 never
-// measured break-even points (us, evaluated per element against table): SiLU dual 18 Mi 21.6 / 22.1, 20 Mi 23.8 / 23.5, 24 Mi
-// 28.0 / 26.8, single 20 Mi 19.6 / 21.8, 24 Mi 23.3 / 24.7 (0.9 / 0.7 us per further Mi); GELU dual 0.31 Mi 3.7 / 4.0, 0.62 Mi
-// 4.3 / 4.1, single 0.31 Mi 3.1 / 3.4, 0.62 Mi 3.7 / 3.5; gated GELU dual 5 Mi 11.2 / 12.7, 10 Mi 19.5 / 19.2, single 10 Mi 16.9 / 17.3,
+// measured break-even points (us, evaluated per element, few or many elements a thread, against table): SiLU dual 18 Mi 21.6 / 22.1, 20 Mi 23.8 / 23.5, 24 Mi
+// 28.0 / 26.8, single 20 Mi 19.6 / 21.8, 24 Mi 23.3 / 24.7 (0.9 / 0.7 us per further Mi); GELU dual 0.98 Mi 3.4 / 4.1, 1.25 Mi
+// 4.3 / 4.4, 2.44 Mi 6.7 / 6.1, single 1.25 Mi 3.4 / 3.5; gated GELU dual 5 Mi 11.2 / 12.7, 10 Mi 19.5 / 19.2, single 10 Mi 16.9 / 17.3,
 // 20 Mi 31.1 / 26.8.
 int64_t table_min(int act, bool dual)
 {
     if (act == SQ_ACT_SILU) return int64_t(dual ? 20 : 30) << 20;
-    return act == SQ_ACT_GELU ? int64_t(1) << 19 : int64_t(dual ? 10 : 12) << 20;
+    return act == SQ_ACT_GELU ? int64_t(5) << 18 : int64_t(dual ? 10 : 12) << 20;
 }
 template <bool MULT>
 const void *tail_kernel(sq_code code, int mode, bool gated)
