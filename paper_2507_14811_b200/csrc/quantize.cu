@@ -878,46 +878,62 @@ quantize_per_row_kernel(const Tin *__restrict__ X, int K, int64_t ld, const SegB
     }
 }
 
-// int8 codes in [-8, 7] <-> two 4-bit codes per byte (code 2j in the low nibble); 16 codes per thread.  A small kernel between
+// int8 codes in [-8, 7] <-> two 4-bit codes per byte (code 2j in the low nibble); 16 codes to a chunk.  A small kernel between
 // two others on every W4A8 call: launched like them, so that its start and theirs overlap the kernel in front (2048 x 4608 ->
-// 1152 whole layer 32.8 -> 30.4 us).
+// 1152 whole layer 32.8 -> 30.4 us).  Bound by memory: a thread takes up to kPackChunks chunks a grid apart, their loads in flight
+// together, and 32-bit divisions where 32 bits count the chunks.  (unpack, us, one chunk a thread and 64-bit divisions / now: 16072 x
+// 10400, 250 MB, 49.9 / 39.9 = 6.3 TB/s; 5552 x 3584 7.4 / 6.2; 504 x 6688 2.1 / 1.9.)
+constexpr int kPackChunks = 4;
+template <typename Index, bool UNPACK, int CHUNKS>
 __global__ void __launch_bounds__(kThreads)
-pack_w4_kernel(uint8_t *__restrict__ w8, int64_t ld8, int64_t N, int K, uint8_t *__restrict__ w4, int64_t ld4, int unpack)
+pack_w4_kernel(uint8_t *__restrict__ w8, int64_t ld8, Index total, uint32_t V, uint8_t *__restrict__ w4, int64_t ld4)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int V = K / kVec;
-    const int64_t idx = int64_t(blockIdx.x) * kThreads + threadIdx.x;
-    if (idx >= N * V) return;
-    const int64_t n = idx / V;
-    const int k0 = int(idx - n * V) * kVec;
-    if (!unpack) {
-        const uint4 v = *reinterpret_cast<const uint4 *>(w8 + n * ld8 + k0);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-        uint32_t o[2];
+    const Index first = Index(blockIdx.x) * kThreads + threadIdx.x, step = Index(gridDim.x) * kThreads;
+    uint8_t *p8[CHUNKS], *p4[CHUNKS];
+    uint4 v8[CHUNKS];
+    uint2 v4[CHUNKS];
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const uint32_t a = w[2 * h], b = w[2 * h + 1];          // 4 codes each
-            const uint32_t pa = (a & 0xF) | ((a >> 4) & 0xF0) | ((a >> 8) & 0xF00) | ((a >> 12) & 0xF000);
-            const uint32_t pb = (b & 0xF) | ((b >> 4) & 0xF0) | ((b >> 8) & 0xF00) | ((b >> 12) & 0xF000);
-            o[h] = pa | (pb << 16);
+    for (int c = 0; c < CHUNKS; c++) {
+        const Index idx = first + Index(c) * step, n = idx / Index(V);
+        const int64_t k0 = int64_t(idx - n * Index(V)) * kVec;
+        p8[c] = w8 + int64_t(n) * ld8 + k0;
+        p4[c] = w4 + int64_t(n) * ld4 + k0 / 2;
+        if (idx < total) {
+            if (UNPACK) v4[c] = *reinterpret_cast<const uint2 *>(p4[c]);
+            else v8[c] = *reinterpret_cast<const uint4 *>(p8[c]);
         }
-        *reinterpret_cast<uint2 *>(w4 + n * ld4 + k0 / 2) = make_uint2(o[0], o[1]);
-    } else {
-        const uint2 v = *reinterpret_cast<const uint2 *>(w4 + n * ld4 + k0 / 2);
-        const uint32_t in[2] = {v.x, v.y};
-        uint32_t o[4];
+    }
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
+    for (int c = 0; c < CHUNKS; c++) {
+        if (first + Index(c) * step >= total) break;
+        if (!UNPACK) {
+            const uint32_t w[4] = {v8[c].x, v8[c].y, v8[c].z, v8[c].w};
+            uint32_t o[2];
 #pragma unroll
-            for (int t = 0; t < 2; t++) {
-                const uint32_t hw = (in[h] >> (16 * t)) & 0xFFFFu;   // 4 nibbles
-                uint32_t bytes = (hw & 0xF) | ((hw & 0xF0) << 4) | ((hw & 0xF00) << 8) | ((hw & 0xF000) << 12);
-                bytes |= (bytes & 0x08080808u) * 0x1Eu;              // sign-extend each nibble: bit 3 copied into bits 4..7
-                o[2 * h + t] = bytes;
+            for (int h = 0; h < 2; h++) {
+                const uint32_t a = w[2 * h], b = w[2 * h + 1];          // 4 codes each
+                const uint32_t pa = (a & 0xF) | ((a >> 4) & 0xF0) | ((a >> 8) & 0xF00) | ((a >> 12) & 0xF000);
+                const uint32_t pb = (b & 0xF) | ((b >> 4) & 0xF0) | ((b >> 8) & 0xF00) | ((b >> 12) & 0xF000);
+                o[h] = pa | (pb << 16);
             }
+            *reinterpret_cast<uint2 *>(p4[c]) = make_uint2(o[0], o[1]);
+        } else {
+            const uint32_t in[2] = {v4[c].x, v4[c].y};
+            uint32_t o[4];
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+#pragma unroll
+                for (int t = 0; t < 2; t++) {
+                    const uint32_t hw = (in[h] >> (16 * t)) & 0xFFFFu;   // 4 nibbles
+                    uint32_t bytes = (hw & 0xF) | ((hw & 0xF0) << 4) | ((hw & 0xF00) << 8) | ((hw & 0xF000) << 12);
+                    bytes |= (bytes & 0x08080808u) * 0x1Eu;              // sign-extend each nibble: bit 3 copied into bits 4..7
+                    o[2 * h + t] = bytes;
+                }
+            }
+            *reinterpret_cast<uint4 *>(p8[c]) = make_uint4(o[0], o[1], o[2], o[3]);
         }
-        *reinterpret_cast<uint4 *>(w8 + n * ld8 + k0) = make_uint4(o[0], o[1], o[2], o[3]);
     }
 }
 
@@ -1174,8 +1190,16 @@ sq_status launch_quantize_per_row(const void *X, sq_dtype dt, int64_t M, int64_t
 sq_status launch_pack_w4(const void *Wq8, int64_t ld8, int64_t N, int64_t K, void *Wq4, int64_t ld4, int unpack,
                          cudaStream_t st)
 {
-    const int64_t blocks = (N * (K / kVec) + kThreads - 1) / kThreads;
-    if (blocks > 0x7FFFFFFF) return SQ_ERR_SHAPE;
+    const int64_t total = N * (K / kVec), chunks = (total + kThreads - 1) / kThreads;
+    if (chunks > 0x7FFFFFFF) return SQ_ERR_SHAPE;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+        return SQ_ERR_CUDA;
+    // several chunks a thread where that leaves every SM some blocks to follow one another (unpack, us, one / four chunks, blocks of
+    // single chunks per SM: 8.8 2.9 / 3.8, 13.5 3.8 / 4.2, 20.3 4.9 / 5.0, 27 6.0 / 5.5)
+    const int per_thread = chunks > int64_t(sms) * 20 ? kPackChunks : 1;
+    const int64_t blocks = (chunks + per_thread - 1) / per_thread;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(unsigned(blocks));
     cfg.blockDim = dim3(kThreads);
@@ -1185,8 +1209,18 @@ sq_status launch_pack_w4(const void *Wq8, int64_t ld8, int64_t N, int64_t K, voi
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, pack_w4_kernel, static_cast<uint8_t *>(const_cast<void *>(Wq8)), ld8, N, int(K),
-                                             static_cast<uint8_t *>(Wq4), ld4, unpack);
+    uint8_t *w8 = static_cast<uint8_t *>(const_cast<void *>(Wq8)), *w4 = static_cast<uint8_t *>(Wq4);
+    const uint32_t V = uint32_t(K / kVec);
+    cudaError_t e;
+    if (blocks * kThreads * per_thread > 0xFFFFFFFFll)
+        e = unpack ? cudaLaunchKernelEx(&cfg, pack_w4_kernel<int64_t, true, kPackChunks>, w8, ld8, total, V, w4, ld4)
+                   : cudaLaunchKernelEx(&cfg, pack_w4_kernel<int64_t, false, kPackChunks>, w8, ld8, total, V, w4, ld4);
+    else if (per_thread > 1)
+        e = unpack ? cudaLaunchKernelEx(&cfg, pack_w4_kernel<uint32_t, true, kPackChunks>, w8, ld8, uint32_t(total), V, w4, ld4)
+                   : cudaLaunchKernelEx(&cfg, pack_w4_kernel<uint32_t, false, kPackChunks>, w8, ld8, uint32_t(total), V, w4, ld4);
+    else
+        e = unpack ? cudaLaunchKernelEx(&cfg, pack_w4_kernel<uint32_t, true, 1>, w8, ld8, uint32_t(total), V, w4, ld4)
+                   : cudaLaunchKernelEx(&cfg, pack_w4_kernel<uint32_t, false, 1>, w8, ld8, uint32_t(total), V, w4, ld4);
     count_launch();
     if (e != cudaSuccess) { note_cuda_error(e); return SQ_ERR_CUDA; }
     return SQ_OK;

@@ -64,3 +64,19 @@ def test_small_zero_point_inputs_equal_rows_of_a_large_one():
     s_x, z_x = torch.tensor([0.02, 0.03], device=DEV), torch.tensor([-7, 100], dtype=torch.int32, device=DEV)
     whole = B.segquant_quantize_act_zero_point(X, seg, s_x, z_x)
     assert torch.equal(whole[40:47], B.segquant_quantize_act_zero_point(X[40:47], seg, s_x, z_x))
+
+
+@pytest.mark.parametrize("N,K", [(1, 16), (7, 48), (257, 4112), (3100, 4096), (2049, 7984)])
+def test_packed_codes_come_back(N, K):
+    """One and several chunks per thread, grids that the chunks do not fill, a row pitch wider than the row."""
+    g = torch.Generator(device=DEV).manual_seed(N)
+    codes = torch.randint(-8, 8, (N, K), generator=g, device=DEV, dtype=torch.int8)
+    w8 = B.new_codes(N, K, DEV)
+    w8.copy_(codes.view(torch.uint8))
+    w4 = B.segquant_pack_w4(w8)
+    low, high = codes[:, 0::2].to(torch.int32) & 15, codes[:, 1::2].to(torch.int32) & 15
+    assert torch.equal(w4.to(torch.int32), low | high << 4)
+    out = torch.full((N + 1, w8.stride(0)), 77, dtype=torch.uint8, device=DEV)
+    B.segquant_unpack_w4(w4, out=out[:N, :K])
+    assert torch.equal(out[:N, :K], codes.view(torch.uint8))
+    assert bool(torch.all(out[:N, K:] == 77)) and bool(torch.all(out[N] == 77))
