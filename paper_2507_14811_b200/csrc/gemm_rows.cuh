@@ -258,7 +258,10 @@ segquant_rows_kernel(const __grid_constant__ CUtensorMap tm_pos, const __grid_co
         }
         __syncwarp();
     } else {
-        if (SRC == 0) grid_dependency_wait();
+        // Every warp that reads global memory waits for the kernel in front itself, also where its inputs come through the producer's
+        // copies: the scales may be what that kernel computes (a calibration lets this launch start with its first instruction
+        // and writes them with its last).
+        grid_dependency_wait();
         if constexpr (SRC != 0) {
             // -------------------------------------------------------------- quantizer: this CTA's tokens x its K range
             // not unrolled, see the epilogue

@@ -109,3 +109,70 @@ def test_output_in_place_of_the_input():
     Y = X.clone()
     layer.forward(Y, Y)
     assert torch.equal(Y, ref)
+
+
+@pytest.mark.parametrize("M,K,kb", [(8, 1024, [0, 1024]), (8, 1056, [0, 320, 1056]), (256, 256, [0, 256]), (256, 288, [0, 96, 288])])
+@pytest.mark.parametrize("code,dual", [("int8", True), ("int8", False), ("e4m3", True), ("e4m3", False)])
+def test_scales_from_the_calibration_in_front(M, K, kb, code, dual):
+    """A layer that quantizes inside, queued right behind the calibration that writes its scales, with and without another
+    such layer between the two, eagerly, from a plan and in a graph: what it gives after a synchronization."""
+    layer, X = make(M, K, 136, kb, [0, 136], dual, code, BF16)
+    other, X_other = make(16, 512, 64, [0, 512], [0, 64], True, "int8", BF16)
+    g = torch.Generator(device=DEV).manual_seed(1)
+    batches = [torch.randn((40000, K), generator=g, device=DEV).to(BF16) * s for s in (1.0, 3.0)]
+    X_cal = torch.empty_like(batches[0])
+    calibrate = lambda batch: B.segquant_calib_scales_static(batch, layer.seg, code, False, dual, s_pos=layer.s_pos, s_neg=layer.s_neg)
+
+    def spoil():
+        for s in (layer.s_pos, layer.s_neg) if dual else (layer.s_pos,):
+            s.fill_(1e3)
+
+    try:
+        B.segquant_set_tuning(segment_mode=ROWS_FORM)
+        Y, Y_plan, Y_other = (torch.empty((m, n), dtype=BF16, device=DEV) for m, n in ((M, 136), (M, 136), (16, 64)))
+        plan = layer.plan(X, Y_plan)
+        want = []
+        for batch in batches:
+            calibrate(batch)
+            torch.cuda.synchronize()
+            want.append(layer.forward(X).clone())
+        assert not torch.equal(*want)
+        n = B.segquant_launch_count()
+        layer.forward(X, Y)
+        plan.run()
+        assert B.segquant_launch_count() == n + 2                        # one launch each
+        torch.cuda.synchronize()
+        for between in (False, True):
+            got = []
+            for i in range(6):
+                torch.cuda._sleep(400_000)                               # the calls below are queued before the first one starts
+                for run, out in ((lambda: layer.forward(X, Y), Y), (plan.run, Y_plan)):
+                    spoil()
+                    calibrate(batches[i % 2])
+                    if between:
+                        other.forward(X_other, Y_other)
+                    run()
+                    got.append((i % 2, out.clone()))
+            assert all(torch.equal(out, want[i]) for i, out in got), between
+
+        stream = torch.cuda.Stream()
+        stream.wait_stream(torch.cuda.current_stream())
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(stream):
+            with torch.cuda.graph(graph, stream=stream, capture_error_mode="relaxed"):
+                spoil()
+                calibrate(X_cal)
+                layer.forward(X, Y)
+                spoil()
+                calibrate(X_cal)
+                other.forward(X_other, Y_other)
+                plan.run()
+        torch.cuda.current_stream().wait_stream(stream)
+        for i in range(6):
+            X_cal.copy_(batches[i % 2])
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(Y, want[i % 2]) and torch.equal(Y_plan, want[i % 2])
+    finally:
+        B.segquant_set_tuning()
+    layer.check_status()
