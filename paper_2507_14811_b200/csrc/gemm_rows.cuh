@@ -295,11 +295,12 @@ segquant_rows_kernel(const __grid_constant__ CUtensorMap tm_pos, const __grid_co
                             asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "r"(src + 16u * v) : "memory");
                             set_piece(raw, v, w);
                         }
+                        if (KIND == 0 && NPOL == 2) bound16(raw);
 #pragma unroll
                         for (int g4 = 0; g4 < 4; g4++) {
                             float x[4];
                             get4(raw, g4, x);
-                            if (fast) quant4<KIND, MODE>(x, cp, cn, float(prm.q_hi), 0, wp[g4], wn[g4]);
+                            if (fast) quant4<KIND, MODE, kBounded<Tin>>(x, cp, cn, float(prm.q_hi), 0, wp[g4], wn[g4]);
                         }
                         if (!fast) {
 #pragma unroll 1

@@ -278,6 +278,7 @@ quantize_kernel(const __grid_constant__ QuantParams prm)
         }
         if (fast) {
             uint32_t wp[4], wn[4];
+            if constexpr (PRE == 0 && DUAL && CODE == SQ_CODE_INT8) bound16(cur);
 #pragma unroll
             for (int g4 = 0; g4 < 4; g4++) {
                 float x[4];
@@ -300,7 +301,7 @@ quantize_kernel(const __grid_constant__ QuantParams prm)
                     for (int i = 0; i < 4; i += 2)
                         unpack2(pre2<Tin>(x[i], x[i + 1], prm.act, mreg[PRE ? 2 * g4 + i / 2 : 0]), x[i], x[i + 1]);
                 }
-                quant4<CODE, MODE>(x, cp, cn, float(hi), zp, wp[g4], wn[g4]);
+                quant4<CODE, MODE, PRE == 0 && kBounded<Tin>>(x, cp, cn, float(hi), zp, wp[g4], wn[g4]);
             }
             *reinterpret_cast<uint4 *>(dp) = make_uint4(wp[0], wp[1], wp[2], wp[3]);
             if (DUAL) *reinterpret_cast<uint4 *>(dn) = make_uint4(wn[0], wn[1], wn[2], wn[3]);
@@ -857,7 +858,7 @@ quantize_per_row_kernel(const Tin *__restrict__ X, int K, int64_t ld, const SegB
                 for (int g4 = 0; g4 < 4; g4++) {
                     float x[4];
                     get4(raw[c], g4, x);
-                    quant4<SQ_CODE_INT8, MODE>(x, cp, cn, float(hi), 0, wp[g4], wn[g4]);
+                    quant4<SQ_CODE_INT8, MODE, true>(x, cp, cn, float(hi), 0, wp[g4], wn[g4]);
                 }
                 *reinterpret_cast<uint4 *>(dp) = make_uint4(wp[0], wp[1], wp[2], wp[3]);
                 if (DUAL) *reinterpret_cast<uint4 *>(dn) = make_uint4(wn[0], wn[1], wn[2], wn[3]);

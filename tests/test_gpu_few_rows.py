@@ -176,3 +176,18 @@ def test_scales_from_the_calibration_in_front(M, K, kb, code, dual):
     finally:
         B.segquant_set_tuning()
     layer.check_status()
+
+
+@pytest.mark.parametrize("code,dual", [("int8", True), ("int8", False), ("e4m3", True)])
+def test_infinite_inputs(code, dual):
+    layer, X = make(24, 288, 40, [0, 96, 288], [0, 40], dual, code, F32)
+    X[::3, ::7], X[1::3, ::5] = float("inf"), -float("inf")
+    outs = []
+    try:
+        for mode in (TILE_FORM, ROWS_FORM):
+            B.segquant_set_tuning(segment_mode=mode)
+            outs.append(layer.forward(X, y_dtype=F32))
+            outs.append(layer.forward(X.clamp(torch.finfo(F32).min, torch.finfo(F32).max), y_dtype=F32))
+    finally:
+        B.segquant_set_tuning()
+    assert all(torch.equal(o, outs[0]) for o in outs) and bool(torch.all(outs[0].isfinite()))

@@ -80,3 +80,37 @@ def test_packed_codes_come_back(N, K):
     B.segquant_unpack_w4(w4, out=out[:N, :K])
     assert torch.equal(out[:N, :K], codes.view(torch.uint8))
     assert bool(torch.all(out[:N, K:] == 77)) and bool(torch.all(out[N] == 77))
+
+
+@pytest.mark.parametrize("code,dual", [("int8", True), ("int8", False), ("e4m3", True), ("e4m3", False)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("M,kb", [(40, [0, 520, 1056]), (6000, [0, 520, 1056]), (6000, [0, 512, 1056])])
+def test_infinities_saturate(M, kb, dtype, code, dual):
+    """Infinite inputs, and infinities that a gated product or a multiplier makes of finite ones, get the ends of the code
+    range: in whole chunks and in those that a segment bound cuts, with few and many elements a thread, by table."""
+    K = kb[-1]
+    big = torch.finfo(dtype).max
+    g = torch.Generator(device=DEV).manual_seed(M)
+    x = torch.randn((M, K), generator=g, device=DEV)
+    pick = torch.randint(0, 8, (M, K), generator=g, device=DEV)
+    seg = B.SegTable(kb, [0, 8])
+    sp = torch.tensor([0.02, 0.03], device=DEV)
+    sn = sp * 0.5 if dual else None
+    put = lambda t, v: torch.where(pick == 0, v, torch.where(pick == 1, -v, t)).to(dtype)
+    ends = (0x7F, 0x80 if dual else 0x81) if code == "int8" else (0x7E, 0xFE)
+
+    def check(codes):
+        for at, pos, neg in ((pick == 0, ends[0], 0), (pick == 1, 0 if dual else ends[1], ends[1])):
+            assert bool(torch.all(codes[0][at] == pos)) and (not dual or bool(torch.all(codes[1][at] == neg)))
+
+    check(B.segquant_quantize_act(put(x, float("inf")), seg, sp, sn, code))
+    check(B.segquant_quantize_act_fused(put(x, big), seg, sp, sn, code, None, torch.full((K,), 4.0, device=DEV)))
+    gated = torch.cat([put(x, big), put(x, 8.0).abs()], 1)               # GELU(8) = 8: the product overflows
+    for mode in (1, 2):
+        check(by_mode(mode, gated, seg, sp, sn, code, "geglu"))
+    if code == "int8" and dual:
+        fused = put(x, big).abs()                                        # (no pre-activation has a large negative SiLU or GELU)
+        for act in ("silu", "gelu"):
+            for mode in (1, 2):
+                c_pos, c_neg = by_mode(mode, fused, seg, sp, sn, code, act, torch.full((K,), 4.0, device=DEV))
+                assert bool(torch.all(c_pos[pick < 2] == 0x7F)) and bool(torch.all(c_neg[pick < 2] == 0))
