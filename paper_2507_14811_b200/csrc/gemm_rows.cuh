@@ -264,7 +264,8 @@ segquant_rows_kernel(const __grid_constant__ CUtensorMap tm_pos, const __grid_co
         grid_dependency_wait();
         if constexpr (SRC != 0) {
             // -------------------------------------------------------------- quantizer: this CTA's tokens x its K range
-            // not unrolled, see the epilogue
+            // not unrolled, see the epilogue.  (Each CTA quantizes for itself, so an element by itself and a division each, as the
+            // quantize kernel has for a bound of -127, would count many times: 8 x 976 -> 616 dual took 7.9 us, 6.5 in two kernels.)
             constexpr int MODE = NPOL == 2 ? kDual : kSingle;
             int cur_p = p_first;
             SegConst cp = seg_const(__ldg(prm.s_pos + cur_p)), cn = seg_const(NPOL == 2 ? __ldg(prm.s_neg + cur_p) : 1.0f);
@@ -287,7 +288,7 @@ segquant_rows_kernel(const __grid_constant__ CUtensorMap tm_pos, const __grid_co
                             cp = seg_const(__ldg(prm.s_pos + cur_p));
                             cn = seg_const(NPOL == 2 ? __ldg(prm.s_neg + cur_p) : 1.0f);
                         }
-                        const bool fast = cp.fast && cn.fast && !(NPOL == 2 && KIND == 0 && prm.q_lo != -128);
+                        const bool fast = cp.fast && cn.fast;
                         Raw16<Tin> raw;
 #pragma unroll
                         for (int v = 0; v < int(sizeof(Tin)); v++) {
@@ -301,6 +302,10 @@ segquant_rows_kernel(const __grid_constant__ CUtensorMap tm_pos, const __grid_co
                             float x[4];
                             get4(raw, g4, x);
                             if (fast) quant4<KIND, MODE, kBounded<Tin>>(x, cp, cn, float(prm.q_hi), 0, wp[g4], wn[g4]);
+                        }
+                        if (KIND == 0 && NPOL == 2 && prm.q_lo != -128) {      // a negative bound of -127: -128 becomes -127
+#pragma unroll
+                            for (int g4 = 0; g4 < 4; g4++) wn[g4] = __vmaxs4(wn[g4], 0x81818181u);
                         }
                         if (!fast) {
 #pragma unroll 1

@@ -191,3 +191,24 @@ def test_infinite_inputs(code, dual):
     finally:
         B.segquant_set_tuning()
     assert all(torch.equal(o, outs[0]) for o in outs) and bool(torch.all(outs[0].isfinite()))
+
+
+@pytest.mark.parametrize("M,K,kb,x_dtype", [(5, 528, [0, 528], BF16), (40, 1152, [0, 64, 96, 1152], F32), (256, 256, [0, 256], BF16)])
+def test_symmetric_code_range(M, K, kb, x_dtype):
+    """A negative bound of -127 (SQ_FLAG_QMIN_SYM), with inputs that a bound of -128 would not clip to it."""
+    layer, X = make(M, K, 136, kb, [0, 136], True, "int8", x_dtype)
+    layer.flags = B.SQ_FLAG_QMIN_SYM
+    layer.calibrate(X * 0.9)
+    _, c_neg = B.segquant_quantize_act(X, layer.seg, layer.s_pos, layer.s_neg, "int8", layer.flags)
+    _, c_128 = B.segquant_quantize_act(X, layer.seg, layer.s_pos, layer.s_neg, "int8")
+    assert not bool(torch.any(c_neg == 0x80)) and bool(torch.any(c_128 == 0x80))
+    outs = []
+    try:
+        for mode, launches in ((TILE_FORM, 2), (ROWS_FORM, 1)):
+            B.segquant_set_tuning(segment_mode=mode)
+            n = B.segquant_launch_count()
+            outs.append(layer.forward(X, y_dtype=F32))
+            assert B.segquant_launch_count() == n + launches
+    finally:
+        B.segquant_set_tuning()
+    assert torch.equal(*outs)
