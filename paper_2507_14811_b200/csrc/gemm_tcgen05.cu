@@ -1976,15 +1976,20 @@ static double tile_form_cost(const GemmArgs &g, int npol, const TilePlan &t, int
            (t.seq ? waves * g.sb.P * (0.308 + 0.159 * w) : waves * g.sb.P * w * 0.905) + (t.cg == 2 ? 1.57 : 0.0);
 }
 
+// Whether any word of segquant_set_tuning is set: then only segment mode 8 takes the GEMM of few rows, where they have a meaning of their own.
+static bool tuned()
+{
+    return g_tune_tile_n.load(std::memory_order_relaxed) || g_tune_stages.load(std::memory_order_relaxed) ||
+           g_tune_cta_group.load(std::memory_order_relaxed) || g_tune_seq.load(std::memory_order_relaxed);
+}
+
 constexpr int kFewRows = 512;          // rows up to which the GEMM of few rows is considered at all
 
 sq_status prepare_fused_layer(const GemmArgs &g, GemmLaunch *out)
 {
     int dev = 0, sm_count = 0;
-    const int tune_seq = g_tune_seq.load(std::memory_order_relaxed);
-    const bool automatic = !tune_seq && !g_tune_tile_n.load(std::memory_order_relaxed) && !g_tune_cta_group.load(std::memory_order_relaxed) &&
-                           !g_tune_stages.load(std::memory_order_relaxed);
-    if (!(tune_seq == kSegmentModeRows || (automatic && g.M <= kFusedRows))) return SQ_ERR_UNSUPPORTED;
+    const bool forced = g_tune_seq.load(std::memory_order_relaxed) == kSegmentModeRows, automatic = !tuned();
+    if (!(forced || (automatic && g.M <= kFusedRows))) return SQ_ERR_UNSUPPORTED;
     if (cudaGetDevice(&dev) != cudaSuccess) return SQ_ERR_CUDA;
     if (cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sm_count <= 0)
         return SQ_ERR_CUDA;
@@ -2022,9 +2027,8 @@ sq_status prepare_gemm(const GemmArgs &g, GemmLaunch *out)
     L.threads = kThreads;
     if (prm.nacc * g.sb.Q > kMaxFactorTable) return SQ_ERR_UNSUPPORTED;
     const TilePlan t = tile_plan(g, npol, sm_count);
-    const int tune_seq = g_tune_seq.load(std::memory_order_relaxed);
-    const bool automatic = !tune_seq && !g_tune_tile_n.load(std::memory_order_relaxed) && !g_tune_cta_group.load(std::memory_order_relaxed);
-    if (tune_seq == kSegmentModeRows || (automatic && g.M <= kFewRows)) {
+    const bool forced = g_tune_seq.load(std::memory_order_relaxed) == kSegmentModeRows, automatic = !tuned();
+    if (forced || (automatic && g.M <= kFewRows)) {
         const double limit = automatic ? rows_gain(g.M, g.K, false) * tile_form_cost(g, npol, t, sm_count) : 1e9;
         const sq_status fr = limit > 0.0 ? prepare_few_rows(g, L, limit, dev, sm_count) : SQ_ERR_UNSUPPORTED;
         if (fr != SQ_ERR_UNSUPPORTED) return fr;

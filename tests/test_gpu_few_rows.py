@@ -3,6 +3,7 @@ quantized inside): bit for bit the results of the tile form, which the parity te
 terms in the same order: int8 sums are exact however a K range is split, e4m3 ones are never split."""
 import pytest
 import torch
+from cuda.bindings import driver
 
 from paper_2507_14811_b200 import binding as B
 from paper_2507_14811_b200.layer import SegQuantLinear
@@ -28,6 +29,31 @@ def gemm(layer, codes, y_dtype, dump=False):
                                          layer.bias, layer.workspace, y_dtype=y_dtype, dump_acc=dump)
     return B.segquant_seglinear_gemm(c_pos, layer.Wq, layer.seg, layer.code, layer.s_pos, layer.s_w, layer.bias, layer.workspace,
                                      y_dtype=y_dtype, dump_acc=dump)
+
+
+TILE_THREADS, ROWS_THREADS = 384, 320
+
+
+def gemm_forms(fn):
+    """Block sizes of the GEMM kernels that fn launches, from the nodes of a graph it is captured into (nothing runs)."""
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.stream(stream):
+        graph.capture_begin(capture_error_mode="relaxed")
+        fn()
+        graph.capture_end()
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    err, _, count = driver.cuGraphGetNodes(raw)
+    err, nodes, _ = driver.cuGraphGetNodes(raw, count)
+    assert err == driver.CUresult.CUDA_SUCCESS
+    threads = []
+    for node in nodes:
+        if driver.cuGraphNodeGetType(node)[1] == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            err, params = driver.cuGraphKernelNodeGetParams(node)
+            assert err == driver.CUresult.CUDA_SUCCESS
+            threads.append(params.blockDimX)
+    return [t for t in threads if t in (TILE_THREADS, ROWS_THREADS)]
 
 
 @pytest.mark.parametrize("case", [
@@ -212,3 +238,21 @@ def test_symmetric_code_range(M, K, kb, x_dtype):
     finally:
         B.segquant_set_tuning()
     assert torch.equal(*outs)
+
+
+@pytest.mark.parametrize("tuning,form", [({}, ROWS_THREADS), ({"segment_mode": ROWS_FORM}, ROWS_THREADS), ({"stages": 4}, TILE_THREADS),
+                                         ({"tile_n": 64}, TILE_THREADS), ({"cta_group": 1}, TILE_THREADS),
+                                         ({"segment_mode": TILE_FORM}, TILE_THREADS)])
+def test_tuning_words_keep_the_tile_form(tuning, form):
+    """Any of them asks for the tile form, whose dimensions they are, in the GEMM alone and in a layer call."""
+    layer, X = make(2, 8192, 640, [0, 8192], [0, 640], True, "int8", BF16)
+    codes = B.segquant_quantize_act(X, layer.seg, layer.s_pos, layer.s_neg, "int8")
+    ref = gemm(layer, codes, BF16)
+    try:
+        B.segquant_set_tuning(**tuning)
+        Y = layer.forward(X)
+        y = gemm(layer, codes, BF16)
+        assert gemm_forms(lambda: layer.forward(X)) == gemm_forms(lambda: gemm(layer, codes, BF16)) == [form]
+    finally:
+        B.segquant_set_tuning()
+    assert torch.equal(Y, ref) and torch.equal(y, ref)
