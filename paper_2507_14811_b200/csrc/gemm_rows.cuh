@@ -635,6 +635,38 @@ bool rows_layout(const GemmArgs &g, const RowsShape &sh, int sm_count, RowsParam
     return true;
 }
 
+// Where the model above falls short of the tile form's, in microseconds on top of it for a shape that has been picked.  900 layers of
+// 1 .. 512 rows, GEMM alone, time here over time of the tile form; K-blocks are cut where a segment ends inside their ring
+// stage, and are then issued MMA by MMA, which shows unless the weights take longer to arrive:
+//   at least 12 cut blocks a CTA, one polarity: 0.86 .. 1.12, 1.00 in the median of 12 layers (8448 wide in 22 segments, 101 rows, 25.6 / 22.8);
+//   at least 28, two polarities of e4m3, whose K range is not split: 1.06 .. 1.21 (4992 in 13 segments, 4 rows, 16.2 / 13.9);
+//   with fewer, or of int8, 0.75 .. 0.93 (nine in ten);
+//   one polarity, several token tiles, each of which reads the weights: 1.00 .. 1.20 for 20 MB of weights and more where the tile
+//   form's 128-column tiles occupy 64 SMs (42 x 8016 -> 8936 19.7 / 16.4), 0.63 .. 0.95 where they do not (31 x 10192 -> 3392).
+template <int KIND, int NPOL>
+double rows_shortfall(const GemmArgs &g, const RowsParams &r, unsigned grid)
+{
+    if (NPOL == 1 && r.num_m > 1 && g.M <= TILE_M && g.N >= 64 * 128 && double(g.N) * double(g.K) >= 20e6) return 1e9;
+    const int64_t stage = int64_t(r.stage_blocks) * BLOCK_K;
+    int most = 0;
+    for (int i = 0; i < r.split; i++) {
+        const int kb0 = i * r.kblocks / r.split, kb1 = (i + 1) * r.kblocks / r.split;
+        int64_t last = -1;
+        int cut = 0;
+        for (int p = r.rank_p0[i] + 1; p <= r.rank_p1[i]; p++) {
+            const int64_t off = g.sb.kb[p] - int64_t(kb0) * BLOCK_K;
+            if (off % stage == 0 || off / stage == last) continue;
+            last = off / stage;
+            cut += std::min(r.stage_blocks, kb1 - kb0 - int(last) * r.stage_blocks);
+        }
+        most = std::max(most, cut);
+    }
+    if (most < (NPOL == 1 ? 12 : 28) || (NPOL == 2 && KIND == 0)) return 0.0;
+    const int per_m = int(grid) / r.num_m / r.split, tiles = (r.num_n + per_m - 1) / per_m;
+    const double idle = 0.183e-6 * double(g.N) * double(g.K) - 0.133 * tiles * r.kblocks / r.split;        // the issuing loop's, uncut
+    return std::max(0.0, (NPOL == 1 ? 0.16 : 0.12) * most * tiles - std::max(0.0, idle));
+}
+
 // The best shape for a layer and the time the model gives it; false where none fits.  Working it out takes some microseconds,
 // so a thread keeps what it has decided for the last few layers (a function of their sizes and segment bounds alone).
 template <int KIND, int NPOL>
@@ -680,6 +712,13 @@ bool rows_plan(const GemmArgs &g, int sm_count, RowsShape *shape, double *cost)
                 *cost = c;
                 *shape = {tokens, rows, split};
             }
+    }
+    if (found && !forced) {
+        RowsParams r{};
+        size_t smem = 0;
+        unsigned grid = 0;
+        rows_layout<KIND, NPOL>(g, *shape, sm_count, &r, &smem, &grid, cost);
+        *cost += rows_shortfall<KIND, NPOL>(g, r, grid);
     }
     if (!forced) {
         Decision &d = kept[turn++ % kKept];

@@ -91,7 +91,13 @@ constexpr uint32_t kStageBytesPerWarp = 32 * 64;       // one 32 x 32 bf16 outpu
 [[maybe_unused]] constexpr uint32_t kStageBytes = kEpiWarps * kStageBytesPerWarp;
 // The GEMM of few rows is taken below this share of the expected time of the tile form (the models' margin; beyond 128 rows that
 // of the tile form is off by up to a quarter), for the GEMM alone or for a whole layer whose activations it quantizes itself
-// against a quantize kernel (1.9 us on a few rows) and the better of the two GEMMs.
+// against a quantize kernel and the better of the two GEMMs.  A quantize kernel moves the end of a layer by 1.1 .. 2.0 us on up to
+// 128 rows, 1.2 .. 3.4 beyond; it also costs the host 2.7 us in an eager call, so it is counted high.
+// Shares: of 580 layers, GEMM alone, 0.92 and 0.70 leave 19 slower than the tile form by more than 3 % (with rows_shortfall 6) at
+// 0.90 of its time on average; 0.97 and 0.90 win another 2 % on average and lose 5 % and more on one layer in forty.
+// Quantizing inside, beyond 128 rows, over the two launches taken otherwise (median, worst; K 256, 384, 512, 768, 1024): 192 .. 256 rows 0.98
+// 1.00, 1.08 1.34, 1.05 1.12, 1.17 1.23, 1.20 1.30; 257 .. 320 rows 1.05 1.12, 1.08 1.39, 1.12 1.19, 1.14 1.23, 1.19 1.30: every
+// CTA quantizes its tokens again for each of its column tiles.  Hence kFusedRows, and the wider margin where K is long.
 [[maybe_unused]] constexpr double kQuantizeLaunch = 1.9;
 [[maybe_unused]] inline double rows_gain(int64_t M, int64_t K, bool fused) { return M <= TILE_M ? 0.92 : fused && K <= 512 ? 0.80 : 0.70; }
 constexpr int kMaxTokenSegments = 32;                  // per-token layers: channel scales of up to 32 K-segments (32 KiB at 256 columns) are staged per tile

@@ -256,3 +256,20 @@ def test_tuning_words_keep_the_tile_form(tuning, form):
     finally:
         B.segquant_set_tuning()
     assert torch.equal(Y, ref) and torch.equal(y, ref)
+
+
+@pytest.mark.parametrize("M,K,N,P,code,dual,form", [
+    (4, 4992, 424, 13, "e4m3", True, TILE_THREADS), (4, 2496, 424, 13, "e4m3", True, ROWS_THREADS),    # blocks that K-segments cut
+    (101, 8448, 1008, 22, "e4m3", False, TILE_THREADS), (38, 3520, 1880, 22, "int8", True, ROWS_THREADS),
+    (42, 8016, 8936, 1, "int8", False, TILE_THREADS), (31, 10192, 3392, 2, "int8", False, ROWS_THREADS),    # weights read per token tile
+])
+def test_layers_that_the_tile_form_takes_in_less_time(M, K, N, P, code, dual, form):
+    layer, X = make(M, K, N, [K * p // P // 32 * 32 for p in range(P)] + [K], [0, N], dual, code, BF16)
+    codes = B.segquant_quantize_act(X, layer.seg, layer.s_pos, layer.s_neg, code)
+    Y = gemm(layer, codes, BF16)
+    assert gemm_forms(lambda: gemm(layer, codes, BF16)) == [form]
+    try:
+        B.segquant_set_tuning(segment_mode=TILE_FORM)
+        assert torch.equal(gemm(layer, codes, BF16), Y)
+    finally:
+        B.segquant_set_tuning()
