@@ -533,6 +533,10 @@ struct RowsShape { int tile_tokens, tile_rows, split; };
 // Shared memory that a CTA with that many columns of tensor memory has to ask for at least (see the top of this file).
 inline size_t smem_for_columns(int cols) { return size_t(228) * 1024 * cols / 512 - 1024; }
 
+// Microseconds of the model below that no shape avoids: the start and end of a launch, and the weights from memory.
+[[maybe_unused]] constexpr double kRowsStart = 2.64, kRowsByteTime = 0.183e-6;
+inline double rows_floor(const GemmArgs &g) { return kRowsStart + kRowsByteTime * double(g.N) * double(g.K); }
+
 // Works out a launch of the given shape; false where it does not fit.  *cost: estimated cycles, for rows_plan.
 template <int KIND, int NPOL>
 bool rows_layout(const GemmArgs &g, const RowsShape &sh, int sm_count, RowsParams *out, size_t *smem, unsigned *grid, double *cost)
@@ -626,11 +630,11 @@ bool rows_layout(const GemmArgs &g, const RowsShape &sh, int sm_count, RowsParam
     const double quant = fused ? (KIND == 0 ? 0.31 : 0.49) + 0.4675 * ((r.tile_tokens * longest * 8 + 255) / 256) * busy : 0.0;
     const double per_block = std::max((r.stage_blocks == 4 ? 0.133 : r.stage_blocks == 2 ? 0.164 : 0.262) + 1.75e-4 * r.ncols * per_sm_now,
                                       6.8e-6 * bytes * per_sm_now);
-    const double chain = blocks * per_block + waves * quant, memory = 0.183e-6 * double(g.N) * double(g.K) + (fused ? 0.27 : 0.0);
+    const double chain = blocks * per_block + waves * quant, memory = kRowsByteTime * double(g.N) * double(g.K) + (fused ? 0.27 : 0.0);
     const double stream = std::max(std::max(memory, chain), 0.04e-6 * resident * blocks * bytes + quant);
     const double epi = 0.148 * most * NPOL * g16 * busy_half + 0.157 * g16;
     const double comb = split > 1 ? 0.894 + 0.129 * pieces * NPOL * (((r.tile_tokens + split - 1) / split + 7) / 8) + 0.082 * most * NPOL * g16 : 0.0;
-    *cost = 2.64 + stream + waves * (tiles_per_cta * epi + comb) + (waves - 1) * 2.95;
+    *cost = kRowsStart + stream + waves * (tiles_per_cta * epi + comb) + (waves - 1) * 2.95;
     r.ahead = int(std::min<double>(longest, std::max(0.0, std::ceil(kRowsAheadBytes / (double(*grid) * r.tile_rows * BLOCK_K)))));
     return true;
 }
@@ -663,73 +667,79 @@ double rows_shortfall(const GemmArgs &g, const RowsParams &r, unsigned grid)
     }
     if (most < (NPOL == 1 ? 12 : 28) || (NPOL == 2 && KIND == 0)) return 0.0;
     const int per_m = int(grid) / r.num_m / r.split, tiles = (r.num_n + per_m - 1) / per_m;
-    const double idle = 0.183e-6 * double(g.N) * double(g.K) - 0.133 * tiles * r.kblocks / r.split;        // the issuing loop's, uncut
+    const double idle = kRowsByteTime * double(g.N) * double(g.K) - 0.133 * tiles * r.kblocks / r.split;        // the issuing loop's, uncut
     return std::max(0.0, (NPOL == 1 ? 0.16 : 0.12) * most * tiles - std::max(0.0, idle));
 }
 
-// The best shape for a layer and the time the model gives it; false where none fits.  Working it out takes some microseconds,
-// so a thread keeps what it has decided for the last few layers (a function of their sizes and segment bounds alone).
+// The best shape for a layer and the time the models give it; false where none fits.  Working it out takes 1.2 (8 rows) to 6.2 us
+// (250 rows) of a call that takes 5 to 10, so a thread keeps what it has decided, a function of sizes and segment bounds alone.
+// An eager call asks two or three times (quantizing inside or not), so 256 decisions serve some eighty layers in rotation.
+struct RowsKey {
+    int64_t M, N, K;
+    int P, Q, fused, x_f32, per_token, sm_count;
+    uint16_t kb[SQ_MAX_P + 1];           // interior bounds are multiples of 32, K of 16 and at most 131072
+    bool operator==(const RowsKey &o) const
+    {
+        return M == o.M && N == o.N && K == o.K && P == o.P && Q == o.Q && fused == o.fused && x_f32 == o.x_f32 &&
+               per_token == o.per_token && sm_count == o.sm_count && std::equal(kb, kb + P + 1, o.kb);
+    }
+    uint32_t hash() const
+    {
+        int64_t w[8 + SQ_MAX_P] = {M, N, K, int64_t(P) << 32 | Q, fused << 2 | x_f32 << 1 | per_token, sm_count};
+        size_t n = 6;
+        for (int p = 1; p < P; p++) w[n++] = kb[p];
+        return hash_words(w, n);
+    }
+};
+struct RowsDecision {
+    bool found;
+    RowsShape shape;
+    double cost;
+};
+
 template <int KIND, int NPOL>
-bool rows_plan(const GemmArgs &g, int sm_count, RowsShape *shape, double *cost)
+RowsDecision rows_search(const GemmArgs &g, int sm_count, bool forced)
 {
-    struct Decision {
-        int64_t M, N, K;
-        int P, Q, fused, x_f32, per_token, sm_count;
-        int kb[SQ_MAX_P + 1];
-        int found;
-        RowsShape shape;
-        double cost;
-    };
-    constexpr unsigned kKept = 16;
-    thread_local Decision kept[kKept];
-    thread_local unsigned turn = 0;
-    const int fused = g.X != nullptr, x_f32 = fused && g.x_dtype == SQ_F32, per_token = g.col_scale != nullptr;
-    const bool forced = g_tune_seq.load(std::memory_order_relaxed) == kSegmentModeRows;
+    RowsDecision best{};
     const int f_rows = forced ? g_tune_tile_n.load(std::memory_order_relaxed) : 0, f_tokens = forced ? g_tune_stages.load(std::memory_order_relaxed) : 0,
               f_split = forced ? g_tune_cta_group.load(std::memory_order_relaxed) : 0;
-    for (unsigned i = 0; i < kKept && !forced; i++) {
-        const Decision &d = kept[i];
-        if (d.M == g.M && d.N == g.N && d.K == g.K && d.P == g.sb.P && d.Q == g.sb.Q && d.fused == fused && d.x_f32 == x_f32 &&
-            d.per_token == per_token && d.sm_count == sm_count && std::equal(d.kb, d.kb + d.P + 1, g.sb.kb)) {
-            *shape = d.shape;
-            *cost = d.cost;
-            return d.found != 0;
-        }
-    }
-    bool found = false;
+    RowsParams r{};
+    size_t smem = 0;
+    unsigned grid = 0;
     for (int tokens : {8, 16, 32, 64, 128, 256}) {
         if (tokens > 8 && tokens / 2 >= g.M && !forced) break;
         for (int rows : {128, 96, 64, 32})
             for (int split : {1, 2, 4, 8}) {
                 if ((f_rows && rows != f_rows) || (f_tokens && tokens != f_tokens) || (f_split && split != f_split)) continue;
-                RowsParams r{};
-                size_t smem = 0;
-                unsigned grid = 0;
                 double c = 0.0;
                 if (!rows_layout<KIND, NPOL>(g, {tokens, rows, split}, sm_count, &r, &smem, &grid, &c)) continue;
-                if (found && c >= *cost) continue;
-                found = true;
-                *cost = c;
-                *shape = {tokens, rows, split};
+                if (best.found && c >= best.cost) continue;
+                best = {true, {tokens, rows, split}, c};
             }
     }
-    if (found && !forced) {
-        RowsParams r{};
-        size_t smem = 0;
-        unsigned grid = 0;
-        rows_layout<KIND, NPOL>(g, *shape, sm_count, &r, &smem, &grid, cost);
-        *cost += rows_shortfall<KIND, NPOL>(g, r, grid);
+    if (best.found && !forced) {
+        rows_layout<KIND, NPOL>(g, best.shape, sm_count, &r, &smem, &grid, &best.cost);
+        best.cost += rows_shortfall<KIND, NPOL>(g, r, grid);
     }
-    if (!forced) {
-        Decision &d = kept[turn++ % kKept];
-        d.M = g.M; d.N = g.N; d.K = g.K;
-        d.P = g.sb.P; d.Q = g.sb.Q; d.fused = fused; d.x_f32 = x_f32; d.per_token = per_token; d.sm_count = sm_count;
-        std::copy(g.sb.kb, g.sb.kb + g.sb.P + 1, d.kb);
-        d.found = found;
-        d.shape = found ? *shape : RowsShape{};
-        d.cost = found ? *cost : 0.0;
-    }
-    return found;
+    return best;
+}
+
+template <int KIND, int NPOL>
+RowsDecision rows_plan(const GemmArgs &g, int sm_count)
+{
+    if (g_tune_seq.load(std::memory_order_relaxed) == kSegmentModeRows) return rows_search<KIND, NPOL>(g, sm_count, true);
+    thread_local Recent<RowsKey, RowsDecision, 8, 32> kept;
+    RowsKey key{};
+    key.M = g.M; key.N = g.N; key.K = g.K;
+    key.P = g.sb.P; key.Q = g.sb.Q;
+    key.fused = g.X != nullptr;
+    key.x_f32 = key.fused && g.x_dtype == SQ_F32;
+    key.per_token = g.col_scale != nullptr;
+    key.sm_count = sm_count;
+    for (int p = 0; p <= g.sb.P; p++) key.kb[p] = uint16_t(g.sb.kb[p] / 16);
+    const uint32_t hash = key.hash();
+    if (const RowsDecision *d = kept.find(hash, key)) return *d;
+    return kept.keep(hash, key, rows_search<KIND, NPOL>(g, sm_count, false));
 }
 
 template <int KIND, int NPOL>
@@ -737,17 +747,18 @@ sq_status prepare_rows_t(const GemmArgs &g, GemmLaunch &L, double limit, int dev
 {
     RowsParams &r = L.rows;
     r = RowsParams{};
-    RowsShape shape{};
-    double cost = 0.0;
-    if (!rows_plan<KIND, NPOL>(g, sm_count, &shape, &cost) || cost >= limit) return SQ_ERR_UNSUPPORTED;
-    if (g.X && g_tune_seq.load(std::memory_order_relaxed) != kSegmentModeRows) {      // quantizing here also has to beat this form behind a quantizer of its own
+    const bool forced = g_tune_seq.load(std::memory_order_relaxed) == kSegmentModeRows;
+    if (!forced && rows_floor(g) >= limit) return SQ_ERR_UNSUPPORTED;      // no shape can be the better one: nothing to search
+    const RowsDecision d = rows_plan<KIND, NPOL>(g, sm_count);
+    if (!d.found || d.cost >= limit) return SQ_ERR_UNSUPPORTED;
+    if (g.X && !forced) {      // quantizing here also has to beat this form behind a quantizer of its own
         GemmArgs codes = g;
         codes.X = nullptr;
-        double apart = 0.0;
-        if (rows_plan<KIND, NPOL>(codes, sm_count, &shape, &apart) && cost >= rows_gain(g.M, g.K, true) * (apart + kQuantizeLaunch)) return SQ_ERR_UNSUPPORTED;
-        rows_plan<KIND, NPOL>(g, sm_count, &shape, &cost);
+        const RowsDecision apart = rows_plan<KIND, NPOL>(codes, sm_count);
+        if (apart.found && d.cost >= rows_gain(g.M, g.K, true) * (apart.cost + kQuantizeLaunch)) return SQ_ERR_UNSUPPORTED;
     }
-    rows_layout<KIND, NPOL>(g, shape, sm_count, &r, &L.smem, &L.grid, &cost);
+    double cost = 0.0;
+    rows_layout<KIND, NPOL>(g, d.shape, sm_count, &r, &L.smem, &L.grid, &cost);
     r.M = int(g.M); r.N = int(g.N); r.K = int(g.K);
     r.sb = g.sb;
     r.s_pos = g.s_pos; r.s_neg = g.s_neg; r.s_w = g.s_w; r.bias = g.bias;

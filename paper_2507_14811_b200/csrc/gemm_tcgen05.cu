@@ -41,6 +41,7 @@
 #include <cstddef>
 #include <type_traits>
 #include "quant_codes.cuh"
+#include "recent.h"
 
 namespace sq {
 
