@@ -13,7 +13,7 @@
 // shared memory, kept for all its tiles) while the first weights are on their way: one launch per layer and no code matrices.
 //   warps 0..7  quantizer (SRC != 0), then epilogue: thread = output channel, two groups of four warps share the tokens
 //   warp 8      TMA producer; warp 9 MMA issuer and owner of the tensor memory
-// A CTA asks for at most 112 KiB of shared memory where it can, so that two share an SM and the set-up of one launch runs
+// A CTA asks for at most 113 KiB of shared memory where it can, so that two share an SM and the set-up of one launch runs
 // under the end of the one before.  Two resident CTAs must never ask for more than the 512 columns of tensor memory an SM
 // has: one would wait for the other, and with clusters round in a circle.  Hence smem_for_columns: shared memory grows with
 // the columns so that what fits in shared memory fits in tensor memory, too.
@@ -82,7 +82,7 @@ segquant_rows_kernel(const __grid_constant__ CUtensorMap tm_pos, const __grid_co
     if (prm.red_alias) sh_red = smem;                   // the ring's memory, free once every MMA of the cluster has retired
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int split = prm.split;
+    const int split = KIND == 0 ? prm.split : 1;        // e4m3: no exchange is compiled
     const uint32_t rank = split > 1 ? cluster_rank() : 0u;
     const int unit = int(blockIdx.x) / split, units = int(gridDim.x) / split;
     const int mt = unit % prm.num_m, m0 = mt * prm.tile_tokens;
@@ -478,7 +478,7 @@ segquant_rows_kernel(const __grid_constant__ CUtensorMap tm_pos, const __grid_co
 #pragma unroll
                             for (int j = 0; j < T; j++) {
                                 const uint32_t v = tl0 + j < tokens ? red[j * prm.tile_rows] : 0u;
-                                acc[pol][j] = fresh ? v : KIND == 0 ? acc[pol][j] + v : __float_as_uint(__uint_as_float(acc[pol][j]) + __uint_as_float(v));
+                                acc[pol][j] = fresh ? v : acc[pol][j] + v;
                             }
                             if (last) {
                                 const int a = p * NPOL + pol;

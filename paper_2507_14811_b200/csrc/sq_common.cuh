@@ -180,7 +180,7 @@ struct RowsParams {
     long long ldx;
     int q_lo, q_hi;
 };
-constexpr int kSegmentModeRows = 8, kSegmentModeNoRows = 9;     // segquant_set_tuning
+constexpr int kSegmentModeRows = 8;     // segquant_set_tuning: the GEMM of few rows wherever it fits
 
 // A GEMM launch worked out ahead of time: kernel instantiation, tensor maps, parameters, grid.
 struct GemmLaunch {
