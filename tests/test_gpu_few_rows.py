@@ -1,6 +1,8 @@
 """The GEMM of few rows (output channels on the MMA's rows, tokens on its columns, K ranges split over clusters, activations
 quantized inside): bit for bit the results of the tile form, which the parity tests hold to the oracle.  Both add the same
 terms in the same order: int8 sums are exact however a K range is split, e4m3 ones are never split."""
+import threading
+
 import pytest
 import torch
 from cuda.bindings import driver
@@ -75,10 +77,19 @@ def test_every_shape_equals_the_tile_form(case, code, dual):
     try:
         B.segquant_set_tuning(segment_mode=TILE_FORM)
         ref, ref_acc = gemm(layer, codes, y_dtype, dump=True)
-        for rows, tokens, split in ((0, 0, 0), (128, 8, 1), (32, 16, 2), (64, 256, 4), (96, 32, 8), (128, 128, 1), (32, 8, 8)):
+        splits = (1, 2, 4, 8, 1, 8) if code == "int8" else (1,) * 6          # e4m3: one CTA has the whole K range
+        for (rows, tokens), split in zip(((0, 0), (128, 8), (32, 16), (64, 256), (96, 32), (128, 128), (32, 8)), (0, *splits)):
             B.segquant_set_tuning(rows, tokens, split, ROWS_FORM)        # shapes that do not fit run the tile form
+            kblocks, t = (K + 127) // 128, min(tokens or 8, M)
+            columns = 2 * ((t + 7) // 8 * 8) if dual else (t + 15) // 16 * 16
+            fits = split <= kblocks and columns <= 256
+            held = (kblocks + max(split, 1) - 1) // max(split, 1) * 128 * (columns + t * X.element_size())   # codes and inputs of a CTA
             Y = torch.full((M + 1, N), 7.0, dtype=y_dtype, device=DEV)
+            n = B.segquant_launch_count()
             layer.forward(X, Y[:M])                                      # quantized inside
+            inside = B.segquant_launch_count() == n + 1
+            assert inside if fits and held <= 100 * 1024 else fits or not inside
+            assert gemm_forms(lambda: gemm(layer, codes, y_dtype, dump=True)) == [ROWS_THREADS if fits else TILE_THREADS]
             y, acc = gemm(layer, codes, y_dtype, dump=True)
             layer.check_status()
             shape = (rows, tokens, split)
@@ -104,6 +115,7 @@ def test_per_token_scales(M, K, N, kb, dual):
         for shape in ((0, 0, 0), (32, 8, 1), (128, 32, 8), (64, 16, 2)):
             B.segquant_set_tuning(*shape, ROWS_FORM)
             assert torch.equal(run(), ref), shape
+            assert gemm_forms(run) == [ROWS_THREADS if shape[2] <= (K + 127) // 128 else TILE_THREADS], shape
     finally:
         B.segquant_set_tuning()
     B.check_device_status(ws)
@@ -273,3 +285,37 @@ def test_layers_that_the_tile_form_takes_in_less_time(M, K, N, P, code, dual, fo
         assert torch.equal(gemm(layer, codes, BF16), Y)
     finally:
         B.segquant_set_tuning()
+
+
+def test_streams_and_host_threads():
+    """Layers of few rows, split over clusters and not, from two host threads with streams, buffers and workspaces of their
+    own: kernels of both share SMs, tensor memory and what the library keeps; every thread has its own layer shapes."""
+    sizes = [(8, 4096, 264, "int8"), (250, 256, 768, "int8"), (40, 1152, 392, "e4m3"), (1, 8192, 136, "int8")]
+    work = [[make(M + t, K, N, [0, K // 64 * 32, K], [0, N], True, code, BF16) for M, K, N, code in sizes] for t in range(2)]
+    want = [[layer.forward(X).clone() for layer, X in w] for w in work]
+    torch.cuda.synchronize()
+    failed = []
+
+    def call(t):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                plans = [(layer.plan(X, y), y) for layer, X in work[t] for y in [torch.empty_like(layer.forward(X))]]
+                for _ in range(60):
+                    got = [layer.forward(X) for layer, X in work[t]]
+                    for plan, _ in plans:
+                        plan.run()
+                torch.cuda.current_stream().synchronize()
+                if not all(torch.equal(g, w) and torch.equal(y, w) for g, (_, y), w in zip(got, plans, want[t])):
+                    failed.append(t)
+        except Exception as e:
+            failed.append(repr(e))
+
+    threads = [threading.Thread(target=call, args=(t,)) for t in range(2)]
+    for thread in threads:
+        thread.start()
+    for thread in threads:
+        thread.join()
+    assert not failed
+    for w in work:
+        for layer, _ in w:
+            layer.check_status()
