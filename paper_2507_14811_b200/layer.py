@@ -54,7 +54,8 @@ class SegQuantLinear:
                                         x_stage=x_stage, y_stage=y_stage, flags=self.flags)
 
     def plan(self, X: torch.Tensor, Y: torch.Tensor) -> "B.LayerPlan":
-        """A prepared call for these device buffers: plan.run() issues the layer's two kernels and nothing else."""
+        """A prepared call for these device buffers: plan.run() issues the layer's two kernels (one for some layers of few
+        rows) and nothing else."""
         return B.LayerPlan(X, self.Wq, self.seg, self.code, self.s_pos, self.s_neg, self.s_w, self.bias, Y,
                            self.scratch_for(X.shape[0]), self.workspace, self.flags)
 
